@@ -22,12 +22,18 @@
 // samples are fl32(C_b -+ t), t = sqrt(fl32(r r - q)) rounded, with outward
 // normals (du / r, dv / r, -+t / r), each operation rounded to nearest.
 //
+// A sphere covers the interval between its two samples, so the ray's result
+// is bounded by the ends of the connected components of its intervals: the
+// spheres' and, for the outer offset, H's solid intervals; for the inner one
+// H's gaps, the result being what lies between the components.  Intervals that
+// touch belong together (the state does not change where one ends and another
+// begins), empty ones do not count, and at an end of a component the sources
+// that change there are exactly the intervals that end (or begin) at its
+// depth, so the first of them in the order above gives the sample.
+//
 // Stages: sphere centres; per image, sphere lists of 8 x 8-pixel tiles
-// (count, scan, fill); per ray (a warp each) a count pass, the scan of the
-// counts into the output offsets, and the write pass.  A ray merges its
-// spheres 64 at a time into the solid accumulated so far; since the first
-// changing source wins at every depth, merging in batches gives the result of
-// merging all at once.
+// (count, scan, fill); per ray (a warp each) the components and the count of
+// its samples; the scan of the counts into the output offsets; the samples.
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -38,9 +44,14 @@
 namespace ldni {
 namespace {
 
-constexpr int kOffWarps = 4;      // rays per block, a warp each
-constexpr int kOffEvents = 512;   // samples one ray can order: H's plus two per sphere
-constexpr int kTile = 8;          // pixels per side of a sphere-list tile
+constexpr int kOffWarps = 8;      // rays (warps) per block: one pixel row of a tile
+constexpr int kStagePer = 2;      // spheres of the tile's list a thread looks at per round
+constexpr int kStage = kOffWarps * 32 * kStagePer;
+constexpr int kBuf = 288;         // intervals of one ray held in shared memory
+constexpr int kMaxComp = 256;     // components a ray may keep when its intervals are merged to make room
+constexpr int kMaxHSamples = 384; // H's samples on one ray
+constexpr int kKept = 8;          // samples whose sources the count pass leaves to the write pass
+constexpr int kTile = kOffWarps;  // pixels per side of a sphere-list tile
 constexpr int kThreads = 256;
 
 struct OffArgs {
@@ -56,6 +67,8 @@ struct OffArgs {
     float h;
     int res;
     float r, r2, eps;
+    float inv_h;
+    float slack[3];  // pixels by which a shadow is widened, per world axis (off_bin)
     int inner;
     // sphere centres and tile lists
     float4 *C;
@@ -65,6 +78,8 @@ struct OffArgs {
     int ntx;        // tiles per side
     // output
     int *cnt[3];    // per-ray output counts
+    int *deep;      // number and list of the rows (image, tile row) with rays of more than kKept samples
+    uint4 *kept[3]; // per ray, the sources of its samples (two uint4), when there are at most kKept
     int *ooff[3];
     float *od[3], *ox[3], *oy[3], *oz[3];
     int *ot[3];
@@ -116,275 +131,450 @@ __global__ void __launch_bounds__(kThreads) off_centres(OffArgs A) {
 }
 
 // Sphere s into the lists of the tiles of image blockIdx.y that its shadow
-// (widened by a pixel) touches: count (kFill = false) or fill.
+// touches: count (kFill = false) or fill.  The lists only have to hold every
+// sphere that can meet a ray of the tile, so the shadow's bounds are taken in
+// FP32 (this GPU runs FP64 at 1/64 of its rate) and widened by `slack` pixels,
+// which covers the rounding of the bounds and of the pixel centres.
+// Neighbouring samples touch the same few tiles, whose counters then take
+// every lane's atomic in turn (70 us a pass for the 42,000 spheres of the
+// 128^2 flower on 768 counters): the lanes of a warp that hold the same tile
+// send one atomic for all (9 us, the bounds in FP32 among it).
 template <bool kFill>
 __global__ void __launch_bounds__(kThreads) off_bin(OffArgs A) {
     const int b = blockIdx.y;
+    const int lane = threadIdx.x & 31;
     const long long s = blockIdx.x * (long long)kThreads + threadIdx.x;
-    if (s >= A.S) return;
-    const float4 c = A.C[s];
+    const float4 c = s < A.S ? A.C[s] : make_float4(INFINITY, INFINITY, INFINITY, 0.0f);
     const int bu = b == 2 ? 0 : b + 1, bv = b == 0 ? 2 : b - 1;
-    const double hh = A.h;
-    const double lo_u = ((double)c4(c, bu) - A.r - A.o[bu]) / hh - 0.5, hi_u = ((double)c4(c, bu) + A.r - A.o[bu]) / hh - 0.5;
-    const double lo_v = ((double)c4(c, bv) - A.r - A.o[bv]) / hh - 0.5, hi_v = ((double)c4(c, bv) + A.r - A.o[bv]) / hh - 0.5;
-    if (!(isfinite(lo_u) && isfinite(hi_u) && isfinite(lo_v) && isfinite(hi_v))) return;  // a sample at infinity
-    const double last = A.res - 1;
-    const double i0 = fmax(floor(lo_u) - 1.0, 0.0), i1 = fmin(ceil(hi_u) + 1.0, last);
-    const double j0 = fmax(floor(lo_v) - 1.0, 0.0), j1 = fmin(ceil(hi_v) + 1.0, last);
-    if (!(i0 <= i1 && j0 <= j1)) return;  // the shadow misses the image (or a coordinate is NaN)
+    const float rp = A.r * A.inv_h, last = (float)(A.res - 1);
+    const float u = (c4(c, bu) - A.o[bu]) * A.inv_h - 0.5f, v = (c4(c, bv) - A.o[bv]) * A.inv_h - 0.5f;
+    const float ru = rp + A.slack[bu], rv = rp + A.slack[bv];
+    const float i0 = fmaxf(floorf(u - ru), 0.0f), i1 = fminf(ceilf(u + ru), last);
+    const float j0 = fmaxf(floorf(v - rv), 0.0f), j1 = fminf(ceilf(v + rv), last);
+    // (false for a sample at infinity and for a shadow that misses the image)
+    const bool live = isfinite(u) && isfinite(v) && isfinite(rp) && i0 <= i1 && j0 <= j1;
     int *tc = pick(A.tcnt, b);
-    const int ti0 = (int)i0 / kTile, ti1 = (int)i1 / kTile, tj0 = (int)j0 / kTile, tj1 = (int)j1 / kTile;
-    for (int tj = tj0; tj <= tj1; ++tj)
-        for (int ti = ti0; ti <= ti1; ++ti) {
-            const int tile = tj * A.ntx + ti;
-            if (!kFill) {
-                atomicAdd(tc + tile, 1);
-            } else {
-                const int slot = pick(A.toff, b)[tile] + atomicAdd(tc + tile, 1);
-                pick(A.tlist, b)[slot] = (int)s;
-            }
+    const int ti0 = live ? (int)i0 / kTile : 0, tj0 = live ? (int)j0 / kTile : 0;
+    const int nti = live ? (int)i1 / kTile - ti0 + 1 : 1, n = live ? nti * ((int)j1 / kTile - tj0 + 1) : 0;
+    const int steps = __reduce_max_sync(0xffffffffu, n);
+    int ti = 0, tj = 0;
+    for (int k = 0; k < steps; ++k) {
+        const int tile = k < n ? (tj0 + tj) * A.ntx + ti0 + ti : -1;
+        if (++ti == nti) {
+            ti = 0;
+            ++tj;
         }
-}
-
-__device__ __forceinline__ unsigned long long ev_key(float d, unsigned low) {
-    unsigned u = __float_as_uint(__fadd_rn(d, 0.0f));
-    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-    return ((unsigned long long)u << 32) | low;
-}
-
-// Low word of an event: kNew marks a sample of a sphere being merged (else a
-// boundary of the solid accumulated so far); kSph marks a sphere's sample
-// (payload 2 s + 0 entering / 1 leaving), else H's sample (payload: its index
-// in the ray).  Ordered by depth, then accumulated boundaries before new
-// samples, H before spheres, spheres by index.
-constexpr unsigned kNew = 0x80000000u, kSph = 0x40000000u, kPay = 0x3fffffffu;
-constexpr unsigned kNone = 0xffffffffu;
-
-__device__ __forceinline__ bool first_wins(unsigned a, unsigned b) {  // a before b in the order H, sphere 0, 1, ...
-    if (!(a & kSph)) return true;
-    if (!(b & kSph)) return false;
-    return ((a & kPay) >> 1) < ((b & kPay) >> 1);
-}
-
-// Merges the sorted events ev[0, n) of the accumulated solid and of new
-// spheres into the accumulated solid's boundaries ev[0, returned): a sweep
-// from below every sample, where the accumulated state flips at each of its
-// boundaries (parity) and each new sphere adds one cover between its two
-// samples.  Where the combined state changes, the boundary takes the source
-// that comes first among those whose own state changes there.  One lane.
-__device__ int sweep_merge(unsigned long long *ev, int n, int inner) {
-    int ain = 0, cover = 0, w = 0;
-    for (int k = 0; k < n;) {
-        const unsigned hi32 = (unsigned)(ev[k] >> 32);
-        int acnt = 0, delta = 0;
-        unsigned atag = kNone, btag = kNone;
-        while (k < n && (unsigned)(ev[k] >> 32) == hi32) {
-            const unsigned low = (unsigned)ev[k];
-            if (!(low & kNew)) {
-                if (acnt++ == 0) atag = low;
-                ++k;
-            } else {
-                delta += (low & 1u) ? -1 : 1;
-                if (btag == kNone) btag = low;
-                ++k;
-            }
-        }
-        const int before = inner ? (ain && cover == 0) : (ain || cover > 0);
-        ain ^= acnt & 1;
-        cover += delta;
-        const int after = inner ? (ain && cover == 0) : (ain || cover > 0);
-        if (before == after) continue;
-        // a new sphere whose two samples share this depth was not kept, so a
-        // new sample here always changes its sphere's state
-        unsigned tag;
-        if ((acnt & 1) && btag != kNone)
-            tag = first_wins(atag, btag) ? atag : btag;
-        else
-            tag = (acnt & 1) ? atag : btag;
-        ev[w++] = ((unsigned long long)hi32 << 32) | (tag & ~kNew);
+        const unsigned same = __match_any_sync(0xffffffffu, tile);
+        const int leader = __ffs(same) - 1;
+        int at = 0;
+        if (lane == leader && tile >= 0) at = atomicAdd(tc + tile, __popc(same));
+        if (!kFill) continue;
+        at = __shfl_sync(0xffffffffu, at, leader);
+        if (tile >= 0)
+            pick(A.tlist, b)[pick(A.toff, b)[tile] + at + __popc(same & ((1u << lane) - 1u))] = (int)s;
     }
-    return w;
 }
 
-// One warp per ray p of image blockIdx.y.  The accumulated solid starts as
-// H's samples; the spheres that meet the ray and can change the result are
-// gathered, kBatch samples at a time, and merged into it.
-constexpr int kBatch = 128;  // new sphere samples per merge
+// ---- components of a ray's intervals -----------------------------------------------
+//
+// An interval is (first key, last key, first source, last source).  Keys order
+// depths as unsigned words (-0 as +0); kLow and kHigh stand below and above
+// every depth.  A source is 0 for H and s + 1 for sphere s, so the smaller one
+// comes first in the order of the step-by-step Booleans.
+constexpr unsigned kLow = 0u, kHigh = 0xffffffffu;
+constexpr unsigned kSph = 0x40000000u;  // sample tag: sphere (2 s + leaving), else H's sample index on the ray
+constexpr unsigned kAll = 0xffffffffu;
 
-template <bool kWrite>
-__global__ void __launch_bounds__(kOffWarps * 32) off_rays(OffArgs A, ldni_info_t *info) {
-    __shared__ unsigned long long sev[kOffWarps][kOffEvents];
-    __shared__ unsigned long long snew[kOffWarps][kBatch];
-    const int b = blockIdx.y;
+__device__ __forceinline__ unsigned depth_key(float d) {
+    const unsigned u = __float_as_uint(__fadd_rn(d, 0.0f));
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+__device__ __forceinline__ float key_depth(unsigned k) {
+    return __uint_as_float((k & 0x80000000u) ? (k ^ 0x80000000u) : ~k);
+}
+
+struct Comp {
+    unsigned lo, hi, lo_src, hi_src;
+};
+
+// A lane's share of the buffer's (first key, last key) pairs: in registers
+// when kRegs of them per lane are enough, else read from the buffer each time.
+constexpr int kRegs = 8;
+
+template <bool kInRegs>
+struct Ends {
+    const uint4 *buf;
+    int nb, lane;
+    uint2 v[kInRegs ? kRegs : 1];
+    __device__ __forceinline__ Ends(const uint4 *buf_, int nb_, int lane_) : buf(buf_), nb(nb_), lane(lane_) {
+        if constexpr (kInRegs) {
+#pragma unroll
+            for (int k = 0; k < kRegs; ++k)
+                v[k] = 32 * k + lane < nb ? *reinterpret_cast<const uint2 *>(buf + 32 * k + lane)
+                                          : make_uint2(kHigh, kHigh);
+        }
+    }
+    template <class F>
+    __device__ __forceinline__ void each(F &&f) const {
+        if constexpr (kInRegs) {
+#pragma unroll
+            for (int k = 0; k < kRegs; ++k) f(v[k].x, v[k].y);
+        } else {
+            for (int i = lane; i < nb; i += 32) {
+                const uint2 u = *reinterpret_cast<const uint2 *>(buf + i);
+                f(u.x, u.y);
+            }
+        }
+    }
+};
+
+// The first component that begins at or above `from`; false when there is
+// none.  Whole warp; every loop moves a key strictly upwards through the
+// buffer's keys, so it ends.
+template <class E>
+__device__ __forceinline__ bool next_comp(const E &ends, unsigned from, Comp &c) {
+    unsigned lo = kHigh;
+    ends.each([&](unsigned e, unsigned) { lo = e >= from ? min(lo, e) : lo; });
+    lo = __reduce_min_sync(kAll, lo);
+    if (lo == kHigh) return false;  // (an interval's first key is below its last)
+    unsigned hi = lo;
+    for (;;) {
+        unsigned m = hi;
+        ends.each([&](unsigned e, unsigned x) { m = e <= hi ? max(m, x) : m; });
+        m = __reduce_max_sync(kAll, m);
+        if (m == hi) break;
+        hi = m;
+    }
+    unsigned lo_src = kAll, hi_src = kAll;
+    int at = ends.lane;
+    ends.each([&](unsigned e, unsigned x) {
+        if (e == lo) lo_src = min(lo_src, ends.buf[at].z);
+        if (x == hi) hi_src = min(hi_src, ends.buf[at].w);
+        at += 32;
+    });
+    c = Comp{lo, hi, __reduce_min_sync(kAll, lo_src), __reduce_min_sync(kAll, hi_src)};
+    return true;
+}
+
+// Turns the entries [first, nb) (centre along the ray, squared half length of
+// the chord, sphere) into intervals; one whose two samples share a depth
+// changes no state and is marked dead.  Whole warp.
+__device__ __forceinline__ void make_intervals(uint4 *buf, int first, int nb, int lane) {
+    __syncwarp();
+    for (int i = first + lane; i < nb; i += 32) {
+        const uint4 v = buf[i];
+        const float c = __uint_as_float(v.x), t = __fsqrt_rn(__uint_as_float(v.y));
+        const float e = __fsub_rn(c, t), x = __fadd_rn(c, t);
+        buf[i] = e < x ? make_uint4(depth_key(e), depth_key(x), v.z + 1u, v.z + 1u) : make_uint4(kHigh, kHigh, kAll, kAll);
+    }
+    __syncwarp();
+}
+
+// Replaces the buffer's intervals by their components (whole warp); returns
+// how many there are.  The first interval of a component becomes it, the
+// others are marked dead (no key is above kHigh) and squeezed out.
+__device__ __noinline__ int merge_buf(uint4 *buf, int nb, int lane) {
+    unsigned from = 0;
+    Comp c;
+    while (next_comp(Ends<false>(buf, nb, lane), from, c)) {
+        __syncwarp();
+        int head = INT_MAX;
+        for (int i = lane; i < nb; i += 32)
+            if (buf[i].x == c.lo) head = min(head, i);
+        head = __reduce_min_sync(kAll, head);
+        for (int i = lane; i < nb; i += 32) {
+            const unsigned e = buf[i].x;
+            if (e < c.lo || e > c.hi || e == kHigh) continue;
+            buf[i] = i == head ? make_uint4(c.lo, c.hi, c.lo_src, c.hi_src) : make_uint4(kHigh, kHigh, kAll, kAll);
+        }
+        __syncwarp();
+        if (c.hi == kHigh) break;
+        from = c.hi + 1u;
+    }
+    int n = 0;
+    for (int i0 = 0; i0 < nb; i0 += 32) {
+        const uint4 v = i0 + lane < nb ? buf[i0 + lane] : make_uint4(kHigh, kHigh, kAll, kAll);
+        const unsigned live = __ballot_sync(kAll, v.x != kHigh);  // (also: every lane has read its slot)
+        if (v.x != kHigh) buf[n + __popc(live & ((1u << lane) - 1u))] = v;
+        n += __popc(live);
+        __syncwarp();
+    }
+    return n;
+}
+
+// One sample of the result at `slot`: H's sample or the sphere's own.
+__device__ __forceinline__ void put_result(const OffArgs &A, int b, long long hb, float pu, float pv, unsigned tag,
+                                           long long slot, ldni_info_t *info) {
+    if (slot >= pick(A.ocap, b)) {
+        set_status(info, LDNI_ST_CAPACITY);
+        return;
+    }
+    float d, nx, ny, nz;
+    int id;
+    if (!(tag & kSph)) {
+        const long long k = hb + tag;
+        d = pick(A.hd, b)[k];
+        nx = pick(A.hx, b)[k];
+        ny = pick(A.hy, b)[k];
+        nz = pick(A.hz, b)[k];
+        id = pick(A.ht, b)[k];
+    } else {
+        const unsigned sid = (tag & ~kSph) >> 1;
+        float e, x, t, du, dv;
+        sphere_hit(A.C[sid], b, pu, pv, A.r2, e, x, t, du, dv);
+        const bool leaving = tag & 1u;
+        const float n = __fdiv_rn(t, A.r);
+        float nb = leaving ? n : -n, nu = __fdiv_rn(du, A.r), nv = __fdiv_rn(dv, A.r);
+        if (A.inner) {  // the spheres are subtracted: inverted normals (Section 4.1)
+            nb = -nb;
+            nu = -nu;
+            nv = -nv;
+        }
+        d = leaving ? x : e;
+        nx = b == 0 ? nb : (b == 1 ? nv : nu);
+        ny = b == 1 ? nb : (b == 2 ? nv : nu);
+        nz = b == 2 ? nb : (b == 0 ? nv : nu);
+        id = (int)(0x80000000u | sid);
+    }
+    pick(A.od, b)[slot] = d;
+    pick(A.ox, b)[slot] = nx;
+    pick(A.oy, b)[slot] = ny;
+    pick(A.oz, b)[slot] = nz;
+    pick(A.ot, b)[slot] = id;
+}
+
+// One pixel row of a tile of image blockIdx.y, a warp per ray.  The block
+// walks the tile's list, kStage spheres at a time (the next ones' loads in
+// flight), and stages those that reach its row (about a third), with their
+// distance from the row, which all its rays share.  Every warp then tests
+// them against its ray; the ones that meet it become intervals, whose
+// components are found by warp-wide minima and maxima, about a dozen sweeps
+// over the five intervals a lane holds (150 a ray on the 128^2 flower by 2.5
+// pixels).  Bound by issue: 50 M warp instructions at 58 % of the issue slots, 88 us.  Ordering
+// the intervals' ends with a bitonic network and sweeping them with one lane,
+// done in both passes, took 589 + 566 us (now 88, and 11 + 19 for the writes);
+// half a tile per block, every list entry tested by every ray, 171 us.
+// kDeep false: every ray's count, and the sources of its samples when there
+// are at most kKept; kDeep true: writes the samples of the rays that have more.
+template <bool kDeep>
+__device__ __forceinline__ void ray_row(const OffArgs &A, int bx, int b, ldni_info_t *info) {
+    __shared__ float4 sc[kStage];  // (centre along the ray, u, squared distance from the row, sphere)
+    __shared__ uint4 sbuf[kOffWarps][kBuf];
+    __shared__ int s_n, s_deep;
+    if (threadIdx.x == 0) s_deep = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const long long N = (long long)A.res * A.res;
-    const long long p = (long long)blockIdx.x * kOffWarps + w;
-    if (p >= N) return;  // the same for the whole warp
-    unsigned long long *ev = sev[w], *nev = snew[w];
-    const int *hoff = pick(A.hoff, b);
-    const float *HD = pick(A.hd, b);
-    long long hb = hoff[p], he = hoff[p + 1];
-    if (hb < 0 || he < hb || he > pick(A.n, b)) {  // offsets that do not fit the stated sample count
-        if (lane == 0) set_status(info, LDNI_ST_CAPACITY);
-        hb = he = 0;
-    }
-    const int nh = (int)(he - hb);
-    if ((nh & 1) && lane == 0 && !kWrite) {
-        atomicAdd(&info->odd_rays, 1u);
-        set_status(info, LDNI_ST_ODD);
-    }
-    bool over = nh > kOffEvents - kBatch;
-    int na = over ? 0 : nh, nn = 0;
-    for (int k = lane; k < na; k += 32) ev[k] = ev_key(HD[hb + k], (unsigned)k);
+    const int tile = bx / kTile;
+    const int i = tile % A.ntx * kTile + w, j = tile / A.ntx * kTile + bx % kTile;
+    if (j >= A.res) return;  // the same for the whole block
+    const bool mine = i < A.res;
+    const long long p = (long long)j * A.res + i;
+    const bool live = mine && (!kDeep || pick(A.cnt, b)[p] > kKept);
     const int bu = b == 2 ? 0 : b + 1, bv = b == 0 ? 2 : b - 1;
-    const int i = (int)(p % A.res), j = (int)(p / A.res);
-    const float pu = pix(i, A.o[bu], A.h), pv = pix(j, A.o[bv], A.h);
-    const int tile = (j / kTile) * A.ntx + i / kTile;
-    const int l0 = pick(A.toff, b)[tile], l1 = pick(A.toff, b)[tile + 1];
-    const int *lst = pick(A.tlist, b);
-    // merge the gathered samples into the accumulated solid (whole warp)
-    bool merged = false, met = false;
-    auto merge = [&]() {
-        merged = true;
-        __syncwarp();
-        if (na + nn > kOffEvents) {
-            over = true;
-            return;
+    const int l0 = pick(A.toff, b)[tile], nl = pick(A.toff, b)[tile + 1] - l0;
+    const int *lst = pick(A.tlist, b) + l0;
+    const float *HD = pick(A.hd, b);
+    uint4 *buf = sbuf[w];
+    long long hb = 0;
+    int nh = 0, nb = 0;
+    if (live) {
+        const int *hoff = pick(A.hoff, b);
+        long long he = hoff[p + 1];
+        hb = hoff[p];
+        if (hb < 0 || he < hb || he > pick(A.n, b)) {  // offsets that do not fit the stated sample count
+            if (lane == 0) set_status(info, LDNI_ST_CAPACITY);
+            hb = he = 0;
         }
-        for (int k = lane; k < nn; k += 32) ev[na + k] = nev[k];
-        int np2 = 1;
-        while (np2 < na + nn) np2 <<= 1;
-        for (int k = na + nn + lane; k < np2; k += 32) ev[k] = ~0ull;
-        __syncwarp();
-        for (int size = 2; size <= np2; size <<= 1)
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                for (int t = lane; t < (np2 >> 1); t += 32) {
-                    const int lo = 2 * stride * (t / stride) + (t % stride), hi = lo + stride;
-                    const unsigned long long u = ev[lo], v = ev[hi];
-                    if ((u > v) == ((lo & size) == 0)) {
-                        ev[lo] = v;
-                        ev[hi] = u;
-                    }
-                }
-                __syncwarp();
-            }
-        int m = 0;
-        if (lane == 0) m = sweep_merge(ev, na + nn, A.inner);
-        na = __shfl_sync(0xffffffffu, m, 0);
-        nn = 0;
-        __syncwarp();
-    };
-    for (int base = l0; base < l1 && !over; base += 32) {
-        const int idx = base + lane;
-        bool keep = false;
-        float e = 0.0f, x = 0.0f;
-        int s = 0;
-        if (idx < l1) {
-            s = lst[idx];
-            float t, du, dv;
-            keep = sphere_hit(A.C[s], b, pu, pv, A.r2, e, x, t, du, dv);
-            met = met || keep;
-            keep = keep && e < x;  // e == x: no change of state
-            // a sphere's samples strictly inside one of H's solid intervals
-            // (inner offset: one of its gaps) change nothing
-            for (int k = 0; keep && k <= nh; k += 2) {
-                const float lo = A.inner ? (k == 0 ? -INFINITY : HD[hb + k - 1]) : (k < nh ? HD[hb + k] : INFINITY);
-                const float hi = A.inner ? (k < nh ? HD[hb + k] : INFINITY) : (k + 1 < nh ? HD[hb + k + 1] : -INFINITY);
-                if (e > lo && x < hi) keep = false;
-            }
+        nh = (int)(he - hb);
+        if ((nh & 1) && lane == 0 && !kDeep) {
+            atomicAdd(&info->odd_rays, 1u);
+            set_status(info, LDNI_ST_ODD);
         }
-        const unsigned m = __ballot_sync(0xffffffffu, keep);
-        if (nn + 2 * __popc(m) > kBatch) merge();
-        if (over) break;
-        const int at = nn + 2 * __popc(m & ((1u << lane) - 1u));
-        if (keep) {
-            nev[at] = ev_key(e, kNew | kSph | ((unsigned)s << 1));
-            nev[at + 1] = ev_key(x, kNew | kSph | ((unsigned)s << 1) | 1u);
-        }
-        nn += 2 * __popc(m);
     }
-    // A sphere met the ray: the step-by-step Booleans then also merge H's
-    // touching intervals and drop its empty ones, so the ray is swept even
-    // when every sphere was set aside.
-    met = __any_sync(0xffffffffu, met);
-    if (!over && (nn > 0 || (met && !merged))) merge();
-    if (over) {  // more than one warp orders: leave the ray empty and say so
+    bool over = nh > kMaxHSamples, met = false;
+    // H's solid intervals (outer) or its gaps (inner); an odd ray's last one has no end
+    const int nhi = over || !live ? 0 : (A.inner ? nh / 2 + 1 : (nh + 1) / 2);
+    for (int k0 = 0; k0 < nhi; k0 += 32) {
+        const int k = 2 * (k0 + lane) - (A.inner ? 1 : 0);
+        const bool in = k0 + lane < nhi;
+        const unsigned lo = !in ? kHigh : (k < 0 ? kLow : depth_key(HD[hb + k]));
+        const unsigned hi = !in ? kHigh : (k + 1 < nh ? depth_key(HD[hb + k + 1]) : kHigh);
+        const bool some = lo < hi;
+        const unsigned m = __ballot_sync(kAll, some);
+        if (some) buf[nb + __popc(m & ((1u << lane) - 1u))] = make_uint4(lo, hi, 0u, 0u);
+        nb += __popc(m);
+    }
+    int nfinal = nb;  // entries before this one are intervals, the others spheres that meet the ray
+    const float pu = pix(i, A.o[bu], A.h), pv = pix(j, A.o[bv], A.h);
+    int sid[kStagePer];
+    float4 cc[kStagePer];
+    auto fetch = [&](int base) {
+#pragma unroll
+        for (int k = 0; k < kStagePer; ++k) {
+            const int idx = base + k * kOffWarps * 32 + (int)threadIdx.x;
+            sid[k] = idx < nl ? lst[idx] : -1;
+        }
+#pragma unroll
+        for (int k = 0; k < kStagePer; ++k) cc[k] = sid[k] >= 0 ? A.C[sid[k]] : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    fetch(0);
+    for (int base = 0; base < nl; base += kStage) {
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();  // the previous round's spheres are read
+#pragma unroll
+        for (int k = 0; k < kStagePer; ++k) {
+            const float dv = __fsub_rn(pv, c4(cc[k], bv)), dv2 = __fmul_rn(dv, dv);
+            const bool in = sid[k] >= 0 && dv2 < A.r2;  // (du du + dv dv, rounded, is no smaller than dv dv)
+            const unsigned m = __ballot_sync(kAll, in);
+            int at = 0;
+            if (lane == 0 && m) at = atomicAdd(&s_n, __popc(m));
+            at = __shfl_sync(kAll, at, 0) + __popc(m & ((1u << lane) - 1u));
+            if (in) sc[at] = make_float4(c4(cc[k], b), c4(cc[k], bu), dv2, __int_as_float(sid[k]));
+        }
+        fetch(base + kStage);
+        __syncthreads();
+        const int ns = s_n;
+        for (int k0 = 0; k0 < ns && live && !over; k0 += 32) {
+            float4 c;
+            float q = INFINITY;
+            if (k0 + lane < ns) {  // as sphere_hit
+                c = sc[k0 + lane];
+                const float du = __fsub_rn(pu, c.y);
+                q = __fadd_rn(__fmul_rn(du, du), c.z);
+            }
+            const bool hit = q < A.r2;
+            const unsigned m = __ballot_sync(kAll, hit);
+            if (nb + __popc(m) > kBuf) {
+                make_intervals(buf, nfinal, nb, lane);
+                nb = nfinal = merge_buf(buf, nb, lane);
+                over = nb > kMaxComp;
+                if (over) break;
+            }
+            if (hit)
+                buf[nb + __popc(m & ((1u << lane) - 1u))] =
+                    make_uint4(__float_as_uint(c.x), __float_as_uint(__fsub_rn(A.r2, q)), __float_as_uint(c.w), 0u);
+            nb += __popc(m);
+            met = met || m != 0u;
+        }
+    }
+    if (!live) return;
+    if (over) {  // more than one warp holds: leave the ray empty and say so
         if (lane == 0) {
             set_status(info, LDNI_ST_EVENTS);
-            if (!kWrite) pick(A.cnt, b)[p] = 0;
+            if (!kDeep) pick(A.cnt, b)[p] = 0;
         }
         return;
     }
-    __syncwarp();
-    if (lane != 0) return;
-    // the accumulated boundaries alternate entering / leaving; small-interval
-    // removal, then the samples
-    const long long oslot = kWrite ? (long long)pick(A.ooff, b)[p] : 0;
-    const long long cap = pick(A.ocap, b);
+    make_intervals(buf, nfinal, nb, lane);
+    // index on the ray of H's first sample with key k
+    auto h_index = [&](unsigned k) {
+        unsigned at = kAll;
+        for (int h = lane; h < nh; h += 32)
+            if (at == kAll && depth_key(HD[hb + h]) == k) at = (unsigned)h;
+        return __reduce_min_sync(kAll, at);
+    };
+    const long long oslot = kDeep ? (long long)pick(A.ooff, b)[p] : 0;
+    unsigned tags[kKept] = {};
     int nout = 0;
-    for (int q = 0; q + 1 < na; q += 2) {
-        float dd[2], nb3[2], nu3[2], nv3[2];
-        int id[2];
-        for (int z = 0; z < 2; ++z) {
-            const unsigned low = (unsigned)ev[q + z];
-            if (!(low & kSph)) {
-                const long long k2 = hb + (low & kPay);
-                dd[z] = HD[k2];
-                if (kWrite) {
-                    const float hx = pick(A.hx, b)[k2], hy = pick(A.hy, b)[k2], hz = pick(A.hz, b)[k2];
-                    nb3[z] = b == 0 ? hx : (b == 1 ? hy : hz);
-                    nu3[z] = bu == 0 ? hx : (bu == 1 ? hy : hz);
-                    nv3[z] = bv == 0 ? hx : (bv == 1 ? hy : hz);
-                    id[z] = pick(A.ht, b)[k2];
+    // one interval of the result, thinner than eps removed
+    auto emit = [&](unsigned tag0, unsigned tag1) {
+        if (kDeep) {
+            if (lane < 2) put_result(A, b, hb, pu, pv, lane ? tag1 : tag0, oslot + nout + lane, info);
+        } else {
+#pragma unroll
+            for (int z = 0; z < kKept; z += 2)
+                if (nout == z) {
+                    tags[z] = tag0;
+                    tags[z + 1] = tag1;
                 }
-            } else {
-                const long long sid = (low & kPay) >> 1;
-                float e, x, t, du, dv;
-                sphere_hit(A.C[sid], b, pu, pv, A.r2, e, x, t, du, dv);
-                const bool leaving = low & 1u;
-                dd[z] = leaving ? x : e;
-                if (kWrite) {
-                    const float na3 = __fdiv_rn(t, A.r);
-                    float n0 = leaving ? na3 : -na3, n1 = __fdiv_rn(du, A.r), n2 = __fdiv_rn(dv, A.r);
-                    if (A.inner) {  // the spheres are subtracted: inverted normals (Section 4.1)
-                        n0 = -n0;
-                        n1 = -n1;
-                        n2 = -n2;
-                    }
-                    nb3[z] = n0;
-                    nu3[z] = n1;
-                    nv3[z] = n2;
-                    id[z] = (int)(0x80000000u | (unsigned)sid);
-                }
-            }
-        }
-        if (__fsub_rn(dd[1], dd[0]) < A.eps) continue;  // a solid interval thinner than eps
-        if (kWrite) {
-            for (int z = 0; z < 2; ++z) {
-                const long long slot = oslot + nout + z;
-                if (slot >= cap) {
-                    set_status(info, LDNI_ST_CAPACITY);
-                    continue;
-                }
-                float n3[3];
-                n3[b] = nb3[z];
-                n3[bu] = nu3[z];
-                n3[bv] = nv3[z];
-                pick(A.od, b)[slot] = dd[z];
-                pick(A.ox, b)[slot] = n3[0];
-                pick(A.oy, b)[slot] = n3[1];
-                pick(A.oz, b)[slot] = n3[2];
-                pick(A.ot, b)[slot] = id[z];
-            }
         }
         nout += 2;
+    };
+    if (!met) {  // no sphere meets the ray: H stays as it is
+        for (int k = 0; k + 1 < nh; k += 2) {
+            if (!(__fsub_rn(HD[hb + k + 1], HD[hb + k]) < A.eps)) emit((unsigned)k, (unsigned)k + 1u);
+        }
+    } else {
+        // A sphere met the ray: the step-by-step Booleans then also merge H's touching
+        // intervals and drop its empty ones.
+        auto sweep = [&](const auto &ends) {
+            Comp c, prev{};
+            bool first = true;
+            unsigned from = 0;
+            while (next_comp(ends, from, c)) {
+                unsigned k0, k1, s0, s1;
+                if (A.inner) {  // from the previous component's end to this one's beginning
+                    k0 = prev.hi, s0 = prev.hi_src, k1 = c.lo, s1 = c.lo_src;
+                } else {
+                    k0 = c.lo, s0 = c.lo_src, k1 = c.hi, s1 = c.hi_src;
+                }
+                const bool whole = A.inner ? !first : c.hi != kHigh;
+                if (whole && !(__fsub_rn(key_depth(k1), key_depth(k0)) < A.eps)) {
+                    const unsigned side = A.inner ? 1u : 0u;  // where the result enters, the sphere leaves
+                    emit(s0 ? (kSph | ((s0 - 1u) << 1) | side) : h_index(k0),
+                         s1 ? (kSph | ((s1 - 1u) << 1) | (side ^ 1u)) : h_index(k1));
+                }
+                if (c.hi == kHigh) break;
+                first = false;
+                prev = c;
+                from = c.hi + 1u;
+            }
+        };
+        if (nb <= 32 * kRegs)
+            sweep(Ends<true>(buf, nb, lane));
+        else
+            sweep(Ends<false>(buf, nb, lane));
     }
-    if (!kWrite) pick(A.cnt, b)[p] = nout;
+    if (!kDeep && lane == 0) {
+        pick(A.cnt, b)[p] = nout;
+        if (nout && nout <= kKept) {
+            uint4 *kp = pick(A.kept, b) + 2 * p;
+            kp[0] = make_uint4(tags[0], tags[1], tags[2], tags[3]);
+            if (nout > 4) kp[1] = make_uint4(tags[4], tags[5], tags[6], tags[7]);
+        }
+        if (nout > kKept && atomicExch(&s_deep, 1) == 0) A.deep[1 + atomicAdd(A.deep, 1)] = b * (A.ntx * A.ntx * kTile) + bx;
+    }
+}
+
+__global__ void __launch_bounds__(kOffWarps * 32) off_count(OffArgs A, ldni_info_t *info) {
+    ray_row<false>(A, (int)blockIdx.x, (int)blockIdx.y, info);
+}
+
+// The rows that hold rays of more than kKept samples, from the list the count
+// pass left (a launch over all rows spends 27 us finding none in most).
+__global__ void __launch_bounds__(kOffWarps * 32) off_deep(OffArgs A, ldni_info_t *info) {
+    const int rows = A.ntx * A.ntx * kTile, n = A.deep[0];
+    for (int q = blockIdx.x; q < n; q += gridDim.x) {
+        const int row = A.deep[1 + q];
+        ray_row<true>(A, row % rows, row / rows, info);
+        __syncthreads();  // the shared buffers are free again
+    }
+}
+
+// The samples of the rays that have at most kKept, from the sources that the
+// count pass left: a thread per ray of image blockIdx.y.
+__global__ void __launch_bounds__(kThreads) off_write(OffArgs A, ldni_info_t *info) {
+    const int b = blockIdx.y;
+    const long long p = blockIdx.x * (long long)kThreads + threadIdx.x;
+    if (p >= (long long)A.res * A.res) return;
+    const int n = pick(A.cnt, b)[p];
+    if (n == 0 || n > kKept) return;
+    const uint4 k = pick(A.kept, b)[2 * p], k2 = n > 4 ? pick(A.kept, b)[2 * p + 1] : k;
+    const unsigned tag[kKept] = {k.x, k.y, k.z, k.w, k2.x, k2.y, k2.z, k2.w};
+    const int bu = b == 2 ? 0 : b + 1, bv = b == 0 ? 2 : b - 1;
+    const float pu = pix((int)p % A.res, A.o[bu], A.h), pv = pix((int)p / A.res, A.o[bv], A.h);
+    const long long hb = max(pick(A.hoff, b)[p], 0), slot = pick(A.ooff, b)[p];
+#pragma unroll
+    for (int z = 0; z < kKept; ++z)
+        if (z < n) put_result(A, b, hb, pu, pv, tag[z], slot + z, info);
 }
 
 struct OffWs {
     float4 *C;
     int *tcnt[3], *toff[3], *tlist[3], *cnt[3];
+    uint4 *kept[3];
+    int *deep;
     long long *partials;
     ldni_info_t *tinfo;
     size_t clear_bytes;  // tile counts and tinfo: one memset from tcnt[0]
@@ -411,7 +601,9 @@ bool carve_offset(Carver &c, long long S, int res, double r_pixels, OffWs &w) {
         w.toff[a] = c.take<int>((size_t)ntiles + 1);
         w.tlist[a] = c.take<int>((size_t)(pairs > 0 ? pairs : 1));
         w.cnt[a] = c.take<int>((size_t)N);
+        w.kept[a] = c.take<uint4>(2 * (size_t)N);
     }
+    w.deep = c.take<int>(1 + 3 * (size_t)ntiles * kTile);
     const size_t parts = std::max(csr_scan_partials(N), csr_scan_partials(ntiles));
     w.partials = c.take<long long>(parts * 3);
     return true;
@@ -473,6 +665,7 @@ extern "C" int ldni_offset(const ldni_layers_t *H, const int64_t *n, const ldni_
         A.toff[a] = w.toff[a];
         A.tlist[a] = w.tlist[a];
         A.cnt[a] = w.cnt[a];
+        A.kept[a] = w.kept[a];
         A.ooff[a] = out[a].offsets;
         A.od[a] = out[a].depth;
         A.ox[a] = out[a].nx;
@@ -489,7 +682,11 @@ extern "C" int ldni_offset(const ldni_layers_t *H, const int64_t *n, const ldni_
     A.r2 = r * r;
     A.eps = eps;
     A.inner = inner;
+    A.inv_h = 1.0f / h;
+    for (int a = 0; a < 3; ++a)  // rounding of the bounds, and of the pixel centres o + (t + 1/2) h
+        A.slack[a] = (float)std::min(1.0, 0.06 + std::ldexp(std::fabs((double)A.o[a]) + grid->width, -22) / h);
     A.C = w.C;
+    A.deep = w.deep;
     A.ntx = (res + kTile - 1) / kTile;
     const long long ntiles = (long long)A.ntx * A.ntx;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -509,8 +706,9 @@ extern "C" int ldni_offset(const ldni_layers_t *H, const int64_t *n, const ldni_
     // the counts become the fill cursors
     if (int rc_ = cuda_check(cudaMemsetAsync(w.tcnt[0], 0, w.clear_bytes, s))) return rc_;
     if (S > 0) LDNI_LAUNCH(K_OFFSET, s, off_bin<true><<<dim3(sblocks, 3), kThreads, 0, s>>>(A));
-    const unsigned wblocks = (unsigned)((N + kOffWarps - 1) / kOffWarps);
-    LDNI_LAUNCH(K_OFFSET, s, off_rays<false><<<dim3(wblocks, 3), kOffWarps * 32, 0, s>>>(A, info));
+    const dim3 tblocks((unsigned)(ntiles * kTile), 3);
+    if (int rc_ = cuda_check(cudaMemsetAsync(w.deep, 0, sizeof(int), s))) return rc_;
+    LDNI_LAUNCH(K_OFFSET, s, off_count<<<tblocks, kOffWarps * 32, 0, s>>>(A, info));
     rc = cuda_status();
     if (rc != LDNI_OK) return rc;
     {
@@ -519,6 +717,7 @@ extern "C" int ldni_offset(const ldni_layers_t *H, const int64_t *n, const ldni_
         rc = csr_scan(cnts, offs, 3, N, w.partials, info, 0, s);
         if (rc != LDNI_OK) return rc;
     }
-    LDNI_LAUNCH(K_OFFSET, s, off_rays<true><<<dim3(wblocks, 3), kOffWarps * 32, 0, s>>>(A, info));
+    LDNI_LAUNCH(K_OFFSET, s, off_write<<<dim3(rblocks, 3), kThreads, 0, s>>>(A, info));
+    LDNI_LAUNCH(K_OFFSET, s, off_deep<<<4 * num_sms(), kOffWarps * 32, 0, s>>>(A, info));
     return cuda_status();
 }

@@ -123,3 +123,14 @@ def test_table4_style_flower_sizes(ldni):
             want = oracle.offset(ref, O3, 1.0, res, rpix / res, inner=inner)
             for a in range(3):
                 assert bit_equal(got[a].numpy(), want[a]), (rpix, inner, a)
+
+
+@pytest.mark.parametrize("slabs,res,rpix", [(5, 33, 0.4), (12, 41, 1.3), (30, 25, 0.3), (2, 17, 6.0)])
+def test_rays_of_many_samples(ldni, slabs, res, rpix):
+    """Results of more samples per ray than the count pass keeps, spheres that
+    join some of the slabs, tile lists longer and shorter than a staging
+    round, ragged resolutions; bit for bit like the other cases."""
+    grid, ref, H = _solid(ldni, M.slab_stack(slabs, axis=1, seed=slabs), res)
+    for inner in (False, True):
+        for eps in (0.0, 0.01):
+            _check(ldni, grid, ref, H, rpix / res, inner, eps=eps)
