@@ -10,10 +10,15 @@
 // the samples of its ray through the node lie strictly below c_a (the
 // odd-to-even ranges are inside, Section 2 after Proposition 1).
 //
-// A ray kernel writes one bit volume per image, the bits of a word running
-// along that image's rays, laid out so that the stores are coalesced; a vote
-// kernel then takes 32 x 32 x 32 node cubes, transposes the y and z bits
-// with warp shuffles and writes the majority in the x-fastest output layout.
+// A ray kernel turns each image into bit words along its rays, and a vote
+// kernel takes 32 x 32 x 32 node cubes, turns the y and z words so that their
+// bits run along x too, and writes the majority in the x-fastest output
+// layout.  Nearly every cube lies wholly inside or outside, so the words of 32
+// neighbouring rays are nearly always all ones or all zeros each: such a group
+// is stored as one mask of 32 bits, which is already the turned word of all 32
+// rows, and only a group that a surface crosses is stored word by word and
+// turned bit by bit.  For 1024^3 nodes that leaves 25 MB of summaries where
+// three whole bit volumes took 402 MB written and read again.
 #include "ldni_host.h"
 
 namespace ldni {
@@ -25,9 +30,9 @@ __device__ __forceinline__ float node_c(int t, float o, float h) {
 }
 
 // First node t in [0, res] with c(t) > d (c increases with t): a float
-// estimate, then corrected with the exact node positions.
-__device__ __forceinline__ int first_above(float d, int res, float o, float h) {
-    float est = (d - o) / h - 0.5f;
+// estimate (inv_h: about 1 / h), then corrected with the exact node positions.
+__device__ __forceinline__ int first_above(float d, int res, float o, float h, float inv_h) {
+    const float est = (d - o) * inv_h - 0.5f;
     int t = !(est > 0.0f) ? 0 : (est >= (float)res ? res : (int)est);
     while (t > 0 && node_c(t - 1, o, h) > d) --t;
     while (t < res && !(node_c(t, o, h) > d)) ++t;
@@ -46,11 +51,6 @@ __device__ __forceinline__ unsigned step_word(int b, int w) {
     return 0xffffffffu << (b - t0);
 }
 
-__device__ __forceinline__ unsigned live_bits(int w, int res) {
-    const int left = res - 32 * w;
-    return left >= 32 ? 0xffffffffu : ((1u << left) - 1u);
-}
-
 __device__ __forceinline__ void ray_range(const int *__restrict__ off, long long cap, long long p, long long &b,
                                           long long &e, ldni_info_t *info, bool report) {
     b = off[p];
@@ -63,38 +63,6 @@ __device__ __forceinline__ void ray_range(const int *__restrict__ off, long long
         if (report) set_status(info, LDNI_ST_CAPACITY);
         e = cap;
         b = min(b, e);
-    }
-}
-
-// One thread per ray of image a, consecutive threads = consecutive rays of
-// one node row, so that every word store is coalesced: word w of the ray
-// holds its nodes 32 w .. 32 w + 31 and sits at V[w res^2 + q], with
-//   x-image ray p = k res + j:  q = k res + j (nodes i)
-//   y-image ray p = i res + k:  q = k res + i (nodes j)
-//   z-image ray p = j res + i:  q = j res + i (nodes k)
-// The thread walks its ray's boundaries once, in order, while it writes the
-// words.
-__global__ void __launch_bounds__(256) node_rays(const int *__restrict__ off, const float *__restrict__ depth,
-                                                 long long cap, int res, int W, float o, float h, int axis,
-                                                 unsigned *V, ldni_info_t *info) {
-    const long long q = blockIdx.x * 256LL + threadIdx.x;
-    if (q >= (long long)res * res) return;
-    const long long p = axis == 1 ? (q % res) * res + q / res : q;
-    long long b, e;
-    ray_range(off, cap, p, b, e, info, true);
-    const long long plane = (long long)res * res;
-    const int n = (int)(e - b);
-    int m = 0;
-    int bm = n > 0 ? first_above(depth[b], res, o, h) : res;
-    unsigned after = 0;  // all ones once an odd number of boundaries lie before the current word
-    for (int w = 0; w < W; ++w) {
-        unsigned word = after;
-        while (m < n && bm < 32 * w + 32) {  // boundaries that reach into this word
-            word ^= step_word(bm, w);
-            after = ~after;
-            if (++m < n) bm = first_above(depth[b + m], res, o, h);
-        }
-        V[w * plane + q] = word & live_bits(w, res);
     }
 }
 
@@ -114,50 +82,158 @@ __device__ __forceinline__ unsigned warp_transpose32(unsigned x, int lane) {
     return x;
 }
 
-// One block per kVoteCubes cubes of 32 (i) x 32 (j) x 32 (k) nodes along i;
-// warp w and lane l produce the output words of row (k = 32 kb + w,
-// j = 32 jb + l) for i-words ib0 .. ib0 + kVoteCubes - 1 and store them
-// together (one 32-byte sector per lane).  For each cube ib:
-//   x: word ib of x-ray (k, j) as stored;
-//   y: warp w loads word jb of the y-rays (k, i = 32 ib + l) and transposes:
-//      lane l then holds the bits over i of row (k, j = 32 jb + l);
-//   z: warp w loads word kb of the z-rays (j = 32 jb + w, i = 32 ib + l) and
-//      transposes: lane l holds the bits over i of row (k = 32 kb + l,
-//      j = 32 jb + w), which reach their row's warp through shared memory.
-constexpr int kVoteCubes = 8;
+// Bit words of the three images.  A group is 32 neighbouring rays (a lane
+// each) of one node row, nb groups per row:
+//   x-image ray p = k res + j: row k, column j (bits: nodes i)
+//   y-image ray p = i res + k: row k, column i (bits: nodes j)
+//   z-image ray p = j res + i: row j, column i (bits: nodes k)
+// and has W words per ray.  sum[group W + w] = (the rays whose word w is all
+// ones; 0 when every ray's word w is all ones or all zeros, else 1).  In the
+// second case word[(group W + w) 32 + l] holds the words of an output row: of
+// the x-image's ray l, and, the other two turned, of the row l of word w's 32
+// nodes over the group's 32 columns.
+struct NodeImg {
+    const int *off[3];
+    const float *depth[3];
+    long long cap[3];
+    float o[3];
+    uint2 *sum[3];
+    unsigned *word[3];
+};
 
-__global__ void __launch_bounds__(1024, 2) node_vote(const unsigned *__restrict__ Vx, const unsigned *__restrict__ Vy,
-                                                  const unsigned *__restrict__ Vz, int res, int W, unsigned *out) {
-    __shared__ unsigned zt[2][32][33];  // [cube parity][k in cube][j in cube]
-    const int ib0 = blockIdx.x * kVoteCubes, jb = blockIdx.y, kb = blockIdx.z;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const long long plane = (long long)res * res;
-    const int k = kb * 32 + w, j = jb * 32 + lane, jz = jb * 32 + w;
-    unsigned word[kVoteCubes];
-#pragma unroll
-    for (int c = 0; c < kVoteCubes; ++c) {
-        const int ib = ib0 + c;
-        const int i = ib * 32 + lane;
-        const bool live = ib < W && i < res;
-        const unsigned zw = (live && jz < res) ? Vz[kb * plane + (long long)jz * res + i] : 0u;
-        const unsigned yw = (live && k < res) ? Vy[jb * plane + (long long)k * res + i] : 0u;
-        const unsigned x = (ib < W && k < res && j < res) ? Vx[ib * plane + (long long)k * res + j] : 0u;
-        zt[c & 1][lane][w] = warp_transpose32(zw, lane);  // row (k = 32 kb + lane, j = 32 jb + w)
-        const unsigned y = warp_transpose32(yw, lane);     // row (k, j)
-        __syncthreads();  // zt[c & 1] complete; the read of zt[c & 1] two cubes back is done
-        const unsigned z = zt[c & 1][w][lane];
-        word[c] = (x & y) | (z & (x | y));  // at least two of three
+// Bits of nodes at or beyond res are left as they come: their lanes or words
+// are never stored, or meet zeros in the vote.
+// Bound by issue (76 % of the slots, 31 M warp instructions for the union of the
+// noisy sphere and the knot at 1024^2): 38 us for the three images; the three
+// launches that wrote every word took 37 us each.
+constexpr int kRowsPerBlock = 8;  // a warp each (the y-image's offsets of 8 rows share their sectors)
+
+__global__ void __launch_bounds__(32 * kRowsPerBlock) node_rays(NodeImg I, int res, int nb, int W, float h,
+                                                                float inv_h, ldni_info_t *info) {
+    const int a = blockIdx.z;
+    const int lane = threadIdx.x & 31;
+    const int row = blockIdx.y * kRowsPerBlock + (threadIdx.x >> 5), col = blockIdx.x * 32 + lane;
+    if (row >= res) return;  // the same for the whole warp
+    const float o = I.o[a];
+    const float *__restrict__ depth = I.depth[a];
+    long long b = 0, e = 0;
+    if (col < res)
+        ray_range(I.off[a], I.cap[a], a == 1 ? (long long)col * res + row : (long long)row * res + col, b, e, info, true);
+    const int n = (int)(e - b);
+    int m = 0;
+    int bm = n > 0 ? first_above(depth[b], res, o, h, inv_h) : res;
+    unsigned after = 0;  // all ones once an odd number of boundaries lie before the current word
+    const long long group = (long long)row * nb + blockIdx.x;
+    uint2 *sum = I.sum[a] + group * W;
+    unsigned *word = I.word[a] + group * W * 32;
+    for (int w0 = 0; w0 < W; w0 += 32) {  // lane l holds the summary of word w0 + l
+        uint2 mine = make_uint2(0u, 0u);
+        const int w1 = min(w0 + 32, W);
+        int w = w0;
+        while (w < w1) {
+            // words before the next boundary of any ray repeat the rays' states
+            const int next = max(w, __reduce_min_sync(0xffffffffu, m < n ? bm >> 5 : W));
+            const unsigned state = __ballot_sync(0xffffffffu, after != 0u);
+            if (w0 + lane >= w && w0 + lane < next) mine = make_uint2(state, 0u);
+            w = next;
+            if (w >= w1) break;
+            unsigned x = after;
+            while (m < n && bm < 32 * w + 32) {  // boundaries that reach into this word
+                x ^= step_word(bm, w);
+                after = ~after;
+                if (++m < n) bm = first_above(depth[b + m], res, o, h, inv_h);
+            }
+            const unsigned ones = __ballot_sync(0xffffffffu, x == 0xffffffffu);
+            const unsigned mixed = __any_sync(0xffffffffu, x != 0u && x != 0xffffffffu);
+            if (w0 + lane == w) mine = make_uint2(ones, mixed ? 1u : 0u);
+            if (mixed) word[32LL * w + lane] = a == 0 ? x : warp_transpose32(x, lane);
+            ++w;
+        }
+        if (w0 + lane < w1) sum[w0 + lane] = mine;
     }
-    if (k >= res || j >= res) return;
-    unsigned *row = out + ((long long)k * res + j) * W;
-    if ((W & 3) == 0 && ib0 + kVoteCubes <= W && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {  // aligned runs
+}
+
+// Majority words of the rows (k, j), j in 32-block jb, k among kVoteK of
+// 32-block kb, for up to 32 words along i; a warp takes a row k at a time.
+// Lane = (row within a store, word ib): a store covers 32 words of the output,
+// several rows where a row is shorter, so that it is contiguous.  For word ib
+// of row (k, j):
+//   x: bit j of the mask of x-group (k, jb) at word ib, or that ray's word;
+//   y: the mask of y-group (k, ib) at word jb, the same for every j;
+//   z: the mask of z-group (j, ib) at word kb, the same for every k (shared
+//      memory).
+// The cubes that a surface crosses (a fifth of the words of a row of cubes that
+// meets the solid) follow one by one, lane = row j.  Bound by the latency of
+// the summaries and of those cubes' words (40 % issue, the 134 MB of output
+// alone would take 20 us at 1024^3): 61 us; 173 us when every cube's words
+// were read from bit volumes and turned, 76 us with summaries but a lane per
+// row j, eight words each.
+constexpr int kVoteWarps = 8, kVoteRows = 2, kVoteK = kVoteWarps * kVoteRows;
+static_assert(kVoteRows == 2, "a warp's two rows are picked by selects");
+
+__global__ void __launch_bounds__(32 * kVoteWarps) node_vote(NodeImg I, int res, int nb, int W, int log_words,
+                                                             unsigned *out) {
+    __shared__ unsigned zs[32][33];  // [j in block][word]: mask
+    __shared__ unsigned zmix[32];    // [j in block]: the words whose group is mixed
+    const int jb = blockIdx.y, kb = blockIdx.z / (32 / kVoteK), kpart = blockIdx.z % (32 / kVoteK);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int ibl = lane & ((1 << log_words) - 1), ib = blockIdx.x * 32 + ibl, js = lane >> log_words;
+    const bool live = ib < W;
+    uint2 sx[kVoteRows], sy[kVoteRows], sz[32 / kVoteWarps];
 #pragma unroll
-        for (int c = 0; c < kVoteCubes; c += 4)
-            *reinterpret_cast<uint4 *>(row + ib0 + c) = make_uint4(word[c], word[c + 1], word[c + 2], word[c + 3]);
-    } else {
+    for (int r = 0; r < 32 / kVoteWarps; ++r) {
+        const int j = jb * 32 + w + r * kVoteWarps;
+        sz[r] = live && j < res ? I.sum[2][((long long)j * nb + ib) * W + kb] : make_uint2(0u, 0u);
+    }
 #pragma unroll
-        for (int c = 0; c < kVoteCubes; ++c)
-            if (ib0 + c < W) row[ib0 + c] = word[c];
+    for (int r = 0; r < kVoteRows; ++r) {
+        const int k = kb * 32 + kpart * kVoteK + w + r * kVoteWarps;
+        const bool in = live && k < res;
+        sx[r] = in ? I.sum[0][((long long)k * nb + jb) * W + ib] : make_uint2(0u, 0u);
+        sy[r] = in ? I.sum[1][((long long)k * nb + ib) * W + jb] : make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int r = 0; r < 32 / kVoteWarps; ++r) {
+        const int jj = w + r * kVoteWarps;
+        if (js == 0) zs[jj][ibl] = sz[r].x;
+        const unsigned m = __ballot_sync(0xffffffffu, js == 0 && sz[r].y != 0u);
+        if (lane == 0) zmix[jj] = m;
+    }
+    __syncthreads();
+    unsigned zall = 0;  // words of cubes with a mixed z-group
+#pragma unroll
+    for (int jj = 0; jj < 32; ++jj) zall |= zmix[jj];
+    const int per = 32 >> log_words;  // rows j per store
+    const int jn = min(32, res - jb * 32);
+#pragma unroll 1
+    for (int r = 0; r < kVoteRows; ++r) {
+        const int kk = kpart * kVoteK + w + r * kVoteWarps, k = kb * 32 + kk;
+        if (k >= res) break;  // the same for the whole warp
+        const unsigned xm = r == 0 ? sx[0].x : sx[1].x, y = r == 0 ? sy[0].x : sy[1].x;
+        const bool xmix = (r == 0 ? sx[0].y : sx[1].y) != 0u, ymix = (r == 0 ? sy[0].y : sy[1].y) != 0u;
+        const bool plain = live && !xmix && !ymix && !((zall >> ibl) & 1u);  // masks only
+        unsigned *o = out + ((long long)k * res + jb * 32) * W + blockIdx.x * 32;
+        {
+            unsigned *oj = o + (long long)js * W + ibl;
+            const long long step = (long long)per * W;
+#pragma unroll 8
+            for (int j = js; j < jn; j += per, oj += step) {
+                const unsigned x = 0u - ((xm >> j) & 1u), z = zs[j][ibl];
+                if (plain) *oj = (x & y) | (z & (x | y));  // at least two of three
+            }
+        }
+        // the cubes that a surface crosses: lane = row j
+        for (unsigned todo = __ballot_sync(0xffffffffu, live && !plain && js == 0); todo; todo &= todo - 1u) {
+            const int c = __ffs(todo) - 1, ic = blockIdx.x * 32 + c;
+            const unsigned xc = __shfl_sync(0xffffffffu, xm, c), yc = __shfl_sync(0xffffffffu, y, c);
+            const bool xw = __shfl_sync(0xffffffffu, xmix, c), yw = __shfl_sync(0xffffffffu, ymix, c);
+            const unsigned zm = (zmix[lane] >> c) & 1u;
+            if (lane >= jn) continue;
+            const unsigned x = xw ? I.word[0][(((long long)k * nb + jb) * W + ic) * 32 + lane] : 0u - ((xc >> lane) & 1u);
+            const unsigned yy = yw ? I.word[1][(((long long)k * nb + ic) * W + jb) * 32 + lane] : yc;
+            const unsigned z = zm ? I.word[2][(((long long)(jb * 32 + lane) * nb + ic) * W + kb) * 32 + kk] : zs[lane][c];
+            o[(long long)lane * W + c] = (x & yy) | (z & (x | yy));
+        }
     }
 }
 
@@ -172,8 +248,8 @@ using namespace ldni;
 
 extern "C" int ldni_classify_nodes_workspace_size(int32_t res, size_t *bytes) {
     if (!bytes || res < 1 || res > 4096) return LDNI_EINVAL;
-    const size_t W = ((size_t)res + 31) / 32;
-    *bytes = align_up(3 * sizeof(unsigned) * (size_t)res * res * W + 2 * kAlign);
+    const size_t W = ((size_t)res + 31) / 32, groups = (size_t)res * W;  // as many groups in a row as words in a ray
+    *bytes = align_up(3 * (align_up(sizeof(uint2) * groups * W) + align_up(sizeof(unsigned) * groups * W * 32)));
     return LDNI_OK;
 }
 
@@ -187,21 +263,27 @@ extern "C" int ldni_classify_nodes(const ldni_layers_t *L, const ldni_grid_t *gr
     int rc = ldni_classify_nodes_workspace_size(res, &need);
     if (rc != LDNI_OK) return rc;
     if (ws_bytes < need) return LDNI_EWORKSPACE;
-    const int W = (res + 31) / 32;
-    const size_t vol = (size_t)res * res * W;
+    const int W = (res + 31) / 32, nb = W;
+    const size_t groups = (size_t)res * nb;
     Carver c(ws, ws_bytes);
-    unsigned *V[3];
-    for (int a = 0; a < 3; ++a) V[a] = c.take<unsigned>(vol);
+    NodeImg I{};
+    for (int a = 0; a < 3; ++a) {
+        I.off[a] = L[a].offsets;
+        I.depth[a] = L[a].depth;
+        I.cap[a] = L[a].capacity;
+        I.o[a] = grid->origin[a];
+        I.sum[a] = c.take<uint2>(groups * W);
+        I.word[a] = c.take<unsigned>(groups * W * 32);
+    }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const float hh = (float)grid->width / (float)res;  // FP32 division, as the node positions are defined
-    const long long nrays = (long long)res * res;
-    for (int a = 0; a < 3; ++a)
-        LDNI_LAUNCH(K_NODES, s,
-                    node_rays<<<(unsigned)((nrays + 255) / 256), 256, 0, s>>>(
-                        L[a].offsets, L[a].depth, L[a].capacity, res, W, grid->origin[a], hh, a, V[a], info));
-    const int nb = (res + 31) / 32;
     LDNI_LAUNCH(K_NODES, s,
-                node_vote<<<dim3((W + kVoteCubes - 1) / kVoteCubes, nb, nb), 1024, 0, s>>>(V[0], V[1], V[2], res, W,
-                                                                                         inside));
+                node_rays<<<dim3(nb, (res + kRowsPerBlock - 1) / kRowsPerBlock, 3), 32 * kRowsPerBlock, 0, s>>>(
+                    I, res, nb, W, hh, 1.0f / hh, info));
+    int log_words = 0;  // lanes per row: the words of a row, at most 32
+    while (log_words < 5 && (1 << log_words) < W) ++log_words;
+    LDNI_LAUNCH(K_NODES, s,
+                node_vote<<<dim3((W + 31) / 32, nb, nb * (32 / kVoteK)), 32 * kVoteWarps, 0, s>>>(I, res, nb, W,
+                                                                                                  log_words, inside));
     return cuda_status();
 }

@@ -55,3 +55,17 @@ def test_union_of_two_solids(ldni):
     ref = nodes.classify([x.numpy() for x in U], O3, 1.0, res)
     assert np.array_equal(nu, ref)
     assert (nu | ~(na | nb)).mean() > 0.99 and (~nu | (na | nb)).mean() > 0.99
+
+
+@pytest.mark.parametrize("res", [1, 31, 33, 64, 96, 129, 260])
+def test_row_lengths(ldni, res):
+    """One word per row up to nine (rows that share a store, whole rows, ragged
+    last words and blocks), from solids that leave most cubes uniform and
+    from thin slabs that leave few."""
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    for mesh in (M.icosphere(6, r=0.37, noise=0.02, seed=3), M.slab_stack(9, axis=2, seed=res)):
+        L = ldni.sample(*mesh, grid, "all")
+        words = ldni.classify_nodes(L)
+        assert np.array_equal(ldni.unpack_nodes(words, res), nodes.classify([x.numpy() for x in L], O3, 1.0, res))
+        if res % 32:
+            assert not (words.cpu().numpy().view(np.uint32)[:, :, -1] >> (res % 32)).any()
