@@ -23,13 +23,13 @@
 //    edge yields a vertex;
 //  - x = m + (A^T A)^+ (A^T b - A^T A m), m the points' mean, eigenvalues of
 //    A^T A below 0.01 of the largest dropped (singular values below 0.1),
-//    in FP64 with a cyclic Jacobi eigensolver; a cluster with no Hermite
-//    data sits at the mean of its corners with no points.
+//    in FP64; a cluster with no Hermite data sits at the mean of its corners
+//    with no points.
 //
 // Stages: active-cell marks (edges with samples, from the samples; edges
 // whose end signs differ, word-parallel from the node bits), their
-// compaction, one thread per active cell writing its record to a dense
-// scratch, and the compaction of the cells that yield a vertex.
+// compaction, the active cells' records in a dense scratch, and the compaction
+// of the cells that yield a vertex.
 #include "ldni_host.h"
 
 namespace ldni {
@@ -165,34 +165,23 @@ __global__ void __launch_bounds__(kThreads) list_cells(const unsigned *act, long
 
 struct Edge {
     int a, q0, q1;  // axis, lower and upper corner
-    int iu, iv, t;  // ray node indices, edge index along a
+    int du, dv;     // ray node indices within the cell, along u and v
 };
 
-__device__ __forceinline__ Edge cell_edge(int e, int i, int j, int k) {
-    Edge E;
+// Edge e = 4 a + x + 2 y of a cell.
+__device__ __forceinline__ Edge cell_edge(int e) {
     const int x = e & 1, y = (e >> 1) & 1;
-    if (e < 4) {  // x-edges at (j + x, k + y)
-        E = Edge{0, 0 + 2 * x + 4 * y, 1 + 2 * x + 4 * y, j + x, k + y, i};
-    } else if (e < 8) {  // y-edges at (i + x, k + y): ray (u, v) = (z, x)
-        E = Edge{1, x + 4 * y, x + 2 + 4 * y, k + y, i + x, j};
-    } else {  // z-edges at (i + x, j + y)
-        E = Edge{2, x + 2 * y, x + 2 * y + 4, i + x, j + y, k};
-    }
-    return E;
+    if (e < 4) return Edge{0, 2 * x + 4 * y, 1 + 2 * x + 4 * y, x, y};  // x-edges at (j + x, k + y)
+    if (e < 8) return Edge{1, x + 4 * y, x + 2 + 4 * y, y, x};          // y-edges at (i + x, k + y): (u, v) = (z, x)
+    return Edge{2, x + 2 * y, x + 2 * y + 4, x, y};                     // z-edges at (i + x, j + y)
 }
-
-struct Kept {
-    unsigned char type;  // 0 empty, 1 none-intersect, 2 intersect, 3 complex
-    unsigned char nk;    // kept samples
-    int s0, s1;          // kept sample indices (ascending depth)
-};
 
 struct Sym3 {  // A^T A, A^T b, sum of points, count
     double xx, xy, xz, yy, yz, zz, bx, by, bz, px, py, pz;
     int n;
 };
 
-__device__ __forceinline__ void add_point(Sym3 &Q, double P[3], double N[3]) {
+__device__ __forceinline__ void add_point(Sym3 &Q, const double (&P)[3], const double (&N)[3]) {
     Q.xx += N[0] * N[0];
     Q.xy += N[0] * N[1];
     Q.xz += N[0] * N[2];
@@ -215,7 +204,7 @@ __device__ __forceinline__ void add_point(Sym3 &Q, double P[3], double N[3]) {
 // exact to second order (about 1e-24 relative) and the eigenvectors to about
 // 1e-12, while FP64 rounding keeps the off-diagonal near 1e-16 of the
 // diagonal, so a stricter bound would only spend sweeps.
-__device__ void jacobi3(double S[3][3], double V[3][3]) {
+__device__ __forceinline__ void jacobi3(double S[3][3], double V[3][3]) {
     for (int r = 0; r < 3; ++r)
         for (int c = 0; c < 3; ++c) V[r][c] = r == c ? 1.0 : 0.0;
     for (int sweep = 0; sweep < 32; ++sweep) {
@@ -249,7 +238,8 @@ __device__ void jacobi3(double S[3][3], double V[3][3]) {
     }
 }
 
-__device__ void qef_solve(const Sym3 &Q, double x[3]) {
+// Any system, by the eigensolver: the general path of qef_solve.
+__device__ __noinline__ void qef_solve_jacobi(const Sym3 &Q, double x[3]) {
     const double m[3] = {Q.px / Q.n, Q.py / Q.n, Q.pz / Q.n};
     double S[3][3] = {{Q.xx, Q.xy, Q.xz}, {Q.xy, Q.yy, Q.yz}, {Q.xz, Q.yz, Q.zz}};
     const double AtA[3][3] = {{Q.xx, Q.xy, Q.xz}, {Q.xy, Q.yy, Q.yz}, {Q.xz, Q.yz, Q.zz}};
@@ -267,196 +257,387 @@ __device__ void qef_solve(const Sym3 &Q, double x[3]) {
     for (int a = 0; a < 3; ++a) x[a] = m[a] + V[a][0] * y[0] + V[a][1] * y[1] + V[a][2] * y[2];
 }
 
-__device__ __forceinline__ void hermite(const CImg &I, int a, int s, int iu, int iv, float o[3], float h,
-                                        double P[3], double N[3]) {
-    const int u = a == 2 ? 0 : a + 1, v = a == 0 ? 2 : a - 1;
-    P[a] = (double)pick(I.d, a)[s];
-    P[u] = (double)node_c(iu, o[u], h);
-    P[v] = (double)node_c(iv, o[v], h);
-    double n3[3] = {(double)pick(I.nx, a)[s], (double)pick(I.ny, a)[s], (double)pick(I.nz, a)[s]};
-    N[0] = n3[0];
-    N[1] = n3[1];
-    N[2] = n3[2];
+// Cyclic Jacobi rotations in FP32 on the matrix (xx, xy, xz, yy, yz, zz): its
+// eigenvectors, to FP32 accuracy, in the columns of V.
+__device__ __forceinline__ void jacobi3f(float xx, float xy, float xz, float yy, float yz, float zz, float (&V)[3][3]) {
+    float S[3][3] = {{xx, xy, xz}, {xy, yy, yz}, {xz, yz, zz}};
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) V[r][c] = r == c ? 1.0f : 0.0f;
+#pragma unroll 1
+    for (int sweep = 0; sweep < 8; ++sweep) {
+        const float off = fabsf(S[0][1]) + fabsf(S[0][2]) + fabsf(S[1][2]);
+        if (!(off > 1e-7f * (S[0][0] + S[1][1] + S[2][2]))) break;
+#pragma unroll
+        for (int z = 0; z < 3; ++z) {
+            const int p = z == 2 ? 1 : 0, q = z == 0 ? 1 : 2, o = 3 - p - q;
+            const float apq = S[p][q];
+            if (fabsf(apq) < 1e-30f) continue;
+            const float theta = 0.5f * (S[q][q] - S[p][p]) / apq;
+            const float t = copysignf(1.0f, theta) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.0f)));
+            const float c = rsqrtf(fmaf(t, t, 1.0f)), s = t * c;
+            S[p][p] -= t * apq;
+            S[q][q] += t * apq;
+            S[p][q] = S[q][p] = 0.0f;
+            const float sop = S[o][p], soq = S[o][q];
+            S[o][p] = S[p][o] = c * sop - s * soq;
+            S[o][q] = S[q][o] = s * sop + c * soq;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                const float vp = V[r][p], vq = V[r][q];
+                V[r][p] = c * vp - s * vq;
+                V[r][q] = s * vp + c * vq;
+            }
+        }
+    }
 }
 
-// One thread per active cell (the first *nact of the list).
-__global__ void __launch_bounds__(128) cell_kernel(CImg I, const unsigned *node, int res, int W, float o0, float o1,
-                                                   float o2, float h, const long long *cells, const int *nact,
-                                                   long long max_active, ldni_cell_t *rec) {
-    const long long q = blockIdx.x * 128LL + threadIdx.x;
-    if (q >= min((long long)*nact, max_active)) return;
-    const int n = res - 1;
-    const long long ci = cells[q];
-    const int i = (int)(ci % n), j = (int)((ci / n) % n), k = (int)(ci / ((long long)n * n));
-    float o[3] = {o0, o1, o2};
-    unsigned sgn = 0;  // bit c: corner c inside
-    for (int c = 0; c < 8; ++c) {
-        const int ii = i + (c & 1), jj = j + ((c >> 1) & 1), kk = k + (c >> 2);
-        const unsigned wd = node[((long long)kk * res + jj) * W + (ii >> 5)];
-        sgn |= ((wd >> (ii & 31)) & 1u) << c;
+__device__ __forceinline__ double dot3(const double (&a)[3], const double (&b)[3]) {
+    return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
+}
+
+// x = m + (A^T A)^+ (A^T b - A^T A m).  This GPU runs FP64 at 1/64 of its FP32
+// rate, and the eigensolver took about 1,800 FP64 operations a cell (the whole
+// call spent 400 of 529 us in it for the 255^3 cells of the united sphere and knot).
+// Here FP32 rotations find the eigenvectors, about 100 FP64 operations make
+// them orthonormal and give the matrix in their frame, S = V^T A V, whose
+// off-diagonal entries e are near 1e-7 of the largest eigenvalue:
+//  - the eigenvalues differ from S's diagonal by at most e, so the cut is
+//    decided by the diagonal unless an entry lies within 1e-5 of it;
+//  - turning the kept directions away from the dropped ones by
+//    e / (gap of their eigenvalues) separates them to second order, below
+//    1e-8 with the gaps of 0.004 asked for here;
+//  - what is left is solved on the kept block with its off-diagonal entries.
+// A system that is not so clear (or not finite) goes to the eigensolver.
+__device__ __forceinline__ void qef_solve(const Sym3 &Q, double (&x)[3]) {
+    const double inv_n = 1.0 / (double)Q.n;
+    const double m[3] = {Q.px * inv_n, Q.py * inv_n, Q.pz * inv_n};
+    const double r[3] = {Q.bx - (Q.xx * m[0] + Q.xy * m[1] + Q.xz * m[2]),
+                         Q.by - (Q.xy * m[0] + Q.yy * m[1] + Q.yz * m[2]),
+                         Q.bz - (Q.xz * m[0] + Q.yz * m[1] + Q.zz * m[2])};
+    float F[3][3];
+    jacobi3f((float)Q.xx, (float)Q.xy, (float)Q.xz, (float)Q.yy, (float)Q.yz, (float)Q.zz, F);
+    double v[3][3];  // v[c]: direction c
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) v[c][a] = (double)F[a][c];
+    double f = 1.5 - 0.5 * dot3(v[0], v[0]);  // one Newton step of 1 / |v|
+#pragma unroll
+    for (int a = 0; a < 3; ++a) v[0][a] *= f;
+    f = dot3(v[0], v[1]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) v[1][a] -= f * v[0][a];
+    f = 1.5 - 0.5 * dot3(v[1], v[1]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) v[1][a] *= f;
+    v[2][0] = v[0][1] * v[1][2] - v[0][2] * v[1][1];
+    v[2][1] = v[0][2] * v[1][0] - v[0][0] * v[1][2];
+    v[2][2] = v[0][0] * v[1][1] - v[0][1] * v[1][0];
+    double S[3][3], g[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double w[3] = {Q.xx * v[c][0] + Q.xy * v[c][1] + Q.xz * v[c][2],
+                             Q.xy * v[c][0] + Q.yy * v[c][1] + Q.yz * v[c][2],
+                             Q.xz * v[c][0] + Q.yz * v[c][1] + Q.zz * v[c][2]};
+#pragma unroll
+        for (int d = c; d < 3; ++d) S[c][d] = S[d][c] = dot3(v[d], w);
+        g[c] = dot3(v[c], r);
     }
-    Kept K[12];
-    for (int e = 0; e < 12; ++e) {
-        const Edge E = cell_edge(e, i, j, k);
+    // everything below that decides or corrects needs FP32 only; S and g keep their FP64 values
+    const float l[3] = {(float)S[0][0], (float)S[1][1], (float)S[2][2]};
+    const float top = fmaxf(l[0], fmaxf(l[1], l[2])), cut = 0.01f * top;
+    bool clear = top > 0.0f && top < 1e30f, keep[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        clear = clear && fabsf(l[c] - cut) > 1e-5f * top;
+        keep[c] = l[c] >= cut;
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            if (d != c) clear = clear && fabsf((float)S[c][d]) <= 1e-5f * top;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            if (d != c && keep[c] && !keep[d]) clear = clear && l[c] - l[d] > 4e-3f * top;
+    if (!clear) {
+        qef_solve_jacobi(Q, x);
+        return;
+    }
+    double u[3][3], h[3], inv[3], y[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {  // kept directions turned away from the dropped ones
+        h[c] = g[c];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) u[c][a] = v[c][a];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            if (d == c) continue;
+            if (keep[c] && !keep[d]) {
+                const double th = (double)((float)S[c][d] / (l[c] - l[d]));
+                h[c] += th * g[d];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) u[c][a] += th * v[d][a];
+            }
+        }
+        const double i0 = (double)(keep[c] ? 1.0f / l[c] : 0.0f);
+        inv[c] = i0 * (2.0 - S[c][c] * i0);  // 1 / S to FP64 accuracy, 0 for a dropped direction
+        y[c] = h[c] * inv[c];
+    }
+    double z[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        double t = h[c];
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            if (d != c && keep[d]) t -= S[c][d] * y[d];
+        z[c] = t * inv[c];
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) x[a] = m[a] + u[0][a] * z[0] + u[1][a] * z[1] + u[2][a] * z[2];
+}
+
+constexpr int kCells = 128;        // cells per block
+constexpr int kCellThreads = 128;  // threads per block
+
+// The records of kCells active cells (of the first *nact of the list), and
+// which of them yield a vertex.
+//  1. a thread per cell finds the corner signs;
+//  2. the kept samples of every (cell, edge) from its ray, the first with its
+//     depth and normal;
+//  3. a thread per cell: clusters as sets of corner bits, then one cluster at a
+//     time, its points' sums in registers, and its vertex;
+//  4. the records leave through shared memory in whole lines.
+// Bound by FP64 in step 3 (1.5 M FP64 warp instructions, 74 us of that pipe):
+// 124 us for the 255^3 cells of the united sphere and knot, 149 with twice the
+// threads searching, 420 with the eigensolver for every cell.
+__global__ void __launch_bounds__(kCellThreads) cell_kernel(CImg I, const unsigned *node, int res, int W, float o0,
+                                                            float o1, float o2, float h, const long long *cells,
+                                                            const int *nact, long long max_active, ldni_cell_t *rec,
+                                                            int *flag) {
+    __shared__ float4 pt[12][kCells];   // the edge's first kept sample: depth, normal
+    __shared__ int second[12][kCells];  // its second kept sample, kOne: there is none, kNo: no sample at all
+    __shared__ short ijk[3][kCells];
+    __shared__ unsigned char corner[kCells];
+    constexpr int kOne = -1, kNo = -2;
+    const long long q0 = (long long)blockIdx.x * kCells;
+    const long long total = min((long long)*nact, max_active);
+    const int m = (int)max(0ll, min((long long)kCells, total - q0));  // cells of this block
+    const int tid = threadIdx.x;
+    if (tid < kCells && tid >= m && q0 + tid < max_active) flag[q0 + tid] = 0;
+    if (m == 0) return;
+    const int n = res - 1;
+    long long ci = 0;
+    if (tid < m) {
+        ci = cells[q0 + tid];
+        const int row = (int)(ci / n);
+        const int i = (int)(ci - (long long)row * n), j = row % n, k = row / n;
+        ijk[0][tid] = (short)i;
+        ijk[1][tid] = (short)j;
+        ijk[2][tid] = (short)k;
+        unsigned sgn = 0;  // bit c: corner c inside
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const unsigned *nw = node + ((long long)(k + (r >> 1)) * res + j + (r & 1)) * W + (i >> 5);
+            const unsigned b0 = nw[0] >> (i & 31);
+            const unsigned b1 = (i & 31) == 31 ? nw[1] : b0 >> 1;
+            sgn |= ((b0 & 1u) | ((b1 & 1u) << 1)) << (2 * r);
+        }
+        corner[tid] = (unsigned char)sgn;
+    }
+    __syncthreads();
+    for (int task = tid; task < 12 * kCells; task += kCellThreads) {
+        const int e = task / kCells, c = task % kCells;
+        if (c >= m) continue;
+        const Edge E = cell_edge(e);
+        const int u = E.a == 2 ? 0 : E.a + 1, v = E.a == 0 ? 2 : E.a - 1;
+        const long long p = (long long)(ijk[v][c] + E.dv) * res + ijk[u][c] + E.du;
+        const int t = ijk[E.a][c];
         const int *off = pick(I.off, E.a);
         const float *D = pick(I.d, E.a);
-        const long long p = (long long)E.iv * res + E.iu;
-        const long long b0 = off[p], e0 = min((long long)off[p + 1], pick(I.cap, E.a));
-        const float lo = node_c(E.t, o[E.a], h), hi = node_c(E.t + 1, o[E.a], h);
+        const int b0 = off[p], e0 = (int)min((long long)off[p + 1], pick(I.cap, E.a));
+        const float oa = E.a == 0 ? o0 : (E.a == 1 ? o1 : o2);
+        const float lo = node_c(t, oa, h), hi = node_c(t + 1, oa, h);
+        const unsigned sgn = corner[c];
         const bool in0 = (sgn >> E.q0) & 1u, in1 = (sgn >> E.q1) & 1u;
-        const double mid = ((double)lo + (double)hi) / 2.0;
-        const float want = in0 ? 1.0f : -1.0f;
-        int cnt = 0, first = -1, last = -1, best = -1, bestc = -1;
-        double bd = 0.0, bdc = 0.0;
-        const float *NA = E.a == 0 ? pick(I.nx, 0) : (E.a == 1 ? pick(I.ny, 1) : pick(I.nz, 2));
-        for (long long s = b0; s < e0; ++s) {
-            const float d = D[s];
-            if (d < lo) continue;
-            if (!(d < hi)) break;  // ascending depths
-            ++cnt;
-            if (first < 0) first = (int)s;
-            last = (int)s;
-            const double dist = fabs((double)d - mid);
-            if (best < 0 || dist < bd) {
-                best = (int)s;
-                bd = dist;
-            }
-            if (NA[s] * want > 0.0f && (bestc < 0 || dist < bdc)) {
-                bestc = (int)s;
-                bdc = dist;
+        int first = -1, last = -1, s = b0;
+        while (s < e0 && D[s] < lo) ++s;  // ascending depths
+        for (; s < e0 && D[s] < hi; ++s) {
+            if (first < 0) first = s;
+            last = s;
+        }
+        int keep = first, more = first < 0 ? kNo : kOne;
+        if (first >= 0 && last > first) {
+            if (in0 != in1) {  // Rule 2
+                const float *NA = E.a == 0 ? I.nx[0] : (E.a == 1 ? I.ny[1] : I.nz[2]);
+                const float want = in0 ? 1.0f : -1.0f;
+                const double mid = ((double)lo + (double)hi) / 2.0;
+                bool fits = false;
+                double bd = 0.0;
+                for (int x = first; x <= last; ++x) {
+                    const bool f = NA[x] * want > 0.0f;
+                    const double dist = fabs((double)D[x] - mid);
+                    if (x == first || (f && !fits) || (f == fits && dist < bd)) {
+                        keep = x;
+                        bd = dist;
+                        fits = f;
+                    }
+                }
+            } else {  // Rule 1
+                more = last;
             }
         }
-        Kept &k2 = K[e];
-        if (in0 != in1) {
-            k2.type = cnt ? 2 : 1;
-            k2.nk = cnt ? 1 : 0;
-            k2.s0 = bestc >= 0 ? bestc : best;
-            k2.s1 = -1;
-        } else {
-            k2.type = cnt ? 3 : 0;
-            k2.nk = cnt >= 2 ? 2 : cnt;
-            k2.s0 = first;
-            k2.s1 = cnt >= 2 ? last : -1;
-        }
+        if (first >= 0)
+            pt[e][c] = make_float4(D[keep], pick(I.nx, E.a)[keep], pick(I.ny, E.a)[keep], pick(I.nz, E.a)[keep]);
+        second[e][c] = more;
     }
-    // flood the outside corners through empty edges
-    unsigned char lab[8];
-    for (int c = 0; c < 8; ++c) lab[c] = 0xff;
-    int ncl = 0;
-    for (int c = 0; c < 8; ++c) {
-        if (((sgn >> c) & 1u) || lab[c] != 0xff) continue;
-        unsigned comp = 1u << c, grow = comp;
-        while (grow) {  // breadth-first over empty edges between outside corners
-            unsigned next = 0;
-            for (int e = 0; e < 12; ++e) {
-                if (K[e].type != 0) continue;
-                const Edge E = cell_edge(e, 0, 0, 0);
-                const unsigned m0 = 1u << E.q0, m1 = 1u << E.q1;
-                if ((sgn & (m0 | m1)) != 0) continue;
-                if ((grow & m0) && !(comp & m1)) next |= m1;
-                if ((grow & m1) && !(comp & m0)) next |= m0;
-            }
-            comp |= next;
-            grow = next;
-        }
-        for (int d = 0; d < 8; ++d)
-            if ((comp >> d) & 1u) lab[d] = (unsigned char)ncl;
-        ++ncl;
-    }
+    __syncthreads();
     ldni_cell_t R;
     R.cell = ci;
     R.nvert = 0;
-    R.labels = 0;
+    R.labels = 0xffffffffu;
     R.npts = 0;
     R.pad_ = 0;
-    for (int c = 0; c < 8; ++c) R.labels |= (unsigned)(lab[c] == 0xff ? 0xf : lab[c]) << (4 * c);
-    for (int v = 0; v < 12; ++v) R.v[v] = 0.0f;
-    if (ncl == 0) {
-        rec[q] = R;
-        return;
-    }
-    // Hermite data and the surface clusters
-    bool surf[4] = {false, false, false, false};
-    Sym3 Q[4];
-    for (int g = 0; g < 4; ++g) Q[g] = Sym3{0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int e = 0; e < 12; ++e) {
-        const Edge E = cell_edge(e, i, j, k);
-        const Kept &k2 = K[e];
-        const bool in0 = (sgn >> E.q0) & 1u;
-        double P[3], N[3];
-        if (k2.type == 2) {
-            const int g = lab[in0 ? E.q1 : E.q0];
-            surf[g] = true;
-            hermite(I, E.a, k2.s0, E.iu, E.iv, o, h, P, N);
-            add_point(Q[g], P, N);
-        } else if (k2.type == 1) {
-            surf[lab[in0 ? E.q1 : E.q0]] = true;
-        } else if (k2.type == 3 && !in0) {
-            const int g0 = lab[E.q0], g1 = lab[E.q1];
-            surf[g0] = surf[g1] = true;
-            if (k2.nk == 2) {
-                hermite(I, E.a, k2.s0, E.iu, E.iv, o, h, P, N);
-                add_point(Q[g0], P, N);
-                hermite(I, E.a, k2.s1, E.iu, E.iv, o, h, P, N);
-                add_point(Q[g1], P, N);
-            } else {
-                const float lo = node_c(E.t, o[E.a], h), hi = node_c(E.t + 1, o[E.a], h);
-                const double mid = ((double)lo + (double)hi) / 2.0;
-                hermite(I, E.a, k2.s0, E.iu, E.iv, o, h, P, N);
-                add_point(Q[P[E.a] < mid ? g0 : g1], P, N);
+#pragma unroll
+    for (int x = 0; x < 12; ++x) R.v[x] = 0.0f;
+    if (tid < m) {
+        const int i = ijk[0][tid], j = ijk[1][tid], k = ijk[2][tid];
+        const unsigned sgn = corner[tid], out = ~sgn & 0xffu;
+        // per axis, bit c: the edge from corner c up along it is empty and both its ends are outside
+        unsigned open[3] = {0, 0, 0}, held = 0;  // held: edges with samples
+#pragma unroll
+        for (int e = 0; e < 12; ++e) {
+            const Edge E = cell_edge(e);
+            if (second[e][tid] != kNo)
+                held |= 1u << e;
+            else
+                open[E.a] |= (out >> E.q0) & (out >> E.q1) & 1u ? 1u << E.q0 : 0u;
+        }
+        // flood the outside corners through empty edges, clusters by lowest corner
+        int ncl = 0;
+        for (unsigned rest = out; rest; ++ncl) {
+            unsigned c = rest & (0u - rest), was;
+            do {
+                was = c;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) c |= ((c & open[a]) << (1 << a)) | ((c >> (1 << a)) & open[a]);
+            } while (c != was);
+            rest &= ~c;
+            unsigned x = (c | (c << 12)) & 0x000f000fu;  // bit c to bit 4 c
+            x = (x | (x << 6)) & 0x03030303u;
+            x = (x | (x << 3)) & 0x11111111u;
+            R.labels ^= x * (0xfu ^ (unsigned)ncl);
+        }
+        // edges that make a surface: ends of different sign, or samples between outside corners
+        unsigned cross = 0, outer = 0;
+#pragma unroll
+        for (int e = 0; e < 12; ++e) {
+            const Edge E = cell_edge(e);
+            const unsigned b0 = (sgn >> E.q0) & 1u, b1 = (sgn >> E.q1) & 1u;
+            cross |= (b0 ^ b1) << e;
+            outer |= (1u ^ (b0 | b1)) << e;
+        }
+        if (ncl > 0 && (cross | (held & outer))) {
+            R.nvert = min(ncl, 4);  // a record has room for four
+            const auto label = [&](int q) { return (int)((R.labels >> (4 * q)) & 0xfu); };
+            for (int g = 0; g < R.nvert; ++g) {
+                Sym3 Q{0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+                for (unsigned todo = held & (cross | outer); todo; todo &= todo - 1u) {
+                    const int e = __ffs(todo) - 1;
+                    const Edge E = cell_edge(e);
+                    const int s1 = second[e][tid];
+                    const int l0 = label(E.q0), l1 = label(E.q1);
+                    bool first = false, last = false;  // this cluster's samples of the edge
+                    float4 f = pt[e][tid];
+                    if ((cross >> e) & 1u) {
+                        first = ((sgn >> E.q0) & 1u ? l1 : l0) == g;
+                    } else if (s1 >= 0) {
+                        first = l0 == g;
+                        last = l1 == g;
+                    } else {  // the nearer corner's
+                        const int t = ijk[E.a][tid];
+                        const float oa = E.a == 0 ? o0 : (E.a == 1 ? o1 : o2);
+                        const double mid = ((double)node_c(t, oa, h) + (double)node_c(t + 1, oa, h)) / 2.0;
+                        first = ((double)f.x < mid ? l0 : l1) == g;
+                    }
+                    if (!first && !last) continue;
+                    const int iu = (E.a == 0 ? j : (E.a == 1 ? k : i)) + E.du, iv = (E.a == 0 ? k : (E.a == 1 ? i : j)) + E.dv;
+                    const float ou = E.a == 0 ? o1 : (E.a == 1 ? o2 : o0), ov = E.a == 0 ? o2 : (E.a == 1 ? o0 : o1);
+                    const float cu = node_c(iu, ou, h), cv = node_c(iv, ov, h);
+                    for (int z = 0; z < 2; ++z) {
+                        if (!(z ? last : first)) continue;
+                        if (z) f = make_float4(pick(I.d, E.a)[s1], pick(I.nx, E.a)[s1], pick(I.ny, E.a)[s1], pick(I.nz, E.a)[s1]);
+                        const double P[3] = {(double)(E.a == 0 ? f.x : (E.a == 1 ? cv : cu)),
+                                             (double)(E.a == 1 ? f.x : (E.a == 2 ? cv : cu)),
+                                             (double)(E.a == 2 ? f.x : (E.a == 0 ? cv : cu))};
+                        const double N[3] = {(double)f.y, (double)f.z, (double)f.w};
+                        add_point(Q, P, N);
+                    }
+                }
+                double x[3];
+                if (Q.n > 0) {
+                    qef_solve(Q, x);
+                } else {  // no Hermite data: the mean of the cluster's corners
+                    int cs = 0;
+                    x[0] = x[1] = x[2] = 0.0;
+                    for (int c = 0; c < 8; ++c) {
+                        if (label(c) != g) continue;
+                        x[0] += (double)node_c(i + (c & 1), o0, h);
+                        x[1] += (double)node_c(j + ((c >> 1) & 1), o1, h);
+                        x[2] += (double)node_c(k + (c >> 2), o2, h);
+                        ++cs;
+                    }
+                    for (int a = 0; a < 3; ++a) x[a] /= cs;
+                }
+#pragma unroll
+                for (int v = 0; v < 4; ++v)
+                    if (v == g) {
+                        R.v[3 * v] = (float)x[0];
+                        R.v[3 * v + 1] = (float)x[1];
+                        R.v[3 * v + 2] = (float)x[2];
+                    }
+                R.npts |= (unsigned)min(Q.n, 255) << (8 * g);
             }
         }
+        flag[q0 + tid] = R.nvert > 0 ? 1 : 0;
     }
-    bool any = false;
-    for (int g = 0; g < ncl; ++g) any = any || surf[g];
-    if (!any) {
-        rec[q] = R;
-        return;
-    }
-    R.nvert = ncl;
-    for (int g = 0; g < ncl; ++g) {
-        double x[3];
-        if (Q[g].n > 0) {
-            qef_solve(Q[g], x);
-        } else {  // no Hermite data: the mean of the cluster's corners
-            double s3[3] = {0.0, 0.0, 0.0};
-            int m = 0;
-            for (int c = 0; c < 8; ++c) {
-                if (lab[c] != g) continue;
-                s3[0] += (double)node_c(i + (c & 1), o[0], h);
-                s3[1] += (double)node_c(j + ((c >> 1) & 1), o[1], h);
-                s3[2] += (double)node_c(k + (c >> 2), o[2], h);
-                ++m;
-            }
-            x[0] = s3[0] / m;
-            x[1] = s3[1] / m;
-            x[2] = s3[2] / m;
-        }
-        R.v[3 * g] = (float)x[0];
-        R.v[3 * g + 1] = (float)x[1];
-        R.v[3 * g + 2] = (float)x[2];
-        R.npts |= (unsigned)min(Q[g].n, 255) << (8 * g);
-    }
-    rec[q] = R;
+    __syncthreads();  // the points are read
+    constexpr int kWords = (int)(sizeof(ldni_cell_t) / 4);
+    static_assert(sizeof(pt) >= kCells * sizeof(ldni_cell_t), "the records fit where the points were");
+    ldni_cell_t *out = reinterpret_cast<ldni_cell_t *>(&pt[0][0]);
+    if (tid < m) out[tid] = R;
+    __syncthreads();
+    const int *from = reinterpret_cast<const int *>(out);
+    int *to = reinterpret_cast<int *>(rec + q0);
+    for (int x = tid; x < m * kWords; x += kCellThreads) to[x] = from[x];
 }
 
-__global__ void __launch_bounds__(kThreads) has_vertex(const ldni_cell_t *rec, const int *nact, long long n,
-                                                       int *flag) {
-    const long long q = blockIdx.x * (long long)kThreads + threadIdx.x;
-    if (q < n) flag[q] = (q < *nact && rec[q].nvert > 0) ? 1 : 0;
-}
-
+// The cells with a vertex, in order: a warp copies 32 records, word by word.
 __global__ void __launch_bounds__(kThreads) compact_cells(const ldni_cell_t *rec, const int *nact, long long n,
-                                                          const int *at, ldni_cell_t *out, long long cap,
-                                                          ldni_info_t *info) {
-    const long long q = blockIdx.x * (long long)kThreads + threadIdx.x;
-    if (q >= n || q >= *nact || rec[q].nvert == 0) return;
-    const long long slot = at[q];
-    if (slot >= cap) {
-        set_status(info, LDNI_ST_CAPACITY);
-        return;
+                                                          const int *flag, const int *at, ldni_cell_t *out,
+                                                          long long cap, ldni_info_t *info) {
+    const int lane = threadIdx.x & 31;
+    const long long q0 = blockIdx.x * (long long)kThreads + (threadIdx.x & ~31), total = min((long long)*nact, n);
+    if (q0 >= total) return;  // the same for the whole warp
+    int slot = -1;
+    if (q0 + lane < total && flag[q0 + lane]) {
+        slot = at[q0 + lane];
+        if (slot >= cap) {
+            set_status(info, LDNI_ST_CAPACITY);
+            slot = -1;
+        }
     }
-    out[slot] = rec[q];
+    constexpr int kWords = (int)(sizeof(ldni_cell_t) / 4);
+    const int *from = reinterpret_cast<const int *>(rec + q0);
+    int *to = reinterpret_cast<int *>(out);
+    const int words = (int)min(32ll, total - q0) * kWords;
+#pragma unroll 6
+    for (int x = lane; x < 32 * kWords; x += 32) {
+        const int c = x / kWords, s = __shfl_sync(0xffffffffu, slot, c);
+        if (x < words && s >= 0) to[(long long)s * kWords + (x - c * kWords)] = from[x];
+    }
 }
 
 struct ContourWs {
@@ -551,10 +732,8 @@ extern "C" int ldni_contour_cells(const ldni_layers_t *L, const ldni_grid_t *gri
                 list_cells<<<(unsigned)((nw + kThreads - 1) / kThreads), kThreads, 0, s>>>(
                     w.act, nw, w.woff, n, Wc, w.cells, max_active, info));
     LDNI_LAUNCH(K_CONTOUR, s,
-                cell_kernel<<<(unsigned)((max_active + 127) / 128), 128, 0, s>>>(I, inside, res, W, o[0], o[1], o[2],
-                                                                                   h, w.cells, nact, max_active,
-                                                                                   w.rec));
-    LDNI_LAUNCH(K_CONTOUR, s, has_vertex<<<ablocks, kThreads, 0, s>>>(w.rec, nact, max_active, w.flag));
+                cell_kernel<<<(unsigned)((max_active + kCells - 1) / kCells), kCellThreads, 0, s>>>(
+                    I, inside, res, W, o[0], o[1], o[2], h, w.cells, nact, max_active, w.rec, w.flag));
     rc = cuda_status();
     if (rc != LDNI_OK) return rc;
     {
@@ -564,6 +743,7 @@ extern "C" int ldni_contour_cells(const ldni_layers_t *L, const ldni_grid_t *gri
         if (rc != LDNI_OK) return rc;
     }
     LDNI_LAUNCH(K_CONTOUR, s,
-                compact_cells<<<ablocks, kThreads, 0, s>>>(w.rec, nact, max_active, w.at, cells, capacity, info));
+                compact_cells<<<ablocks, kThreads, 0, s>>>(w.rec, nact, max_active, w.flag, w.at, cells, capacity,
+                                                           info));
     return cuda_status();
 }

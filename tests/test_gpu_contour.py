@@ -108,3 +108,27 @@ def test_inside_from_classify_nodes(ldni):
     a = ldni.contour_cells(H, inside=_t(_bits(ins).view(np.int32)))
     b = ldni.contour_cells(H)
     assert a.tobytes() == b.tobytes()
+
+
+@pytest.mark.parametrize("res", [2, 9, 33])
+@pytest.mark.parametrize("spread", [0.0, 0.08, 0.12, 0.3, 2.0])
+def test_normals_around_the_cut(ldni, res, spread):
+    """Normals scattered about one direction, so that the smaller eigenvalues
+    lie at 0, about the 0.01 cut, above it, or anywhere: vertices of one, two
+    and three kept directions against the oracle (same bound as above)."""
+    ref = [oracle.as_f32(oracle.sample(*M.icosphere(4, r=0.36), O3, 1.0, res, a, "scan")) for a in range(3)]
+    rng = np.random.default_rng(res)
+    for L in ref:
+        n = np.array([0.6, -0.48, 0.64]) + spread * rng.standard_normal((len(L["depth"]), 3))
+        L["nrm"] = (n / np.linalg.norm(n, axis=1, keepdims=True)).astype(np.float32)
+    ins = nodes.classify(ref, O3, 1.0, res)
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    got = ldni.contour_cells([_upload(ldni, grid, a, L) for a, L in enumerate(ref)], inside=_t(_bits(ins).view(np.int32)))
+    want = C.contour(ref, ins, O3, 1.0, res)
+    assert got["cell"].tolist() == sorted(want)
+    for rec, key in zip(got, sorted(want)):
+        w = want[key]
+        nv = min(4, len(w["vertices"]))  # a record has room for four (at res 2 every corner is cut off)
+        assert rec["nvert"] == nv
+        if not any(abs(r - C.QEF_TRUNC) < 1e-6 for rs in w["ratios"] for r in rs):
+            assert np.abs(rec["v"][:nv] - np.asarray(w["vertices"])[:nv]).max() <= 2e-6, key
