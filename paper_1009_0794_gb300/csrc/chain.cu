@@ -6,11 +6,13 @@
 // exact because every operand shares the grid).
 //
 // Every step treats each ray on its own, so the whole chain is a fold along
-// each ray: a thread carries its ray's accumulated samples from step to step
+// each ray: a thread carries its ray's accumulated result from step to step
 // and never waits for another ray or another step.  Two passes over the
 // rays (count, then write, with the CSR scan between them) replace the n - 1
 // Booleans of the step-by-step evaluation, whose intermediate images would
-// each be written to and read back from memory.
+// each be written to and read back from memory.  Without small-interval
+// removal the fold is a union of intervals (unite_pass); with it, or where that
+// does not fit, it merges sample by sample (fold_pass).
 //
 // The result equals the step-by-step chain bit for bit: each step is the
 // same merge (merge.cuh) with the accumulated solid as the first operand, so
@@ -36,116 +38,403 @@ struct Entry {
     int idx;   // source sample in that part
 };
 
-// The fold of ray p of image img: the accumulated samples in acc (returns
-// their number), or -1 when a step needed more than kChainMaxLayers.
+// Sample range of ray p in part P.
+__device__ __forceinline__ void part_range(const ldni_layers_t &P, long long p, int &b, int &e) {
+    b = (int)min((long long)P.offsets[p], (long long)P.capacity);
+    e = (int)min((long long)P.offsets[p + 1], (long long)P.capacity);
+}
+
+// Parts k0 .. k0 + 63 that have samples on ray p, as bits.  Most parts have
+// none on most rays, and one part's offsets say nothing about where the next
+// part's are, so the offsets of kAhead parts are loaded together: loaded part
+// by part between the merges, 64 round trips to memory made up the fold.  odd
+// counts the parts with an odd number of samples (Definition 4).
+constexpr int kAhead = 8;
+__device__ __forceinline__ unsigned long long parts_present(const ldni_layers_t *__restrict__ parts, int count, int k0,
+                                                            long long p, int &odd) {
+    unsigned long long mask = 0;
+    const int n = min(count - k0, 64);
+    for (int q0 = 0; q0 < n; q0 += kAhead) {
+        int b[kAhead], e[kAhead];
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) {
+            const int *off = parts[k0 + min(q0 + q, n - 1)].offsets;
+            b[q] = __ldg(off + p);
+            e[q] = __ldg(off + p + 1);
+        }
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) {
+            if (q0 + q >= n) continue;
+            odd += (e[q] - b[q]) & 1;
+            if (e[q] != b[q]) mask |= 1ull << (q0 + q);
+        }
+    }
+    return mask;
+}
+
+// The fold of ray p: the accumulated samples in acc[cur] (returns their
+// number), or -1 when a step needed more than kChainMaxLayers.  have(k0): the
+// parts k0 .. k0 + 63 that may have samples on the ray.
+template <class Have>
 __device__ __forceinline__ int fold_ray(const ldni_layers_t *__restrict__ parts, int count, long long p, float eps,
-                                        Entry (&acc)[2][kChainMaxLayers], int &cur) {
+                                        Entry (&acc)[2][kChainMaxLayers], int &cur, Have have) {
     cur = 0;
     int na = 0;
-    {
-        const ldni_layers_t &P = parts[0];
-        const long long b = min((long long)P.offsets[p], (long long)P.capacity);
-        const long long e = min((long long)P.offsets[p + 1], (long long)P.capacity);
-        if (e - b > kChainMaxLayers) return -1;
-        for (long long x = b; x < e; ++x) acc[0][na++] = Entry{P.depth[x], 0, (int)x};
-    }
-    for (int k = 1; k < count; ++k) {
-        const ldni_layers_t &P = parts[k];
-        const long long b = min((long long)P.offsets[p], (long long)P.capacity);
-        const long long e = min((long long)P.offsets[p + 1], (long long)P.capacity);
-        // uniting a merged result (strictly ascending, no empty interval) with nothing, and no thin
-        // pieces to remove, changes nothing
-        if (e == b && eps == 0.0f && k > 1) continue;
-        const Entry *A = acc[cur];
-        Entry *O = acc[cur ^ 1];
-        bool over = false;
-        struct AccDepth {
-            const Entry *a;
-            __device__ __forceinline__ float operator[](int i) const { return a[i].d; }
-        };
-        const float *dB = P.depth + b;
-        const int m = merge_core<int>(AccDepth{A}, 0, na, dB, 0, (int)(e - b), LDNI_OP_UNION, eps,
-                                      [&](bool pb, int pi, bool cb, int ci, int mm) {
-                                          if (mm + 2 > kChainMaxLayers) {
-                                              over = true;
-                                              return;
-                                          }
-                                          O[mm] = pb ? Entry{dB[pi], k, (int)(b + pi)} : A[pi];
-                                          O[mm + 1] = cb ? Entry{dB[ci], k, (int)(b + ci)} : A[ci];
-                                      });
-        if (over) return -1;
-        na = m;
-        cur ^= 1;
+    for (int k0 = 0; k0 < count; k0 += 64) {
+        unsigned long long todo = have(k0);
+        if (k0 == 0) {
+            if (todo & 1ull) {
+                int b, e;
+                part_range(parts[0], p, b, e);
+                if (e - b > kChainMaxLayers) return -1;
+                for (int x = b; x < e; ++x) acc[0][na++] = Entry{parts[0].depth[x], 0, x};
+                // the first union merges touching intervals and removes thin ones even where it adds nothing
+                if (count > 1) todo |= 2ull;
+            }
+            todo &= ~1ull;
+        }
+        // Uniting a merged result (strictly ascending, no interval that is empty or thinner than eps) with
+        // nothing changes nothing: parts without samples are passed over.
+        for (; todo; todo &= todo - 1ull) {
+            const int k = k0 + __ffsll((long long)todo) - 1;
+            const ldni_layers_t &P = parts[k];
+            int b, e;
+            part_range(P, p, b, e);
+            if (e <= b && k > 1) continue;
+            const Entry *A = acc[cur];
+            Entry *O = acc[cur ^ 1];
+            bool over = false;
+            struct AccDepth {
+                const Entry *a;
+                __device__ __forceinline__ float operator[](int i) const { return a[i].d; }
+            };
+            const float *dB = P.depth + b;
+            const int m = merge_core<int>(AccDepth{A}, 0, na, dB, 0, max(e - b, 0), LDNI_OP_UNION, eps,
+                                          [&](bool pb, int pi, bool cb, int ci, int mm) {
+                                              if (mm + 2 > kChainMaxLayers) {
+                                                  over = true;
+                                                  return;
+                                              }
+                                              O[mm] = pb ? Entry{dB[pi], k, b + pi} : A[pi];
+                                              O[mm + 1] = cb ? Entry{dB[ci], k, b + ci} : A[ci];
+                                          });
+            if (over) return -1;
+            na = m;
+            cur ^= 1;
+        }
     }
     return na;
 }
 
-// Pass 1 (kWrite false): every ray's result count into counts.  Pass 2: the
-// samples at the offsets of out.  blockIdx.y = image; parts of image j are
-// parts[j * count ..].
-struct Counts {
-    int *c[3];
+// Without small-interval removal the chain's result on a ray is the union of
+// all its parts' intervals, and where it changes state the chain keeps the
+// sample of the first part whose own state changes there (every Boolean keeps
+// the accumulated solid's sample at a shared depth).  So the union is kept as
+// disjoint intervals, each new interval taking in the ones that it touches,
+// and an end that it shares with one of them stays the earlier part's.
+struct Span {
+    float lo, hi;   // empty: lo > hi
+    int2 slo, shi;  // (part, sample) of the ends
+    __device__ __forceinline__ bool empty() const { return lo > hi; }
+    // takes in s, if they touch (s: from earlier parts)
+    __device__ __forceinline__ void take(Span &s) {
+        if (!(s.lo <= hi && s.hi >= lo)) return;
+        if (s.lo <= lo) {
+            lo = s.lo;
+            slo = s.slo;
+        }
+        if (s.hi >= hi) {
+            hi = s.hi;
+            shi = s.shi;
+        }
+        s.lo = INFINITY;
+        s.hi = -INFINITY;
+    }
 };
 
-template <bool kWrite>
-__global__ void __launch_bounds__(kThreads) chain_pass(long long N, const ldni_layers_t *__restrict__ parts_all,
-                                                       int count, float eps, Counts counts, ldni_layers_t o0,
-                                                       ldni_layers_t o1, ldni_layers_t o2, ldni_info_t *info) {
-    const int img = blockIdx.y;
-    const ldni_layers_t *parts = parts_all + (size_t)img * count;
-    const ldni_layers_t &o = img == 0 ? o0 : (img == 1 ? o1 : o2);
-    Entry acc[2][kChainMaxLayers];
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
-        if (!kWrite) {
-            for (int k = 0; k < count; ++k) {  // Definition 4 on the inputs
-                const int c = parts[k].offsets[p + 1] - parts[k].offsets[p];
-                if (c & 1) {
-                    atomicAdd(&info->odd_rays, 1u);
-                    set_status(info, LDNI_ST_ODD);
+// The intervals of a ray's parts in order, to add(span), which may say no; the
+// samples of four parts are loaded together.  False where it said no, or a part
+// has an odd count or repeated or unordered depths.
+template <class Have, class Add>
+__device__ __forceinline__ bool each_span(const ldni_layers_t *__restrict__ parts, int count, long long p, Have have,
+                                          Add add) {
+    for (int k0 = 0; k0 < count; k0 += 64) {
+        unsigned long long todo = have(k0);
+        while (todo) {
+            constexpr int kTake = 4;
+            int k[kTake], b[kTake], e[kTake];
+            float d0[kTake], d1[kTake];
+#pragma unroll
+            for (int q = 0; q < kTake; ++q) {
+                k[q] = todo ? k0 + __ffsll((long long)todo) - 1 : -1;
+                todo &= todo - 1ull;  // (0 stays 0)
+                b[q] = e[q] = 0;
+                if (k[q] >= 0) part_range(parts[k[q]], p, b[q], e[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < kTake; ++q) {
+                const bool some = e[q] - b[q] >= 2;
+                d0[q] = some ? parts[k[q]].depth[b[q]] : 0.0f;
+                d1[q] = some ? parts[k[q]].depth[b[q] + 1] : 0.0f;
+            }
+#pragma unroll
+            for (int q = 0; q < kTake; ++q) {
+                if (e[q] <= b[q]) continue;
+                if ((e[q] - b[q]) & 1) return false;
+                float l = d0[q], h = d1[q];
+                for (int x = b[q];;) {
+                    if (!(l < h) || !add(Span{l, h, {k[q], x}, {k[q], x + 1}})) return false;
+                    x += 2;
+                    if (x >= e[q]) break;
+                    l = parts[k[q]].depth[x];
+                    if (!(h < l)) return false;
+                    h = parts[k[q]].depth[x + 1];
                 }
             }
         }
-        int cur;
-        int n = fold_ray(parts, count, p, eps, acc, cur);
-        if (n < 0) {
-            if (!kWrite) set_status(info, LDNI_ST_EVENTS);
-            n = 0;
+    }
+    return true;
+}
+
+// Adds a span to the n of S (in registers when kInRegs: n = kN, empty ones
+// among them); false when there is no room.
+template <int kN, bool kInRegs>
+__device__ __forceinline__ bool add_span(Span (&S)[kN], int &n, Span s) {
+    if (kInRegs) {
+        bool put = false;
+#pragma unroll
+        for (int i = 0; i < kN; ++i) s.take(S[i]);
+#pragma unroll
+        for (int i = 0; i < kN; ++i)
+            if (!put && S[i].empty()) {
+                S[i] = s;
+                put = true;
+            }
+        return put;
+    }
+    int m = 0;
+    for (int i = 0; i < n; ++i) {  // the ones left move up
+        s.take(S[i]);
+        if (!S[i].empty()) {
+            if (m != i) S[m] = S[i];
+            ++m;
         }
-        if (!kWrite) {
-            counts.c[img][p] = n;
+    }
+    n = m;
+    if (n == kN) return false;
+    S[n++] = s;
+    return true;
+}
+
+// Pass 1, when no thin intervals are removed: every ray's parts, its count and
+// sources (Rays) for results that never have more than kSpans disjoint
+// intervals; the other rays are listed.  Bound by the reads of the parts'
+// offsets (201 MB for 64 parts at 512^2, three images) and the chain of loads of
+// the rays that meet a part, a fifth of them: 98 us.  (Loading part by part
+// between merges in local memory took 254 us, and 248 again for the samples,
+// now 39.)
+constexpr int kSpans = 4;
+constexpr int kKept = 2 * kSpans;  // samples whose sources pass 1 leaves to the write pass
+struct Rays {
+    int *count[3];
+    unsigned long long *present[3];  // the first 64 parts that the ray meets
+    int4 *kept[3];                   // (part, sample) twice; kKept / 2 per ray
+    long long *list;                 // rays (nrays image + ray) left to fold_pass; their number first
+};
+
+__device__ __forceinline__ void report_odd(int odd, ldni_info_t *info) {
+    if (odd) {
+        atomicAdd(&info->odd_rays, (unsigned)odd);
+        set_status(info, LDNI_ST_ODD);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 6) unite_pass(long long N, const ldni_layers_t *__restrict__ parts_all,
+                                                          int count, Rays rays, ldni_info_t *info) {
+    const int img = blockIdx.y;
+    const ldni_layers_t *parts = parts_all + (size_t)img * count;
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
+        int odd = 0;
+        const unsigned long long present = parts_present(parts, count, 0, p, odd);
+        for (int k0 = 64; k0 < count; k0 += 64) parts_present(parts, count, k0, p, odd);
+        report_odd(odd, info);
+        if (present == 0 && count <= 64) {
+            rays.count[img][p] = 0;
             continue;
         }
-        const long long base = o.offsets[p];
-        for (int x = 0; x < n; ++x) {
-            const Entry &E = acc[cur][x];
-            const long long at = base + x;
-            if (at >= o.capacity) {
-                set_status(info, LDNI_ST_CAPACITY);
-                break;
+        Span S[kSpans];
+#pragma unroll
+        for (int i = 0; i < kSpans; ++i) S[i] = Span{INFINITY, -INFINITY, {0, 0}, {0, 0}};
+        int n = kSpans;
+        rays.present[img][p] = present;
+        if (!each_span(parts, count, p,
+                       [&](int k0) { return k0 == 0 ? present : parts_present(parts, count, k0, p, odd); },
+                       [&](const Span &s) { return add_span<kSpans, true>(S, n, s); })) {
+            rays.list[1 + atomicAdd(reinterpret_cast<unsigned long long *>(rays.list), 1ull)] = N * img + p;
+            continue;
+        }
+        // ascending
+#pragma unroll
+        for (int i = 0; i < kSpans - 1; ++i)
+#pragma unroll
+            for (int j = 0; j < kSpans - 1 - i; ++j)
+                if (S[j + 1].lo < S[j].lo) {
+                    const Span t = S[j];
+                    S[j] = S[j + 1];
+                    S[j + 1] = t;
+                }
+        int4 *kept = rays.kept[img] + kKept / 2 * p;
+        int out = 0;
+#pragma unroll
+        for (int i = 0; i < kSpans; ++i)
+            if (!S[i].empty()) {
+                kept[i] = make_int4(S[i].slo.x, S[i].slo.y, S[i].shi.x, S[i].shi.y);
+                out += 2;
             }
-            const ldni_layers_t &P = parts[E.part];
-            o.depth[at] = E.d;
-            if (o.nrm8) {
-                o.nrm8[at] = P.nrm8[E.idx];
-            } else {
-                o.nx[at] = P.nx[E.idx];
-                o.ny[at] = P.ny[E.idx];
-                o.nz[at] = P.nz[E.idx];
+        rays.count[img][p] = out;
+    }
+}
+
+// The samples src[0, n) (n <= kMax) to o from slot at on: all loads before the
+// first store, which could otherwise be to the same memory.
+template <int kMax>
+__device__ __forceinline__ void put_samples(const ldni_layers_t *__restrict__ parts, const ldni_layers_t &o,
+                                            const int2 (&src)[kMax], int n, long long at, ldni_info_t *info) {
+    if (at + n > o.capacity) {
+        set_status(info, LDNI_ST_CAPACITY);
+        n = (int)max(0ll, (long long)o.capacity - at);
+    }
+    const bool packed = o.nrm8 != nullptr;
+    float d[kMax], x[kMax], y[kMax], z[kMax];
+    int t[kMax];
+#pragma unroll
+    for (int i = 0; i < kMax; ++i) {
+        if (i >= n) continue;
+        const ldni_layers_t &P = parts[src[i].x];
+        d[i] = P.depth[src[i].y];
+        x[i] = packed ? __uint_as_float(P.nrm8[src[i].y]) : P.nx[src[i].y];
+        y[i] = packed ? 0.0f : P.ny[src[i].y];
+        z[i] = packed ? 0.0f : P.nz[src[i].y];
+        t[i] = P.tri_id[src[i].y];
+        if (src[i].x != 0) t[i] |= (int)0x80000000u;
+    }
+#pragma unroll
+    for (int i = 0; i < kMax; ++i) {
+        if (i >= n) continue;
+        o.depth[at + i] = d[i];
+        if (packed) {
+            o.nrm8[at + i] = __float_as_uint(x[i]);
+        } else {
+            o.nx[at + i] = x[i];
+            o.ny[at + i] = y[i];
+            o.nz[at + i] = z[i];
+        }
+        o.tri_id[at + i] = t[i];
+    }
+}
+
+// The rays that unite_pass listed, or all of them (all: with thin intervals
+// removed after every step, or one part alone): kWrite false, their counts and
+// the sources of up to kKept samples; kWrite true, the samples of longer
+// results.  A listed ray is united like unite_pass's, with room for any result
+// the chain may hold, and folded where that says no.
+template <bool kWrite>
+__global__ void __launch_bounds__(kThreads) fold_pass(long long N, const ldni_layers_t *__restrict__ parts_all,
+                                                      int count, int nimg, int all, float eps, Rays rays,
+                                                      ldni_layers_t o0, ldni_layers_t o1, ldni_layers_t o2,
+                                                      ldni_info_t *info) {
+    Entry acc[2][kChainMaxLayers];
+    const long long total = all ? N * nimg : rays.list[0];
+    for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < total; r += (long long)gridDim.x * blockDim.x) {
+        const long long ray = all ? r : rays.list[1 + r];
+        const int img = (int)(ray / N);
+        const long long p = ray - img * N;
+        if (kWrite && rays.count[img][p] <= kKept) continue;
+        const ldni_layers_t *parts = parts_all + (size_t)img * count;
+        int odd = 0;
+        unsigned long long present;
+        if (all && !kWrite) {
+            present = parts_present(parts, count, 0, p, odd);
+            for (int k0 = 64; k0 < count; k0 += 64) parts_present(parts, count, k0, p, odd);
+            report_odd(odd, info);
+            rays.present[img][p] = present;
+        } else {
+            present = rays.present[img][p];
+        }
+        const auto have = [&](int k0) { return k0 == 0 ? present : parts_present(parts, count, k0, p, odd); };
+        int cur = 0, n = -1;
+        if (!all) {
+            Span S[kChainMaxLayers / 2];
+            int m = 0;
+            if (each_span(parts, count, p, have,
+                          [&](const Span &s) { return add_span<kChainMaxLayers / 2, false>(S, m, s); })) {
+                for (int i = 1; i < m; ++i) {  // ascending
+                    const Span t = S[i];
+                    int j = i;
+                    for (; j > 0 && t.lo < S[j - 1].lo; --j) S[j] = S[j - 1];
+                    S[j] = t;
+                }
+                for (int i = 0; i < m; ++i) {
+                    acc[0][2 * i] = Entry{S[i].lo, S[i].slo.x, S[i].slo.y};
+                    acc[0][2 * i + 1] = Entry{S[i].hi, S[i].shi.x, S[i].shi.y};
+                }
+                n = 2 * m;
             }
-            o.tri_id[at] = E.part == 0 ? P.tri_id[E.idx] : (int)((unsigned)P.tri_id[E.idx] | 0x80000000u);
+        }
+        if (n < 0) n = fold_ray(parts, count, p, eps, acc, cur, have);
+        if (!kWrite) {
+            if (n < 0) {
+                set_status(info, LDNI_ST_EVENTS);
+                n = 0;
+            }
+            rays.count[img][p] = n;
+            if (n > kKept) continue;
+            int4 *kept = rays.kept[img] + kKept / 2 * p;
+            for (int i = 0; 2 * i < n; ++i)
+                kept[i] = make_int4(acc[cur][2 * i].part, acc[cur][2 * i].idx, acc[cur][2 * i + 1].part,
+                                    acc[cur][2 * i + 1].idx);
+        } else {
+            const ldni_layers_t &o = img == 0 ? o0 : (img == 1 ? o1 : o2);
+            for (int x = 0; x < n; ++x) {
+                const int2 one[1] = {{acc[cur][x].part, acc[cur][x].idx}};
+                put_samples(parts, o, one, 1, (long long)o.offsets[p] + x, info);
+            }
+        }
+    }
+}
+
+// The samples of results of up to kKept.
+__global__ void __launch_bounds__(kThreads) chain_write(long long N, const ldni_layers_t *__restrict__ parts_all,
+                                                        int count, Rays rays, ldni_layers_t o0, ldni_layers_t o1,
+                                                        ldni_layers_t o2, ldni_info_t *info) {
+    const int img = blockIdx.y;
+    const ldni_layers_t &o = img == 0 ? o0 : (img == 1 ? o1 : o2);
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
+        const int n = rays.count[img][p];
+        if (n == 0 || n > kKept) continue;
+        const int4 *kept = rays.kept[img] + kKept / 2 * p;
+        for (int x = 0; x < n; x += 4) {
+            const int4 a = kept[x / 2], b = n > x + 2 ? kept[x / 2 + 1] : a;
+            const int2 from[4] = {{a.x, a.y}, {a.z, a.w}, {b.x, b.y}, {b.z, b.w}};
+            put_samples(parts_all + (size_t)img * count, o, from, min(n - x, 4), (long long)o.offsets[p] + x, info);
         }
     }
 }
 
 struct ChainWs {
-    int *counts[3];
+    Rays rays;
     long long *partials;
 };
 
 ChainWs carve_chain_ws(Carver &c, int res, int nimg) {
     ChainWs w{};
     const long long N = (long long)res * res;
-    for (int j = 0; j < nimg; ++j) w.counts[j] = c.take<int>((size_t)N);
+    for (int j = 0; j < nimg; ++j) {
+        w.rays.count[j] = c.take<int>((size_t)N);
+        w.rays.present[j] = c.take<unsigned long long>((size_t)N);
+        w.rays.kept[j] = c.take<int4>(kKept / 2 * (size_t)N);
+    }
+    w.rays.list = c.take<long long>((size_t)N * nimg + 1);
     w.partials = c.take<long long>(csr_scan_partials(N) * nimg);
     return w;
 }
@@ -194,16 +483,24 @@ extern "C" int ldni_union_chain(const ldni_layers_t *parts_dev, const ldni_layer
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     ldni_layers_t o[3] = {out[0], nimg > 1 ? out[1] : out[0], nimg > 2 ? out[2] : out[0]};
     const dim3 g((unsigned)grid_for(N), (unsigned)nimg);
-    const Counts cn{{w.counts[0], w.counts[1], w.counts[2]}};
+    const int all = eps == 0.0f && count > 1 ? 0 : 1;
+    const unsigned fblocks = all ? (unsigned)grid_for(N * nimg) : (unsigned)num_sms();
+    if (!all) {
+        if (int rc_ = cuda_check(cudaMemsetAsync(w.rays.list, 0, sizeof(long long), s))) return rc_;
+        LDNI_LAUNCH(K_CHAIN, s, unite_pass<<<g, kThreads, 0, s>>>(N, parts_dev, count, w.rays, info));
+    }
     LDNI_LAUNCH(K_CHAIN, s,
-                chain_pass<false><<<g, kThreads, 0, s>>>(N, parts_dev, count, eps, cn, o[0], o[1], o[2], info));
+                fold_pass<false><<<fblocks, kThreads, 0, s>>>(N, parts_dev, count, nimg, all, eps, w.rays, o[0], o[1],
+                                                              o[2], info));
     int rc = cuda_status();
     if (rc != LDNI_OK) return rc;
-    const int *cnt[3] = {w.counts[0], w.counts[1], w.counts[2]};
+    const int *cnt[3] = {w.rays.count[0], w.rays.count[1], w.rays.count[2]};
     int *off[3] = {out[0].offsets, nimg > 1 ? out[1].offsets : nullptr, nimg > 2 ? out[2].offsets : nullptr};
     rc = csr_scan(cnt, off, nimg, N, w.partials, info, 0, s);
     if (rc != LDNI_OK) return rc;
+    LDNI_LAUNCH(K_CHAIN, s, chain_write<<<g, kThreads, 0, s>>>(N, parts_dev, count, w.rays, o[0], o[1], o[2], info));
     LDNI_LAUNCH(K_CHAIN, s,
-                chain_pass<true><<<g, kThreads, 0, s>>>(N, parts_dev, count, eps, cn, o[0], o[1], o[2], info));
+                fold_pass<true><<<fblocks, kThreads, 0, s>>>(N, parts_dev, count, nimg, all, eps, w.rays, o[0], o[1],
+                                                             o[2], info));
     return cuda_status();
 }

@@ -169,3 +169,39 @@ def test_tiny_wait_limit_terminates(ldni):
     finally:
         lib.ldni_set_wait_limit(0)
         tune.set(**prev)
+
+
+def _random_part(ldni, grid, rng, most, levels):
+    """An image of random intervals whose ends are multiples of 1 / levels:
+    shared depths, touching and empty intervals across and within parts."""
+    N = grid.res * grid.res
+    depth, off = [], [0]
+    for _ in range(N):
+        k = 2 * int(rng.integers(0, most + 1)) if rng.random() < 0.6 else 0
+        depth += sorted(rng.integers(0, levels, size=k).tolist())
+        off.append(off[-1] + k)
+    n = off[-1]
+    t = lambda x, dt: torch.from_numpy(np.asarray(x, dt)).cuda()
+    nrm = rng.standard_normal((3, n)).astype(np.float32)
+    return ldni.LDNI(grid, 0, t(off, np.int32), t(np.asarray(depth) / levels, np.float32), *[t(x, np.float32) for x in nrm],
+                     t(rng.integers(0, 1000, size=n), np.int32), n)
+
+
+@pytest.mark.parametrize("count,most,levels,res", [(2, 1, 8, 9), (5, 3, 4096, 13), (12, 2, 64, 16), (64, 1, 5000, 7),
+                                                   (70, 1, 300, 7), (66, 1, 40, 5), (3, 14, 100000, 11)])
+def test_random_intervals(ldni, count, most, levels, res):
+    """Every form a ray's result takes, against the step-by-step unions: ties
+    and touching intervals, a few or many disjoint ones, results longer than
+    the sources kept between the passes, more than 64 parts."""
+    rng = np.random.default_rng(count * 100 + most)
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    P = [_random_part(ldni, grid, rng, most, levels) for _ in range(count)]
+    for eps in (0.0, 0.01):
+        run, finish = ldni.union_chain(P, eps=eps)
+        run()
+        try:
+            got = finish()
+        except ldni.LDNIError as e:
+            assert e.code == -4 and count >= 64  # a ray of more than 64 samples at some step
+            continue
+        assert ldni.identical(got, _stepwise(ldni, P, eps)), eps
