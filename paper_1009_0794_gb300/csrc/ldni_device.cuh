@@ -55,6 +55,21 @@ __device__ __forceinline__ void face_normal(const float3 &p0, const float3 &p1, 
     }
 }
 
+// Count words: a ray's crossings so far in the low 30 bits (a ray crosses a
+// triangle at most once and a mesh has fewer than 2^30), how many of them leave
+// the solid, modulo 4, in the top two.  One atomic per crossing keeps both, and
+// a ray of two crossings is exactly an entry and an exit iff the word is
+// kPairWord.
+constexpr unsigned kCountMask = (1u << 30) - 1u, kPairWord = (1u << 30) | 2u;
+__device__ __forceinline__ int count_word(int exiting) { return (int)(1u + ((unsigned)exiting << 30)); }
+__device__ __forceinline__ int count_of(int word) { return (int)((unsigned)word & kCountMask); }
+
+// Cursors: the ray's first slot, and in bit 31 whether it is a pair, whose
+// entry takes that slot and whose exit the next one without any atomic.
+__device__ __forceinline__ int make_cursor(int first, int word) {
+    return (int)((unsigned)first | ((unsigned)word == kPairWord ? 0x80000000u : 0u));
+}
+
 // Packed approximate normal (Section 3 item 1): three 8-bit codes
 // q = rint(fl32(fl32(n + 1) * 127.5)), half to even, clamped to [0, 255].
 __device__ __forceinline__ unsigned normal_code8(float n) {

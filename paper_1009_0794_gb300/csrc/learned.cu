@@ -45,8 +45,7 @@ constexpr int kMaxLayerCap = 64;   // largest k_t the layout hands out
 constexpr int kOnepassBlocksPerSm = LDNI_ONEPASS_BLOCKS;
 
 struct LImg {
-    int *count[3];
-    int *exitc[3];               // crossings whose face leaves the solid (two-layer tiles)
+    int *count[3];               // count words
     const int *offsets[3];
     float *depth[3];
     float *nx[3];
@@ -307,13 +306,12 @@ __device__ __forceinline__ void onepass_hit(int a, long long p, float d, int t, 
     const int tile = (int)(p >> kTileBits);
     const int kt = pick3(o.kcap, a)[tile];
     if (kt == 2) {
-        atomicAdd(pick3(o.count, a) + p, 1);
-        if (exiting) atomicAdd(pick3(o.exitc, a) + p, 1);
+        atomicAdd(pick3(o.count, a) + p, count_word(exiting));
         const long long slot = pick3(o.slab_base, a)[tile] + (p & (kTilePix - 1)) * 2 + exiting;
         if (range_ok(slot, slot + 1, o.slab_cap, o.info)) o.slab[slot] = make_int2(__float_as_int(d), t);
         return;
     }
-    const int k = atomicAdd(pick3(o.count, a) + p, 1);
+    const int k = count_of(atomicAdd(pick3(o.count, a) + p, count_word(exiting)));
     if (k < kt) {
         const long long slot = pick3(o.slab_base, a)[tile] + (p & (kTilePix - 1)) * kt + k;
         if (range_ok(slot, slot + 1, o.slab_cap, o.info)) o.slab[slot] = make_int2(__float_as_int(d), t);
@@ -335,6 +333,7 @@ __device__ __forceinline__ void onepass_hits(const Setup32 &S, unsigned m, int t
                                              const LImg &o) {
     const int wdiv = (256 + S.w - 1) / S.w;  // y = (b * wdiv) >> 8 = b / w for b < 16, w <= 16
     int *cnt = pick3(o.count, A);
+    const int word = count_word(S.exiting);
     const int *kc = pick3(o.kcap, A);
     const long long *sb = pick3(o.slab_base, A);
     while (m) {
@@ -357,15 +356,14 @@ __device__ __forceinline__ void onepass_hits(const Setup32 &S, unsigned m, int t
             base[u] = v[u] ? sb[tile] : 0;
         }
 #pragma unroll
-        for (int u = 0; u < kHitBatch; ++u) k[u] = v[u] && kt[u] != 2 ? atomicAdd(cnt + pr[u], 1) : 0;
+        for (int u = 0; u < kHitBatch; ++u) k[u] = v[u] && kt[u] != 2 ? count_of(atomicAdd(cnt + pr[u], word)) : 0;
 #pragma unroll
         for (int u = 0; u < kHitBatch; ++u) {
             if (!v[u]) continue;
             const int q = pr[u] & (kTilePix - 1);
             long long slot;
             if (kt[u] == 2) {
-                atomicAdd(cnt + pr[u], 1);
-                if (S.exiting) atomicAdd(pick3(o.exitc, A) + pr[u], 1);
+                atomicAdd(cnt + pr[u], word);
                 slot = base[u] + q * 2 + S.exiting;
             } else if (k[u] < kt[u]) {
                 slot = base[u] + (long long)q * kt[u] + k[u];
@@ -448,7 +446,7 @@ __global__ void __launch_bounds__(kThreads) onepass_big(const float *__restrict_
 __device__ __forceinline__ void redo_hit(int a, long long p, float d, int t, const LImg &o, const float3 &n,
                                          ldni_info_t *info) {
     if (!pick3(o.over, a)[p >> kTileBits]) return;
-    const int k = atomicSub(pick3(o.count, a) + p, 1) - 1;
+    const int k = count_of(atomicSub(pick3(o.count, a) + p, 1)) - 1;
     const long long slot = (long long)pick3(o.offsets, a)[p] + k;
     if (k < 0 || slot >= pick3(o.cap, a)) {
         set_status(info, LDNI_ST_CAPACITY);
@@ -770,7 +768,6 @@ __global__ void normalise_kernel(int ntiles, long long nrays, int naxes, const f
 
 struct LearnedWs {
     int *count[3];
-    int *exitc[3];
     int *big_n;
     int *any_over;
     float *feat[3];
@@ -793,17 +790,14 @@ LearnedWs carve_learned_ws(Carver &c, long long nt, int res, int naxes, long lon
     const long long stride = (N + 63) / 64 * 64;
     const long long ntiles = (N + kTilePix - 1) / kTilePix;
     const long long tstride = (ntiles + 63) / 64 * 64;
-    // one cleared block: counts | 64 ints (queue counts at 0 and 1, any_over at 8, slab cursor at
-    // 10..11) | features | overflow marks | exiting counts | deep-ray marks
-    const size_t deep_at = (size_t)(stride * naxes + 64 + tstride * naxes * kRawFeat + tstride * naxes + stride * naxes);
+    // one cleared block: count words | 64 ints (queue counts at 0 and 1, any_over at 8, slab cursor at
+    // 10..11) | features | overflow marks | deep-ray marks
+    const size_t deep_at = (size_t)(stride * naxes + 64 + tstride * naxes * kRawFeat + tstride * naxes);
     const long long dstride = ((N + 1023) / 1024 + 63) / 64 * 64;  // words of chunk marks per image
     const size_t ints = deep_at + (size_t)dstride * naxes;
     int *block = c.take<int>(ints);
     for (int a = 0; a < naxes; ++a) {
         w.count[a] = block ? block + (size_t)a * stride : nullptr;
-        w.exitc[a] = block ? block + (size_t)stride * naxes + 64 + (size_t)tstride * naxes * kRawFeat +
-                                 (size_t)tstride * naxes + (size_t)a * stride
-                           : nullptr;
         w.feat[a] = block ? reinterpret_cast<float *>(block + (size_t)stride * naxes + 64) + (size_t)a * tstride * kRawFeat
                           : nullptr;
         w.over[a] = block ? block + (size_t)stride * naxes + 64 + (size_t)tstride * naxes * kRawFeat + (size_t)a * tstride
@@ -882,7 +876,6 @@ extern "C" int ldni_sample_learned(const float *verts, int64_t nv, const int32_t
         if (!L.offsets || L.capacity < 0 || !samples_ok(L))
             return LDNI_EINVAL;
         o.count[a] = w.count[k];
-        o.exitc[a] = w.exitc[k];
         o.offsets[a] = L.offsets;
         o.depth[a] = L.depth;
         normal_arrays(L, o.nx[a], o.ny[a], o.nz[a]);
@@ -938,12 +931,11 @@ extern "C" int ldni_sample_learned(const float *verts, int64_t nv, const int32_t
     if (rc != LDNI_OK) return rc;
     ScanVerify ver{};
     for (int k = 0; k < naxes; ++k) {
-        ver.exitc[k] = w.exitc[k];
         ver.kcap[k] = w.kcap[k];
         ver.over[k] = w.over[k];
     }
     ver.any_over = w.any_over;
-    rc = csr_scan(cnt, off, naxes, N, w.scan_words, info, ax_lo, s, nullptr, &ver);
+    rc = csr_scan(cnt, off, naxes, N, w.scan_words, info, ax_lo, s, nullptr, &ver, kScanWords);
     if (rc != LDNI_OK) return rc;
     if (nt > 0) {
             // the triangle sweep on as many blocks as stay resident (every block

@@ -374,6 +374,46 @@ struct RayOut {
     float *X, *Y, *Z;  // FP32 normals, or packed 8-bit normals in X with Y = Z = nullptr
 };
 
+// Takes the next slot of ray p (cursor word at cur + p) for a crossing that
+// leaves the solid or enters it: a pair's two slots follow from that alone, so
+// its cursor is only read, and stays in L1 for the neighbouring crossings.
+__device__ __forceinline__ long long claim_slot(int *cur, long long p, int exiting) {
+    const unsigned c = (unsigned)cur[p];
+    return c & 0x80000000u ? (long long)(c & 0x7fffffffu) + exiting : (long long)(unsigned)atomicAdd(cur + p, 1);
+}
+
+// Unit normals of a mesh's triangles, w: packed 8-bit codes.  An index outside
+// the mesh (a slot that no crossing filled: the mesh changed between count and
+// fill) reads as triangle 0.
+struct NormalTable {
+    const float4 *n;
+    int nt;
+    __device__ __forceinline__ float4 operator()(int t) const { return n[(unsigned)t < (unsigned)nt ? t : 0]; }
+};
+
+__device__ __forceinline__ void put_normal(const RayOut &o, long long at, const float4 &q) {
+    o.X[at] = o.Y ? q.x : q.w;
+    if (o.Y) {
+        o.Y[at] = q.y;
+        o.Z[at] = q.z;
+    }
+}
+
+// source of a ray's samples that were filled without normals
+struct TableSrc {
+    RayOut o;
+    long long b;
+    NormalTable nrm;
+    __device__ __forceinline__ void operator()(int i, float &d, int &t, float &x, float &y, float &z) const {
+        d = o.D[b + i];
+        t = o.Tr[b + i];
+        const float4 q = nrm(t);
+        x = o.Y ? q.x : q.w;
+        y = q.y;
+        z = q.z;
+    }
+};
+
 // source of a ray's samples that sits where the ordered ray goes
 struct InPlace {
     RayOut o;
@@ -515,6 +555,61 @@ __device__ __forceinline__ void order_warp_rays(long long b, int n, long long sb
         else
             rank_long(bb, nn, oo, st, lane);
     }
+}
+
+// Orders the rays of a warp's lanes whose samples were filled without normals,
+// and gives every sample its normal.  Every lane calls it, with n = 0 when it
+// has none.  pairs8: the arrays are 8-byte aligned.
+template <bool kOneOut>
+__device__ __forceinline__ void finish_warp_rays(long long b, int n, const RayOut &r, const NormalTable &nrm, bool pairs8,
+                                                 SortStage &st, int lane) {
+    if (n == 2) {  // the common case: everything in registers
+        const bool even = pairs8 && (b & 1) == 0;  // one 8-byte access per field
+        float d0, d1;
+        int t0, t1;
+        if (even) {
+            const float2 d = *reinterpret_cast<const float2 *>(r.D + b);
+            const int2 t = *reinterpret_cast<const int2 *>(r.Tr + b);
+            d0 = d.x, d1 = d.y, t0 = t.x, t1 = t.y;
+        } else {
+            d0 = r.D[b], d1 = r.D[b + 1], t0 = r.Tr[b], t1 = r.Tr[b + 1];
+        }
+        if (key_less(d1, t1, d0, t0)) {
+            r.D[b] = d1, r.D[b + 1] = d0;
+            r.Tr[b] = t1, r.Tr[b + 1] = t0;
+            const int t = t0;
+            t0 = t1;
+            t1 = t;
+        }
+        const float4 q0 = nrm(t0), q1 = nrm(t1);
+        if (even) {
+            *reinterpret_cast<float2 *>(r.X + b) = r.Y ? make_float2(q0.x, q1.x) : make_float2(q0.w, q1.w);
+            if (r.Y) {
+                *reinterpret_cast<float2 *>(r.Y + b) = make_float2(q0.y, q1.y);
+                *reinterpret_cast<float2 *>(r.Z + b) = make_float2(q0.z, q1.z);
+            }
+        } else {
+            put_normal(r, b, q0);
+            put_normal(r, b + 1, q1);
+        }
+        n = 0;
+    } else if (n == 1) {
+        put_normal(r, b, nrm(r.Tr[b]));
+        n = 0;
+    }
+    // rays that are ordered in place get their normals first
+    unsigned longer = __ballot_sync(0xffffffffu, n > kWarpSortMax);
+    while (longer) {
+        const int src = __ffs(longer) - 1;
+        longer &= longer - 1;
+        const RayOut o = kOneOut ? r : shfl_out(r, src);
+        const long long bb = __shfl_sync(0xffffffffu, b, src);
+        const int nn = __shfl_sync(0xffffffffu, n, src);
+        for (int i = lane; i < nn; i += 32) put_normal(o, bb + i, nrm(o.Tr[bb + i]));
+        __syncwarp();
+    }
+    order_warp_rays<kOneOut>(
+        b, n, b, [&](long long, long long at, const RayOut &o) { return TableSrc{o, at, nrm}; }, r, st, lane);
 }
 
 }  // namespace ldni

@@ -28,9 +28,16 @@ struct AxisPtrs {
     const int *counts[3];
     int *offsets[3];
     int2 *tinfo[3];
+    int *cursor[3];  // the counts, overwritten by cursors (kScanCursors)
     ScanVerify ver;
     bool verify;
 };
+
+// counts of four count words (kForm: ScanForm)
+template <int kForm>
+__device__ __forceinline__ int4 counts_of(int4 v) {
+    return kForm != kScanCounts ? make_int4(count_of(v.x), count_of(v.y), count_of(v.z), count_of(v.w)) : v;
+}
 
 // 16-byte load when the address allows it (c + e aligned), scalar otherwise
 __device__ __forceinline__ int4 load4(const int *c, long long e, long long N, bool vec) {
@@ -41,6 +48,17 @@ __device__ __forceinline__ int4 load4(const int *c, long long e, long long N, bo
     if (e + 2 < N) v.z = c[e + 2];
     if (e + 3 < N) v.w = c[e + 3];
     return v;
+}
+
+__device__ __forceinline__ void store4(int *c, long long e, long long N, bool vec, const int4 &v) {
+    if (vec && e + 3 < N) {
+        *reinterpret_cast<int4 *>(c + e) = v;
+        return;
+    }
+    if (e < N) c[e] = v.x;
+    if (e + 1 < N) c[e + 1] = v.y;
+    if (e + 2 < N) c[e + 2] = v.z;
+    if (e + 3 < N) c[e + 3] = v.w;
 }
 
 __device__ __forceinline__ int clamp_int(long long x) { return (int)(x < INT_MAX ? x : INT_MAX); }
@@ -54,31 +72,26 @@ constexpr int kMaxSumChunks = 1024;
 #define LDNI_SCAN_ONE_LAUNCH 0
 #endif
 
+// v: the counts or count words as stored; tsum: the sums of the counts
+template <int kForm>
 __device__ __forceinline__ void load_chunk(const int *cnt, long long base, long long N, int4 (&v)[kSlices],
                                            long long (&tsum)[kSlices]) {
     const bool vec_in = ((reinterpret_cast<uintptr_t>(cnt) & 15) == 0);
 #pragma unroll
     for (int m = 0; m < kSlices; ++m) {
         v[m] = load4(cnt, base + (long long)m * kSlice + threadIdx.x * kVec, N, vec_in);
-        tsum[m] = (long long)v[m].x + v[m].y + v[m].z + v[m].w;
+        const int4 c = counts_of<kForm>(v[m]);
+        tsum[m] = (long long)c.x + c.y + c.z + c.w;
     }
 }
 
 // Two-layer check of one-pass sampling (ScanVerify) for chunk c of image a.
-__device__ __forceinline__ void verify_chunk(const AxisPtrs &ap, int a, int c, long long base, long long N,
-                                             const int4 (&v)[kSlices]) {
+__device__ __forceinline__ void verify_chunk(const AxisPtrs &ap, int a, int c, const int4 (&v)[kSlices]) {
     if (!ap.verify || ap.ver.kcap[a][c] != 2) return;  // block-uniform
-    const int *ex = ap.ver.exitc[a];
-    const bool vec_ex = ((reinterpret_cast<uintptr_t>(ex) & 15) == 0);
+    const auto good = [](int w) { return w == 0 || (unsigned)w == kPairWord; };
     bool bad = false;
 #pragma unroll
-    for (int m = 0; m < kSlices; ++m) {
-        const int4 x = load4(ex, base + (long long)m * kSlice + threadIdx.x * kVec, N, vec_ex);
-        bad |= !(v[m].x == 0 || (v[m].x == 2 && x.x == 1));
-        bad |= !(v[m].y == 0 || (v[m].y == 2 && x.y == 1));
-        bad |= !(v[m].z == 0 || (v[m].z == 2 && x.z == 1));
-        bad |= !(v[m].w == 0 || (v[m].w == 2 && x.w == 1));
-    }
+    for (int m = 0; m < kSlices; ++m) bad |= !(good(v[m].x) && good(v[m].y) && good(v[m].z) && good(v[m].w));
     if (__syncthreads_or(bad) && threadIdx.x == 0) {
         ap.ver.over[a][c] = 1;
         *ap.ver.any_over = 1;
@@ -104,6 +117,7 @@ __device__ __forceinline__ long long warp_inclusive(long long x, int lane) {
 
 // ---- one-launch form: decoupled look-back ---------------------------------------
 
+template <int kForm>
 __global__ void __launch_bounds__(kThreads, 6) scan_lookback(AxisPtrs ap, long long N, int nchunk,
                                                              unsigned long long *words, ldni_info_t *info,
                                                              int info_base, int spin_limit) {
@@ -126,8 +140,8 @@ __global__ void __launch_bounds__(kThreads, 6) scan_lookback(AxisPtrs ap, long l
     {
         int4 v[kSlices];
         long long tsum[kSlices];
-        load_chunk(ap.counts[a], base, N, v, tsum);
-        verify_chunk(ap, a, c, base, N, v);
+        load_chunk<kForm>(ap.counts[a], base, N, v, tsum);
+        verify_chunk(ap, a, c, v);
 #pragma unroll
         for (int m = 0; m < kSlices; ++m) {
             sv[m][threadIdx.x] = v[m];
@@ -164,15 +178,14 @@ __global__ void __launch_bounds__(kThreads, 6) scan_lookback(AxisPtrs ap, long l
         const long long e = base + (long long)m * kSlice + threadIdx.x * kVec;
         const long long o0 = b0 + excl[m];
         const int4 v = sv[m][threadIdx.x];  // this thread's own counts
-        const int4 w = make_int4(clamp_int(o0), clamp_int(o0 + v.x), clamp_int(o0 + v.x + v.y),
-                                 clamp_int(o0 + v.x + v.y + v.z));
-        if (vec_ok && e + 3 < N) {
-            *reinterpret_cast<int4 *>(out + e) = w;
-        } else {
-            if (e < N) out[e] = w.x;
-            if (e + 1 < N) out[e + 1] = w.y;
-            if (e + 2 < N) out[e + 2] = w.z;
-            if (e + 3 < N) out[e + 3] = w.w;
+        const int4 n = counts_of<kForm>(v);
+        const int4 w = make_int4(clamp_int(o0), clamp_int(o0 + n.x), clamp_int(o0 + n.x + n.y),
+                                 clamp_int(o0 + n.x + n.y + n.z));
+        store4(out, e, N, vec_ok, w);
+        if (kForm == kScanCursors) {
+            int *cur = ap.cursor[a];
+            store4(cur, e, N, (reinterpret_cast<uintptr_t>(cur) & 15) == 0,
+                   make_int4(make_cursor(w.x, v.x), make_cursor(w.y, v.y), make_cursor(w.z, v.z), make_cursor(w.w, v.w)));
         }
     }
     if (c == nchunk - 1 && threadIdx.x == 0) {
@@ -189,14 +202,15 @@ __global__ void __launch_bounds__(kThreads, 6) scan_lookback(AxisPtrs ap, long l
 // leave one value per warp (and per slice) in shared memory, which every
 // thread then adds up itself.
 
+template <int kForm>
 __global__ void __launch_bounds__(kThreads) scan_sums(AxisPtrs ap, long long N, int nchunk, long long *sums) {
     __shared__ long long sh[kWarps];
     const int a = blockIdx.y, c = blockIdx.x;
     const long long base = (long long)c * kChunk;
     int4 v[kSlices];
     long long tsum[kSlices];
-    load_chunk(ap.counts[a], base, N, v, tsum);
-    verify_chunk(ap, a, c, base, N, v);
+    load_chunk<kForm>(ap.counts[a], base, N, v, tsum);
+    verify_chunk(ap, a, c, v);
     const long long ws = warp_sum(tsum[0] + tsum[1] + tsum[2] + tsum[3]);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = ws;
     __syncthreads();
@@ -208,6 +222,7 @@ __global__ void __launch_bounds__(kThreads) scan_sums(AxisPtrs ap, long long N, 
     }
 }
 
+template <int kForm>
 __global__ void __launch_bounds__(kThreads, 6) scan_prefix(AxisPtrs ap, long long N, int nchunk, const long long *sums,
                                                         ldni_info_t *info, int info_base) {
     __shared__ long long sh[kSlices + 1][kWarps];  // per slice: warp totals; last row: warp sums of `before`
@@ -222,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, 6) scan_prefix(AxisPtrs ap, long lon
     {
         int4 v[kSlices];
         long long tsum[kSlices];
-        load_chunk(ap.counts[a], base, N, v, tsum);
+        load_chunk<kForm>(ap.counts[a], base, N, v, tsum);
 #pragma unroll
         for (int m = 0; m < kSlices; ++m) {
             sv[m][threadIdx.x] = v[m];
@@ -261,15 +276,14 @@ __global__ void __launch_bounds__(kThreads, 6) scan_prefix(AxisPtrs ap, long lon
         const long long e = base + (long long)m * kSlice + threadIdx.x * kVec;
         const long long o0 = b0 + excl[m];
         const int4 v = sv[m][threadIdx.x];  // this thread's own counts: no barrier needed
-        const int4 w = make_int4(clamp_int(o0), clamp_int(o0 + v.x), clamp_int(o0 + v.x + v.y),
-                                 clamp_int(o0 + v.x + v.y + v.z));
-        if (vec_ok && e + 3 < N) {
-            *reinterpret_cast<int4 *>(out + e) = w;
-        } else {
-            if (e < N) out[e] = w.x;
-            if (e + 1 < N) out[e + 1] = w.y;
-            if (e + 2 < N) out[e + 2] = w.z;
-            if (e + 3 < N) out[e + 3] = w.w;
+        const int4 n = counts_of<kForm>(v);
+        const int4 w = make_int4(clamp_int(o0), clamp_int(o0 + n.x), clamp_int(o0 + n.x + n.y),
+                                 clamp_int(o0 + n.x + n.y + n.z));
+        store4(out, e, N, vec_ok, w);
+        if (kForm == kScanCursors) {
+            int *cur = ap.cursor[a];
+            store4(cur, e, N, (reinterpret_cast<uintptr_t>(cur) & 15) == 0,
+                   make_int4(make_cursor(w.x, v.x), make_cursor(w.y, v.y), make_cursor(w.z, v.z), make_cursor(w.w, v.w)));
         }
     }
     if (c == nchunk - 1 && threadIdx.x == 0) {
@@ -293,8 +307,31 @@ size_t csr_scan_partials(long long N) {
     return (size_t)(n + 1);  // one status word per chunk + the ticket
 }
 
+namespace {
+
+template <int kForm>
+int launch_scan(const AxisPtrs &ap, int naxes, long long N, int nchunk, long long *partials, ldni_info_t *info,
+                int info_base, cudaStream_t s) {
+    if (!LDNI_SCAN_ONE_LAUNCH && nchunk <= kMaxSumChunks) {
+        LDNI_LAUNCH(K_SCAN_TOP, s, scan_sums<kForm><<<dim3(nchunk, naxes), kThreads, 0, s>>>(ap, N, nchunk, partials));
+        LDNI_LAUNCH(K_SCAN_DOWN, s,
+                    scan_prefix<kForm><<<dim3(nchunk, naxes), kThreads, 0, s>>>(ap, N, nchunk, partials, info,
+                                                                               info_base));
+        return cuda_status();
+    }
+    unsigned long long *words = reinterpret_cast<unsigned long long *>(partials);
+    if (int rc_ = cuda_check(cudaMemsetAsync(words, 0, sizeof(unsigned long long) * (size_t)(nchunk + 1) * naxes, s))) return rc_;
+    LDNI_LAUNCH(K_SCAN_DOWN, s,
+                scan_lookback<kForm><<<dim3(nchunk, naxes), kThreads, 0, s>>>(ap, N, nchunk, words, info, info_base,
+                                                                               wait_limit()));
+    return cuda_status();
+}
+
+}  // namespace
+
 int csr_scan(const int *const *counts, int *const *offsets, int naxes, long long N, long long *partials,
-             ldni_info_t *info, int info_base, cudaStream_t s, int2 *const *tinfo, const ScanVerify *verify) {
+             ldni_info_t *info, int info_base, cudaStream_t s, int2 *const *tinfo, const ScanVerify *verify,
+             ScanForm form) {
     AxisPtrs ap{};
     if (verify) {
         ap.ver = *verify;
@@ -304,24 +341,18 @@ int csr_scan(const int *const *counts, int *const *offsets, int naxes, long long
         ap.counts[a] = counts[a];
         ap.offsets[a] = offsets[a];
         ap.tinfo[a] = tinfo ? tinfo[a] : nullptr;
+        ap.cursor[a] = form == kScanCursors ? const_cast<int *>(counts[a]) : nullptr;
     }
     const int nchunk = (int)((N + kChunk - 1) / kChunk);
     if (nchunk == 0) {
         LDNI_LAUNCH(K_SCAN_TOP, s, scan_empty<<<naxes, 1, 0, s>>>(ap, info, info_base));
         return cuda_status();
     }
-    if (!LDNI_SCAN_ONE_LAUNCH && nchunk <= kMaxSumChunks) {
-        LDNI_LAUNCH(K_SCAN_TOP, s, scan_sums<<<dim3(nchunk, naxes), kThreads, 0, s>>>(ap, N, nchunk, partials));
-        LDNI_LAUNCH(K_SCAN_DOWN, s,
-                    scan_prefix<<<dim3(nchunk, naxes), kThreads, 0, s>>>(ap, N, nchunk, partials, info, info_base));
-        return cuda_status();
+    switch (form) {
+        case kScanWords: return launch_scan<kScanWords>(ap, naxes, N, nchunk, partials, info, info_base, s);
+        case kScanCursors: return launch_scan<kScanCursors>(ap, naxes, N, nchunk, partials, info, info_base, s);
+        default: return launch_scan<kScanCounts>(ap, naxes, N, nchunk, partials, info, info_base, s);
     }
-    unsigned long long *words = reinterpret_cast<unsigned long long *>(partials);
-    if (int rc_ = cuda_check(cudaMemsetAsync(words, 0, sizeof(unsigned long long) * (size_t)(nchunk + 1) * naxes, s))) return rc_;
-    LDNI_LAUNCH(K_SCAN_DOWN, s,
-                scan_lookback<<<dim3(nchunk, naxes), kThreads, 0, s>>>(ap, N, nchunk, words, info, info_base,
-                                                                        wait_limit()));
-    return cuda_status();
 }
 
 }  // namespace ldni
