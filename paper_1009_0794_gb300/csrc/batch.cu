@@ -1,10 +1,14 @@
 // Many meshes, of uneven size and resolution, sampled by ONE launch per stage
 // (count, scan, fill, sort) for the whole batch - the exact two-pass form of
 // sample.cu spread over every triangle, chunk and ray of the batch at once.
-// Each thread finds its mesh by a binary search over prefix tables that a
-// setup kernel builds on the device from the caller's device array of item
+// Each block finds its mesh by a binary search over prefix tables that a setup
+// kernel builds on the device from the caller's device array of item
 // descriptors, so a batch call needs no host synchronisation and can be
-// captured in a CUDA graph.
+// captured in a CUDA graph.  A block's triangles or rays are of one mesh: its
+// descriptor's pointers are the same for all threads, and are read once (and
+// its fixed-point scale is divided out once in the setup kernel: a division in
+// FP64, at 1/64 of the FP32 rate, for every triangle and every thread of a big
+// pair was most of the big passes' time: 308 -> 75 us for the counts of 48 meshes).
 #include "lookback.cuh"
 #include "sample_common.cuh"
 
@@ -15,32 +19,38 @@ constexpr int kThreads = 256;
 
 struct Tables {
     long long *tri_prefix;    // [count + 1]
-    long long *ray_prefix;    // [3 count + 1]  rays of image (m, a) at 3 m + a
+    long long *tile_prefix;   // [count + 1]      tiles of kThreads triangles
     long long *chunk_prefix;  // [3 count + 1]  scan chunks
     long long *count_base;    // [3 count]      start of the image's counts
+    float *scale;             // [count]        fixed-point units per world unit (an FP64 division)
+    float4 *nrm;              // per-triangle normals of all items (x, y, z, packed codes)
     long long *big;           // queued big (item, triangle, image): item << 34 | tri << 2 | a
     long long qcap;
-    int *big_n;               // counts of the queue's two ends
+    int *big_n;               // counts of the queue's two ends, and of rest
+    long long *rest;          // runs of 32 rays left to batch_rest
 };
 
-__device__ __forceinline__ int find(const long long *prefix, int n, long long x) {  // prefix[k] <= x < prefix[k+1]
+// k with prefix[k] <= x < prefix[k + 1], the same x in the whole warp: a search
+// in 32 parts at a time (two dependent loads for up to a thousand entries, where
+// halving took ten in every block's first microseconds).
+__device__ __forceinline__ int find(const long long *prefix, int n, long long x) {
+    const int lane = threadIdx.x & 31;
     int lo = 0, hi = n;
     while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (prefix[mid] <= x)
-            lo = mid;
-        else
-            hi = mid;
+        const int part = (hi - lo + 31) / 32, at = lo + (lane + 1) * part;
+        const int k = __popc(__ballot_sync(0xffffffffu, at < hi && prefix[at] <= x));
+        lo += k * part;
+        hi = min(hi, lo + part);
     }
     return lo;
 }
 
-__device__ __forceinline__ GridDev grid_dev(const ldni_grid_t &g) {
+__device__ __forceinline__ GridDev grid_dev(const ldni_grid_t &g, float scale) {
     GridDev d;
     d.o[0] = g.origin[0];
     d.o[1] = g.origin[1];
     d.o[2] = g.origin[2];
-    d.s = (float)((double)g.res * (double)kSubpix / (double)g.width);  // as the host computes it
+    d.s = scale;
     d.res = g.res;
     return d;
 }
@@ -55,22 +65,23 @@ __global__ void __launch_bounds__(kThreads) setup_kernel(const ldni_batch_item_t
     __syncthreads();
     for (int m0 = 0; m0 < count; m0 += kThreads) {
         const int m = m0 + threadIdx.x;
-        long long v[4] = {0, 0, 0, 0};  // triangles, rays, chunks, count ints of one image
+        long long v[4] = {0, 0, 0, 0};  // triangles, tiles; chunks, count ints of one image
         if (m < count) {
             const long long N = (long long)items[m].grid.res * items[m].grid.res;
             v[0] = items[m].nt;
-            v[1] = N;
+            v[1] = (v[0] + kThreads - 1) / kThreads;
             v[2] = (N + kScanChunk - 1) / kScanChunk;
             v[3] = (N + 63) / 64 * 64;
         }
         long long ex[4], tot[4];
-        ex[0] = block_exclusive_scan<kThreads>(v[0], sh[0], &tot[0]);
 #pragma unroll
-        for (int q = 1; q < 4; ++q) ex[q] = block_exclusive_scan<kThreads>(3 * v[q], sh[q], &tot[q]);
+        for (int q = 0; q < 4; ++q) ex[q] = block_exclusive_scan<kThreads>(q < 2 ? v[q] : 3 * v[q], sh[q], &tot[q]);
         if (m < count) {
+            const ldni_grid_t &g = items[m].grid;
+            T.scale[m] = (float)((double)g.res * (double)kSubpix / (double)g.width);  // as the host computes it
             T.tri_prefix[m] = carry[0] + ex[0];
+            T.tile_prefix[m] = carry[1] + ex[1];
             for (int a = 0; a < 3; ++a) {
-                T.ray_prefix[3 * m + a] = carry[1] + ex[1] + a * v[1];
                 T.chunk_prefix[3 * m + a] = carry[2] + ex[2] + a * v[2];
                 T.count_base[3 * m + a] = carry[3] + ex[3] + a * v[3];
             }
@@ -81,48 +92,25 @@ __global__ void __launch_bounds__(kThreads) setup_kernel(const ldni_batch_item_t
     }
     if (threadIdx.x == 0) {
         T.tri_prefix[count] = carry[0];
-        T.ray_prefix[3 * count] = carry[1];
+        T.tile_prefix[count] = carry[1];
         T.chunk_prefix[3 * count] = carry[2];
     }
 }
 
-template <bool kFill>
-__device__ __forceinline__ void batch_emit(const ldni_batch_item_t &it, int a, long long p, float d, int t,
-                                           const float3 &n, int *cnt, ldni_info_t *info) {
-    if (!kFill) {
-        atomicAdd(cnt + p, 1);
-        return;
-    }
-    const ldni_layers_t &L = it.out[a];
-    const int k = atomicSub(cnt + p, 1) - 1;
-    const long long slot = (long long)L.offsets[p] + k;
-    if (k < 0 || slot >= L.capacity) {
-        set_status(info, LDNI_ST_CAPACITY);
-        return;
-    }
-    L.depth[slot] = d;
-    L.tri_id[slot] = t;
-    if (L.nrm8) {  // approximate normals (Section 3 item 1)
-        L.nrm8[slot] = encode_normal8(n.x, n.y, n.z);
-    } else {
-        L.nx[slot] = n.x;
-        L.ny[slot] = n.y;
-        L.nz[slot] = n.z;
-    }
-}
-
-// The fill pass over a triangle's box, two crossings at a time: both slot
-// claims and both row offsets are in flight before either sample is stored
-// (as the single-mesh fill).  mk: the box's crossings, bit x + w y.
+// The fill pass over a triangle's box, two crossings at a time: both cursors
+// are in flight before either sample is stored (as the single-mesh fill).
+// mk: the box's crossings, bit x + w y.
 template <int A>
 __device__ __forceinline__ void batch_fill_hits(const ldni_batch_item_t &it, const Setup32 &S, unsigned mk, int t,
-                                                const float3 &n, int *cnt, int res, ldni_info_t *info) {
+                                                int *cur, int res, ldni_info_t *info) {
     const ldni_layers_t &L = it.out[A];
-    const int *off = L.offsets;
+    float *D = L.depth;
+    int *Tr = L.tri_id;
     const long long cap = L.capacity;
     const int wdiv = (256 + S.w - 1) / S.w;  // y = (b * wdiv) >> 8 = b / w for b < 16, w <= 16
     while (mk) {
-        int pr[2], k[2], row[2];
+        int pr[2];
+        unsigned c[2];
         float d[2];
         bool v[2];
 #pragma unroll
@@ -131,40 +119,33 @@ __device__ __forceinline__ void batch_fill_hits(const ldni_batch_item_t &it, con
             const int b = v[u] ? __ffs(mk) - 1 : 0;
             mk &= mk - 1u;
             const int y = (b * wdiv) >> 8, x = b - y * S.w;
+            pr[u] = (S.j0 + y) * res + S.i0 + x;
+            c[u] = v[u] ? (unsigned)cur[pr[u]] : 0u;
             int e0, e1, e2;
             S.edges(S.i0 + x, S.j0 + y, e0, e1, e2);
-            pr[u] = (S.j0 + y) * res + S.i0 + x;
             d[u] = S.depth_from(e0, e1, e2);
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            k[u] = v[u] ? atomicSub(cnt + pr[u], 1) - 1 : -1;
-            row[u] = v[u] ? off[pr[u]] : 0;
+            if (!v[u]) continue;
+            c[u] = c[u] & 0x80000000u ? (c[u] & 0x7fffffffu) + (unsigned)S.exiting : (unsigned)atomicAdd(cur + pr[u], 1);
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             if (!v[u]) continue;
-            const long long slot = (long long)row[u] + k[u];
-            if (k[u] < 0 || slot >= cap) {
+            if ((long long)c[u] >= cap) {
                 set_status(info, LDNI_ST_CAPACITY);
                 continue;
             }
-            L.depth[slot] = d[u];
-            L.tri_id[slot] = t;
-            if (L.nrm8) {  // approximate normals (Section 3 item 1)
-                L.nrm8[slot] = encode_normal8(n.x, n.y, n.z);
-            } else {
-                L.nx[slot] = n.x;
-                L.ny[slot] = n.y;
-                L.nz[slot] = n.z;
-            }
+            D[c[u]] = d[u];
+            Tr[c[u]] = t;
         }
     }
 }
 
 template <bool kFill, int A>
 __device__ __forceinline__ void batch_axis(const ldni_batch_item_t &it, int m, const TriView &Tv, int t,
-                                           const float3 &n, int res, int *counts, const Tables &T, ldni_info_t *info) {
+                                           int res, int *counts, const Tables &T, ldni_info_t *info) {
     Setup32 S;
     const int kind = setup_axis<A, kFill>(Tv, res, S);
     if (kind == kNone) return;
@@ -175,151 +156,218 @@ __device__ __forceinline__ void batch_axis(const ldni_batch_item_t &it, int m, c
     }
     int *cnt = counts + T.count_base[3 * m + A];
     if (!kFill) {
-        S.for_each_hit([&](int i, int j, int, int, int) { atomicAdd(cnt + (long long)j * res + i, 1); });
+        const int word = count_word(S.exiting);
+        S.for_each_hit([&](int i, int j, int, int, int) { atomicAdd(cnt + (long long)j * res + i, word); });
         return;
     }
-    batch_fill_hits<A>(it, S, S.hit_bits(), t, n, cnt, res, info);
+    batch_fill_hits<A>(it, S, S.hit_bits(), t, cnt, res, info);
 }
 
 template <bool kFill>
 __global__ void __launch_bounds__(kThreads) batch_tri_pass(const ldni_batch_item_t *items, int count, Tables T,
                                                            int *counts, ldni_info_t *infos) {
-    const long long total = T.tri_prefix[count];
-    for (long long gt = blockIdx.x * (long long)blockDim.x + threadIdx.x; gt < total;
-         gt += (long long)gridDim.x * blockDim.x) {
-        const int m = find(T.tri_prefix, count, gt);
-        const ldni_batch_item_t &it = items[m];
-        const int t = (int)(gt - T.tri_prefix[m]);
-        const GridDev g = grid_dev(it.grid);
-        TriView Tv;
-        const unsigned bad = load_tri(it.verts, it.tris, t, (int)it.nv, g, Tv);
-        if (bad) {
-            if (!kFill) set_status(infos + m, bad);
-            continue;
-        }
-        float3 n = make_float3(0.f, 0.f, 0.f);
-        if (kFill) face_normal(Tv.p[0], Tv.p[1], Tv.p[2], n.x, n.y, n.z);
-        batch_axis<kFill, 0>(it, m, Tv, t, n, g.res, counts, T, infos + m);
-        batch_axis<kFill, 1>(it, m, Tv, t, n, g.res, counts, T, infos + m);
-        batch_axis<kFill, 2>(it, m, Tv, t, n, g.res, counts, T, infos + m);
+    const long long tile = blockIdx.x;
+    const int m = find(T.tile_prefix, count, tile);
+    const ldni_batch_item_t &it = items[m];
+    const long long t0 = (tile - T.tile_prefix[m]) * kThreads + threadIdx.x;
+    if (t0 >= it.nt) return;
+    const int t = (int)t0;
+    const GridDev g = grid_dev(it.grid, T.scale[m]);
+    TriView Tv;
+    const unsigned bad = load_tri(it.verts, it.tris, t, (int)it.nv, g, Tv);
+    if (bad) {
+        if (!kFill) set_status(infos + m, bad);
+        return;
     }
+    if (kFill) {
+        float3 n;
+        face_normal(Tv.p[0], Tv.p[1], Tv.p[2], n.x, n.y, n.z);
+        T.nrm[T.tri_prefix[m] + t] = make_float4(n.x, n.y, n.z, __uint_as_float(encode_normal8(n.x, n.y, n.z)));
+    }
+    batch_axis<kFill, 0>(it, m, Tv, t, g.res, counts, T, infos + m);
+    batch_axis<kFill, 1>(it, m, Tv, t, g.res, counts, T, infos + m);
+    batch_axis<kFill, 2>(it, m, Tv, t, g.res, counts, T, infos + m);
 }
 
 template <bool kFill>
-__global__ void __launch_bounds__(kThreads) batch_big(const ldni_batch_item_t *items, Tables T, int *counts,
+__global__ void __launch_bounds__(kThreads, 4) batch_big(const ldni_batch_item_t *items, Tables T, int *counts,
                                                       int huge_blocks, ldni_info_t *infos) {
     for_each_big(T.big, T.qcap, T.big_n, (int)blockIdx.x, (int)gridDim.x, huge_blocks,
                  [&](long long code, int first, int step) {
         const int m = (int)(code >> 34), t = (int)((code >> 2) & 0xFFFFFFFF), a = (int)(code & 3);
         const ldni_batch_item_t &it = items[m];
-        const GridDev g = grid_dev(it.grid);
+        const GridDev g = grid_dev(it.grid, T.scale[m]);
         TriView Tv;
         if (load_tri(it.verts, it.tris, t, (int)it.nv, g, Tv)) return;
         Setup64 S;
         int i0, i1, j0, j1;
         if (!setup_big(Tv, a, g.res, S, i0, i1, j0, j1)) return;
-        float3 n = make_float3(0.f, 0.f, 0.f);
-        if (kFill) face_normal(Tv.p[0], Tv.p[1], Tv.p[2], n.x, n.y, n.z);
         int *cnt = counts + T.count_base[3 * m + a];
-        const int w = i1 - i0 + 1;
-        const long long npx = (long long)w * (j1 - j0 + 1);
-        for (long long k = first; k < npx; k += step) {
-            const int j = j0 + (int)(k / w), i = i0 + (int)(k % w);
-            if (S.inside(i, j))
-                batch_emit<kFill>(it, a, (long long)j * g.res + i, kFill ? S.depth(i, j) : 0.0f, t, n, cnt, infos + m);
+        if (!kFill) {
+            const int word = count_word(S.exiting);
+            sweep_box<1>(S, i0, i1, j0, j1, first, step, [&](auto &, auto &i, auto &j, auto) {
+                atomicAdd(cnt + (long long)j[0] * g.res + i[0], word);
+            });
+            return;
         }
+        const ldni_layers_t &L = it.out[a];
+        float *D = L.depth;
+        int *Tr = L.tri_id;
+        const long long cap = L.capacity;
+        sweep_box<kFillBatch>(S, i0, i1, j0, j1, first, step, [&](auto &v, auto &i, auto &j, auto depth) {
+            fill_batch(v, i, j, g.res, S.exiting, t, cnt, D, Tr, cap, infos + m, depth);
+        });
     });
 }
 
-// Scan of every image's counts: chunks of all images in one launch; the
-// look-back of a chunk stops at the first chunk of its own image.
+// Scan of every image's count words: chunks of all images in one launch; the
+// look-back of a chunk stops at the first chunk of its own image.  Offsets go
+// to the image, cursors over the words.  A thread's 16 words come as four
+// 16-byte loads of whole lines per warp each: 45 us for the 12.5 M rays of 48
+// meshes, 89 us with sixteen 4-byte loads 64 bytes apart.
 __global__ void __launch_bounds__(kThreads) batch_scan(const ldni_batch_item_t *items, int count, Tables T,
-                                                       const int *counts, unsigned long long *words,
-                                                       ldni_info_t *infos, int spin_limit) {
-    __shared__ long long sh[kThreads / 32 + 1];
+                                                       int *counts, unsigned long long *words, ldni_info_t *infos,
+                                                       int spin_limit) {
+    constexpr int kSlices = kScanChunk / (4 * kThreads), kWarps = kThreads / 32;
+    __shared__ long long tot[kSlices][kWarps];  // samples of each warp's words, per slice
     __shared__ long long s_chunk, s_base;
     const long long nchunks = T.chunk_prefix[3 * count];
     if (threadIdx.x == 0) s_chunk = (long long)atomicAdd(words + nchunks, 1ull);
     __syncthreads();
     const long long c = s_chunk;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int img = find(T.chunk_prefix, 3 * count, c);
     const int m = img / 3, a = img % 3;
     const long long local = c - T.chunk_prefix[img];
     const long long N = (long long)items[m].grid.res * items[m].grid.res;
-    const int *cnt = counts + T.count_base[img];
+    int *cnt = counts + T.count_base[img];  // 256-byte aligned, padded to 64 words (zeros)
     int *out = items[m].out[a].offsets;
     const long long base = local * kScanChunk;
-    constexpr int kPer = kScanChunk / kThreads;  // 16 counts per thread
-    int v[kPer];
-    long long mine = 0;
+    int4 v[kSlices];
+    long long xin[kSlices];  // samples before the thread's words within its warp
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        const long long e = base + (long long)threadIdx.x * kPer + k;
-        v[k] = e < N ? cnt[e] : 0;
-        mine += v[k];
+    for (int s = 0; s < kSlices; ++s) {
+        const long long e = base + s * 4 * kThreads + threadIdx.x * 4;
+        v[s] = e < N ? *reinterpret_cast<const int4 *>(cnt + e) : make_int4(0, 0, 0, 0);
     }
-    long long total;
-    const long long excl = block_exclusive_scan<kThreads>(mine, sh, &total);
+    long long wtot[kSlices];
+#pragma unroll
+    for (int s = 0; s < kSlices; ++s) {
+        const long long mine = (long long)count_of(v[s].x) + count_of(v[s].y) + count_of(v[s].z) + count_of(v[s].w);
+        long long x = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        xin[s] = x - mine;
+        wtot[s] = x;
+    }
+    if (lane == 31)
+#pragma unroll
+        for (int s = 0; s < kSlices; ++s) tot[s][warp] = wtot[s];
+    __syncthreads();
+    long long carry = 0;
+#pragma unroll
+    for (int s = 0; s < kSlices; ++s) {
+        long long lead = 0, all = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            const long long t = tot[s][w];
+            all += t;
+            if (w < warp) lead += t;
+        }
+        xin[s] += carry + lead;
+        carry += all;
+    }
     if (threadIdx.x < 32) {
         // image-local status words: chunk 0 of the image starts at prefix 0
-        const long long b = lookback_warp(words + T.chunk_prefix[img], (int)local, total, infos + m, spin_limit);
+        const long long b = lookback_warp(words + T.chunk_prefix[img], (int)local, carry, infos + m, spin_limit);
         if (threadIdx.x == 0) s_base = b;
     }
     __syncthreads();
-    long long run = s_base + excl;
+    const bool vec = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        const long long e = base + (long long)threadIdx.x * kPer + k;
-        if (e < N) out[e] = (int)min(run, (long long)INT_MAX);
-        run += v[k];
+    for (int s = 0; s < kSlices; ++s) {
+        const long long e = base + s * 4 * kThreads + threadIdx.x * 4;
+        if (e >= N) continue;
+        const long long o0 = s_base + xin[s], o1 = o0 + count_of(v[s].x), o2 = o1 + count_of(v[s].y),
+                        o3 = o2 + count_of(v[s].z);
+        const auto clamp = [](long long x) { return (int)min(x, (long long)INT_MAX); };
+        const int4 w = make_int4(clamp(o0), clamp(o1), clamp(o2), clamp(o3));
+        *reinterpret_cast<int4 *>(cnt + e) = make_int4(make_cursor(w.x, v[s].x), make_cursor(w.y, v[s].y),
+                                                       make_cursor(w.z, v[s].z), make_cursor(w.w, v[s].w));
+        if (vec && e + 3 < N) {
+            *reinterpret_cast<int4 *>(out + e) = w;
+        } else {
+            out[e] = w.x;
+            if (e + 1 < N) out[e + 1] = w.y;
+            if (e + 2 < N) out[e + 2] = w.z;
+            if (e + 3 < N) out[e + 3] = w.w;
+        }
     }
     if (local == T.chunk_prefix[img + 1] - T.chunk_prefix[img] - 1 && threadIdx.x == 0) {
-        const long long n_img = s_base + total;
+        const long long n_img = s_base + carry;
         out[N] = (int)min(n_img, (long long)INT_MAX);
         infos[m].n[a] = n_img;
         if (n_img > INT_MAX) set_status(infos + m, LDNI_ST_TOOLARGE);
     }
 }
 
-// Ordering of every ray of the batch as in the single-mesh sampling: a warp
-// takes 32 consecutive rays of the batch; its first lane finds the image of
-// the first ray, and the others step forward from there.
+// Ordering of every ray of the batch, and its samples' normals, as in the
+// single-mesh sampling: kSortParts blocks per chunk, and the runs of 32 rays
+// with others than two samples listed (image << 32 | run) for batch_rest.
+constexpr int kSortParts = 4, kSortRays = kScanChunk / kSortParts;
+
+struct ItemImage {
+    const int *off;
+    RayOut r;
+    NormalTable nrm;
+    long long cap, N;
+    bool pairs8;
+};
+__device__ __forceinline__ ItemImage item_image(const ldni_batch_item_t *items, const Tables &T, int img) {
+    const int m = img / 3, a = img % 3;
+    const ldni_layers_t &L = items[m].out[a];
+    ItemImage I;
+    I.off = L.offsets;
+    I.r = L.nrm8 ? RayOut{L.depth, L.tri_id, reinterpret_cast<float *>(L.nrm8), nullptr, nullptr}
+                 : RayOut{L.depth, L.tri_id, L.nx, L.ny, L.nz};
+    I.nrm = NormalTable{T.nrm + T.tri_prefix[m], (int)items[m].nt};
+    I.cap = L.capacity;
+    I.N = (long long)items[m].grid.res * items[m].grid.res;
+    I.pairs8 = ((reinterpret_cast<uintptr_t>(I.r.D) | reinterpret_cast<uintptr_t>(I.r.Tr) |
+                 reinterpret_cast<uintptr_t>(I.r.X) | reinterpret_cast<uintptr_t>(I.r.Y) |
+                 reinterpret_cast<uintptr_t>(I.r.Z)) & 7) == 0;
+    return I;
+}
+
 __global__ void __launch_bounds__(kThreads) batch_sort(const ldni_batch_item_t *items, int count, Tables T,
                                                        ldni_info_t *infos) {
-    __shared__ SortStage stage[kThreads / 32];
-    const long long total = T.ray_prefix[3 * count];
     const int lane = threadIdx.x & 31;
-    SortStage &st = stage[threadIdx.x >> 5];
-    const auto in_place = [](long long, long long b, const RayOut &o) { return InPlace{o, b}; };
-    for (long long wb = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); wb < total;
-         wb += (long long)gridDim.x * blockDim.x) {
-        int img = lane == 0 ? find(T.ray_prefix, 3 * count, wb) : 0;
-        img = __shfl_sync(0xffffffffu, img, 0);
-        const long long gr = wb + lane;
-        const bool act = gr < total;
-        if (act)
-            while (gr >= T.ray_prefix[img + 1]) ++img;
-        const int m = img / 3, a = img % 3;
-        RayOut r{};
-        long long b = 0;
-        int n = 0;
-        if (act) {
-            const ldni_layers_t &L = items[m].out[a];
-            r = L.nrm8 ? RayOut{L.depth, L.tri_id, reinterpret_cast<float *>(L.nrm8), nullptr, nullptr}
-                       : RayOut{L.depth, L.tri_id, L.nx, L.ny, L.nz};
-            const long long p = gr - T.ray_prefix[img];
-            b = L.offsets[p];
-            long long e = L.offsets[p + 1];
-            if ((e - b) & 1) {
-                atomicAdd(&infos[m].odd_rays, 1u);
-                set_status(infos + m, LDNI_ST_ODD);
-            }
-            if (e > L.capacity) e = L.capacity;
-            if (e - b >= 2) n = (int)(e - b);
-        }
-        // the rays of a warp may belong to two or more images: each is
-        // ordered with the arrays of its own lane
-        order_warp_rays<false>(b, n, b, in_place, r, st, lane);
+    const long long c = blockIdx.x / kSortParts;
+    const int img = find(T.chunk_prefix, 3 * count, c);
+    const ItemImage I = item_image(items, T, img);
+    const long long p0 = (c - T.chunk_prefix[img]) * kScanChunk + (blockIdx.x % kSortParts) * kSortRays;
+    for (int q = threadIdx.x & ~31; q < kSortRays && p0 + q < I.N; q += kThreads) {
+        long long b;
+        const int n = ray_samples(I.off, p0 + q, I.N, I.cap, lane, true, infos + img / 3, b);
+        if (__any_sync(0xffffffffu, n != 0 && n != 2) && lane == 0)
+            T.rest[atomicAdd(T.big_n + 2, 1)] = ((long long)img << 32) | ((p0 + q) >> 5);
+        if (n == 2) finish_pair(b, I.r, I.nrm, I.pairs8);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) batch_rest(const ldni_batch_item_t *items, Tables T, ldni_info_t *infos) {
+    __shared__ SortStage stage[kThreads / 32];
+    const int lane = threadIdx.x & 31, warps = gridDim.x * (kThreads / 32);
+    for (int q = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); q < T.big_n[2]; q += warps) {
+        const long long code = T.rest[q];
+        const int img = (int)(code >> 32);
+        const ItemImage I = item_image(items, T, img);
+        long long b;
+        const int n = ray_samples(I.off, (code & 0xffffffffll) << 5, I.N, I.cap, lane, false, infos + img / 3, b);
+        finish_rest(b, n == 2 ? 0 : n, I.r, I.nrm, stage[threadIdx.x >> 5], lane);
     }
 }
 
@@ -346,9 +394,12 @@ BatchWs carve_batch(Carver &c, const ldni_batch_item_t *items_host, int count) {
     w.words = c.take<unsigned long long>((size_t)chunks + 1);
     w.words_bytes = sizeof(unsigned long long) * ((size_t)chunks + 1);
     w.T.tri_prefix = c.take<long long>((size_t)count + 1);
-    w.T.ray_prefix = c.take<long long>(3 * (size_t)count + 1);
+    w.T.tile_prefix = c.take<long long>((size_t)count + 1);
     w.T.chunk_prefix = c.take<long long>(3 * (size_t)count + 1);
     w.T.count_base = c.take<long long>(3 * (size_t)count);
+    w.T.scale = c.take<float>((size_t)count);
+    w.T.nrm = c.take<float4>((size_t)(tris > 0 ? tris : 1));
+    w.T.rest = c.take<long long>((size_t)chunks * (kScanChunk / 32));
     w.T.qcap = 3 * tris > 0 ? 3 * tris : 1;
     w.T.big = c.take<long long>((size_t)w.T.qcap);
     return w;
@@ -367,12 +418,6 @@ bool items_ok(const ldni_batch_item_t *items, int count) {
         }
     }
     return count < (1 << 29);
-}
-
-int blocks_for(long long work) {
-    long long b = (work + kThreads - 1) / kThreads;
-    const long long lim = (long long)num_sms() * 16;
-    return (int)(b < 1 ? 1 : (b > lim ? lim : b));
 }
 
 }  // namespace
@@ -394,11 +439,11 @@ extern "C" int ldni_sample_batch(const ldni_batch_item_t *items_dev, const ldni_
     Carver c(ws, ws_bytes);
     BatchWs w = carve_batch(c, items_host, count);
     if (!c.fits()) return LDNI_EWORKSPACE;
-    long long tris = 0, rays = 0, chunks = 0;
+    long long tris = 0, tiles = 0, chunks = 0;
     for (int m = 0; m < count; ++m) {
         const long long N = (long long)items_host[m].grid.res * items_host[m].grid.res;
         tris += items_host[m].nt;
-        rays += 3 * N;
+        tiles += (items_host[m].nt + kThreads - 1) / kThreads;
         chunks += 3 * ((N + kScanChunk - 1) / kScanChunk);
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -407,7 +452,7 @@ extern "C" int ldni_sample_batch(const ldni_batch_item_t *items_dev, const ldni_
     if (int rc_ = cuda_check(cudaMemsetAsync(infos, 0, sizeof(ldni_info_t) * (size_t)count, s))) return rc_;
     LDNI_LAUNCH(K_BATCH, s, setup_kernel<<<1, kThreads, 0, s>>>(items_dev, count, w.T));
     if (tris > 0) {
-        LDNI_LAUNCH(K_BATCH, s, batch_tri_pass<false><<<blocks_for(tris), kThreads, 0, s>>>(items_dev, count, w.T,
+        LDNI_LAUNCH(K_BATCH, s, batch_tri_pass<false><<<(unsigned)tiles, kThreads, 0, s>>>(items_dev, count, w.T,
                                                                                              w.counts, infos));
         LDNI_LAUNCH(K_BATCH, s,
                     batch_big<false><<<5 * num_sms(), kThreads, 0, s>>>(items_dev, w.T, w.counts, num_sms(), infos));
@@ -416,11 +461,13 @@ extern "C" int ldni_sample_batch(const ldni_batch_item_t *items_dev, const ldni_
                 batch_scan<<<(unsigned)chunks, kThreads, 0, s>>>(items_dev, count, w.T, w.counts, w.words, infos,
                                                                   wait_limit()));
     if (tris > 0) {
-        LDNI_LAUNCH(K_BATCH, s, batch_tri_pass<true><<<blocks_for(tris), kThreads, 0, s>>>(items_dev, count, w.T,
+        LDNI_LAUNCH(K_BATCH, s, batch_tri_pass<true><<<(unsigned)tiles, kThreads, 0, s>>>(items_dev, count, w.T,
                                                                                             w.counts, infos));
         LDNI_LAUNCH(K_BATCH, s,
                     batch_big<true><<<5 * num_sms(), kThreads, 0, s>>>(items_dev, w.T, w.counts, num_sms(), infos));
     }
-    LDNI_LAUNCH(K_BATCH, s, batch_sort<<<blocks_for(rays), kThreads, 0, s>>>(items_dev, count, w.T, infos));
+    LDNI_LAUNCH(K_BATCH, s,
+                batch_sort<<<(unsigned)(chunks * kSortParts), kThreads, 0, s>>>(items_dev, count, w.T, infos));
+    LDNI_LAUNCH(K_BATCH, s, batch_rest<<<2 * num_sms(), kThreads, 0, s>>>(items_dev, w.T, infos));
     return cuda_status();
 }

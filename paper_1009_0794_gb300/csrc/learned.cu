@@ -432,12 +432,9 @@ __global__ void __launch_bounds__(kThreads) onepass_big(const float *__restrict_
         if (!setup_big(T, a, g.res, S, i0, i1, j0, j1)) return;
         float3 n;
         face_normal(T.p[0], T.p[1], T.p[2], n.x, n.y, n.z);
-        const int w = i1 - i0 + 1;
-        const long long npx = (long long)w * (j1 - j0 + 1);
-        for (long long k = first; k < npx; k += step) {
-            const int j = j0 + (int)(k / w), i = i0 + (int)(k % w);
-            if (S.inside(i, j)) onepass_hit(a, (long long)j * g.res + i, S.depth(i, j), t, n, S.exiting, o);
-        }
+        sweep_box<1>(S, i0, i1, j0, j1, first, step, [&](auto &, auto &i, auto &j, auto depth) {
+            onepass_hit(a, (long long)j[0] * g.res + i[0], depth(0), t, n, S.exiting, o);
+        });
     });
 }
 
@@ -502,12 +499,9 @@ __device__ __forceinline__ void redo_big_block(const float *__restrict__ verts, 
         if (!setup_big(T, a, g.res, S, i0, i1, j0, j1)) return;
         float3 n;
         face_normal(T.p[0], T.p[1], T.p[2], n.x, n.y, n.z);
-        const int w = i1 - i0 + 1;
-        const long long npx = (long long)w * (j1 - j0 + 1);
-        for (long long k = first; k < npx; k += step) {
-            const int j = j0 + (int)(k / w), i = i0 + (int)(k % w);
-            if (S.inside(i, j)) redo_hit(a, (long long)j * g.res + i, S.depth(i, j), t, o, n, info);
-        }
+        sweep_box<1>(S, i0, i1, j0, j1, first, step, [&](auto &, auto &i, auto &j, auto depth) {
+            redo_hit(a, (long long)j[0] * g.res + i[0], depth(0), t, o, n, info);
+        });
     });
 }
 
@@ -734,9 +728,9 @@ __global__ void __launch_bounds__(kThreads) order_deep(long long nrays, int ax_l
                         n = 0;
                 }
                 if (t_over)  // the same in every lane: a chunk lies in one tile
-                    order_warp_rays<true>(b, n, b, in_place, r, st, lane);
+                    order_warp_rays(b, n, b, in_place, r, st, lane);
                 else
-                    order_warp_rays<true>(b, n, sb[tile] + (p & (kTilePix - 1)) * kt, from_slab, r, st, lane);
+                    order_warp_rays(b, n, sb[tile] + (p & (kTilePix - 1)) * kt, from_slab, r, st, lane);
             }
         }
     }

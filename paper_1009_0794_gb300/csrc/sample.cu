@@ -22,11 +22,13 @@
 // few as the CSR form allows: for the 1.31 M-triangle sphere at 2048^2 146 us with
 // 20 M stores and 10 M cursor loads, 454 us with 51 M stores, 10 M returned
 // atomics and 10 M offset loads.  The normals, three fifths of a sample, are
-// stored by the sort pass, ray after ray (94 us, 102 without them but with the
-// pairs' swaps).
+// stored by the sort passes, ray after ray (79 us; 102 us when it had only the
+// swaps to do).
 //
 // Triangles whose pixel box is large are handed to a block-per-triangle
 // kernel with 64-bit edge functions.
+#include <algorithm>
+
 #include "sample_common.cuh"
 
 namespace ldni {
@@ -49,23 +51,6 @@ struct Img {
 };
 
 __device__ __forceinline__ int *sel(int *const (&arr)[3], int a) { return a == 0 ? arr[0] : (a == 1 ? arr[1] : arr[2]); }
-
-// One crossing at depth d: count it, or take a slot of ray p and store the sample.
-template <bool kFill>
-__device__ __forceinline__ void emit(float d, int a, int t, long long p, int exiting, const Img &o, ldni_info_t *info) {
-    int *cnt = sel(o.count, a);
-    if (!kFill) {
-        atomicAdd(cnt + p, count_word(exiting));
-        return;
-    }
-    const long long slot = claim_slot(cnt, p, exiting);
-    if (slot >= (a == 0 ? o.cap[0] : (a == 1 ? o.cap[1] : o.cap[2]))) {
-        set_status(info, LDNI_ST_CAPACITY);
-        return;
-    }
-    (a == 0 ? o.depth[0] : (a == 1 ? o.depth[1] : o.depth[2]))[slot] = d;
-    (a == 0 ? o.tri[0] : (a == 1 ? o.tri[1] : o.tri[2]))[slot] = t;
-}
 
 // The fill pass over a triangle's box, two crossings at a time: both cursors
 // are in flight before either sample is stored.  m: the box's crossings, bit
@@ -157,8 +142,8 @@ __global__ void __launch_bounds__(kThreads) tri_pass(const float *__restrict__ v
     }
 }
 
-// The queued big (triangle, image) pairs, a warp or a block per pair
-// (for_each_big); the pair's threads stride over its box pixels.
+// The queued big (triangle, image) pairs (for_each_big), each swept by its
+// threads.
 template <bool kFill>
 __global__ void __launch_bounds__(kThreads) big_pass(const float *__restrict__ verts, const int *__restrict__ tris,
                                                      int nv, GridDev g, Img o, const int *big_q, long long qcap,
@@ -170,49 +155,68 @@ __global__ void __launch_bounds__(kThreads) big_pass(const float *__restrict__ v
         Setup64 S;
         int i0, i1, j0, j1;
         if (!setup_big(T, a, g.res, S, i0, i1, j0, j1)) return;
-        const int w = i1 - i0 + 1;
-        const long long npx = (long long)w * (j1 - j0 + 1);
-        for (long long k = first; k < npx; k += step) {
-            const int j = j0 + (int)(k / w), i = i0 + (int)(k % w);
-            if (S.inside(i, j)) emit<kFill>(kFill ? S.depth(i, j) : 0.0f, a, t, (long long)j * g.res + i, S.exiting, o, info);
+        int *cnt = sel(o.count, a);
+        if (!kFill) {
+            const int word = count_word(S.exiting);
+            sweep_box<1>(S, i0, i1, j0, j1, first, step, [&](auto &, auto &i, auto &j, auto) {
+                atomicAdd(cnt + (long long)j[0] * g.res + i[0], word);
+            });
+            return;
         }
+        float *D = a == 0 ? o.depth[0] : (a == 1 ? o.depth[1] : o.depth[2]);
+        int *Tr = a == 0 ? o.tri[0] : (a == 1 ? o.tri[1] : o.tri[2]);
+        const long long cap = a == 0 ? o.cap[0] : (a == 1 ? o.cap[1] : o.cap[2]);
+        sweep_box<kFillBatch>(S, i0, i1, j0, j1, first, step, [&](auto &v, auto &i, auto &j, auto depth) {
+            fill_batch(v, i, j, g.res, S.exiting, t, cnt, D, Tr, cap, info, depth);
+        });
     });
 }
 
-// Per-ray ordering by (depth, tri_id) in place, and the samples' normals; also
-// flags odd rays.  A warp takes 32 consecutive rays: two samples are ordered
-// by their lane directly, longer rays by the rank orderings.
-__global__ void __launch_bounds__(kThreads) sort_rays(long long nrays, int ax_lo, Img o, ldni_info_t *info) {
-    __shared__ SortStage stage[kThreads / 32];
-    const int a = ax_lo + blockIdx.y;
-    const int *off = a == 0 ? o.offsets[0] : (a == 1 ? o.offsets[1] : o.offsets[2]);
+struct Image {  // one image's arrays
+    const int *off;
     RayOut r;
-    r.D = a == 0 ? o.depth[0] : (a == 1 ? o.depth[1] : o.depth[2]);
-    r.Tr = a == 0 ? o.tri[0] : (a == 1 ? o.tri[1] : o.tri[2]);
-    r.X = a == 0 ? o.nx[0] : (a == 1 ? o.nx[1] : o.nx[2]);
-    r.Y = a == 0 ? o.ny[0] : (a == 1 ? o.ny[1] : o.ny[2]);
-    r.Z = a == 0 ? o.nz[0] : (a == 1 ? o.nz[1] : o.nz[2]);
-    const long long cap = a == 0 ? o.cap[0] : (a == 1 ? o.cap[1] : o.cap[2]);
+    long long cap;
+};
+__device__ __forceinline__ Image image_of(const Img &o, int a) {
+    Image m;
+    m.off = a == 0 ? o.offsets[0] : (a == 1 ? o.offsets[1] : o.offsets[2]);
+    m.r.D = a == 0 ? o.depth[0] : (a == 1 ? o.depth[1] : o.depth[2]);
+    m.r.Tr = a == 0 ? o.tri[0] : (a == 1 ? o.tri[1] : o.tri[2]);
+    m.r.X = a == 0 ? o.nx[0] : (a == 1 ? o.nx[1] : o.nx[2]);
+    m.r.Y = a == 0 ? o.ny[0] : (a == 1 ? o.ny[1] : o.ny[2]);
+    m.r.Z = a == 0 ? o.nz[0] : (a == 1 ? o.nz[1] : o.nz[2]);
+    m.cap = a == 0 ? o.cap[0] : (a == 1 ? o.cap[1] : o.cap[2]);
+    return m;
+}
+
+// Per-ray ordering by (depth, tri_id) in place, and the samples' normals; also
+// flags odd rays.  A warp takes 32 consecutive rays; the runs with rays of
+// other than two samples are listed (image << 28 | run) for sort_rest.
+__global__ void __launch_bounds__(kThreads, 8) sort_rays(long long nrays, int ax_lo, Img o, int *rest, int *rest_n,
+                                                         ldni_info_t *info) {
+    const int a = ax_lo + blockIdx.y;
+    const Image m = image_of(o, a);
     const NormalTable nrm{o.nrm, o.nt};
     const int lane = threadIdx.x & 31;
-    SortStage &st = stage[threadIdx.x >> 5];
     for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); base < nrays;
          base += (long long)gridDim.x * blockDim.x) {
-        const long long p = base + lane;
-        long long b = p < nrays ? off[p] : 0;
-        long long e = __shfl_down_sync(0xffffffffu, b, 1);
-        int n = 0;
-        if (p < nrays) {
-            if (lane == 31 || p + 1 == nrays) e = off[p + 1];
-            if ((e - b) & 1) {
-                atomicAdd(&info->odd_rays, 1u);
-                set_status(info, LDNI_ST_ODD);
-            }
-            if (e > cap) e = cap;
-            if (!range_ok(b, max(b, e), cap, info)) e = b;
-            n = (int)max(e - b, 0ll);
-        }
-        finish_warp_rays<true>(b, n, r, nrm, o.pairs8, st, lane);
+        long long b;
+        const int n = ray_samples(m.off, base, nrays, m.cap, lane, true, info, b);
+        if (__any_sync(0xffffffffu, n != 0 && n != 2) && lane == 0) rest[atomicAdd(rest_n, 1)] = (a << 28) | (int)(base >> 5);
+        if (n == 2) finish_pair(b, m.r, nrm, o.pairs8);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) sort_rest(long long nrays, Img o, const int *rest, const int *rest_n,
+                                                      ldni_info_t *info) {
+    __shared__ SortStage stage[kThreads / 32];
+    const int lane = threadIdx.x & 31, warps = gridDim.x * (kThreads / 32);
+    for (int q = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); q < *rest_n; q += warps) {
+        const int code = rest[q];
+        const Image m = image_of(o, code >> 28);
+        long long b;
+        const int n = ray_samples(m.off, (long long)(code & 0xfffffff) << 5, nrays, m.cap, lane, false, info, b);
+        finish_rest(b, n == 2 ? 0 : n, m.r, NormalTable{o.nrm, o.nt}, stage[threadIdx.x >> 5], lane);
     }
 }
 
@@ -399,7 +403,8 @@ __global__ void __launch_bounds__(kThreads) tile_pass(const float *__restrict__ 
 
 struct SampleWs {
     int *count[3];
-    int *big_n;          // two queue counts right after the counts: one memset clears all
+    int *big_n;          // two queue counts and rest's right after the counts: one memset clears all
+    int *rest;           // runs of 32 rays left to sort_rest
     long long qcap;
     size_t clear_bytes;
     long long *scan_words;
@@ -411,10 +416,11 @@ SampleWs carve_sample_ws(Carver &c, long long nt, int res, int naxes) {
     SampleWs w{};
     const long long N = (long long)res * res;
     const long long stride = (N + 63) / 64 * 64;  // every image's counts start 256-byte aligned
-    int *block = c.take<int>((size_t)(stride * naxes + 2));
+    int *block = c.take<int>((size_t)(stride * naxes + 3));
     for (int a = 0; a < naxes; ++a) w.count[a] = block ? block + (size_t)a * stride : nullptr;
     w.big_n = block ? block + (size_t)stride * naxes : nullptr;
-    w.clear_bytes = sizeof(int) * (size_t)(stride * naxes + 2);
+    w.clear_bytes = sizeof(int) * (size_t)(stride * naxes + 3);
+    w.rest = c.take<int>((size_t)((N + 31) / 32 * naxes));
     w.scan_words = c.take<long long>(csr_scan_partials(N) * naxes);
     w.qcap = nt * naxes > 0 ? nt * naxes : 1;
     w.big_q = c.take<int>((size_t)w.qcap);
@@ -509,6 +515,17 @@ int run_count(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, c
     return csr_scan(cnt, off, C.naxes, C.nrays, C.w.scan_words, info, C.ax_lo, C.s, nullptr, nullptr, kScanCursors);
 }
 
+void run_sort(const Call &C, ldni_info_t *info) {
+    int *rest_n = C.w.big_n + 2;
+    LDNI_LAUNCH(K_SORT, C.s,
+                sort_rays<<<dim3(grid_blocks(C.nrays), C.naxes), kThreads, 0, C.s>>>(C.nrays, C.ax_lo, C.o, C.w.rest,
+                                                                                    rest_n, info));
+    const long long runs = (C.nrays + 31) / 32 * C.naxes, blocks = (runs + kThreads / 32 - 1) / (kThreads / 32);
+    LDNI_LAUNCH(K_SORT, C.s,
+                sort_rest<<<(unsigned)std::min(blocks, 3ll * num_sms()), kThreads, 0, C.s>>>(C.nrays, C.o, C.w.rest,
+                                                                                           rest_n, info));
+}
+
 int run_fill(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, const Call &C, ldni_info_t *info) {
     if (nt > 0) {
         LDNI_LAUNCH(K_FILL_TRI, C.s,
@@ -519,8 +536,7 @@ int run_fill(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, co
                     big_pass<true><<<5 * num_sms(), kThreads, 0, C.s>>>(verts, tris, (int)nv, C.g, C.o, C.w.big_q,
                                                                        C.w.qcap, C.w.big_n, num_sms(), info));
     }
-    LDNI_LAUNCH(K_SORT, C.s,
-                sort_rays<<<dim3(grid_blocks(C.nrays), C.naxes), kThreads, 0, C.s>>>(C.nrays, C.ax_lo, C.o, info));
+    run_sort(C, info);
     return cuda_status();
 }
 
@@ -622,8 +638,7 @@ int run_binned_fill(const float *verts, int64_t nv, const int32_t *tris, int64_t
         LDNI_LAUNCH(K_FILL_BIG, C.s,
                     big_pass<true><<<5 * num_sms(), kThreads, 0, C.s>>>(verts, tris, (int)nv, C.g, C.o, C.w.big_q,
                                                                        C.w.qcap, C.w.big_n, num_sms(), info));
-    LDNI_LAUNCH(K_SORT, C.s,
-                sort_rays<<<dim3(grid_blocks(C.nrays), C.naxes), kThreads, 0, C.s>>>(C.nrays, C.ax_lo, C.o, info));
+    run_sort(C, info);
     return cuda_status();
 }
 

@@ -15,7 +15,8 @@ constexpr int kTileBits = 12;
 constexpr int kTilePix = 1 << kTileBits;  // rays per tile (= one scan chunk)
 static_assert(kTilePix == kScanChunk, "a tile is one scan chunk");
 constexpr int kBigPixels = 16;            // pixel-centre box of a thread-handled triangle (fits one mask)
-constexpr int kHugePixels = 2048;         // boxes above this take a whole block, smaller big ones a warp
+constexpr int kHugePixels = 2048;         // boxes above this take whole blocks, smaller big ones a few threads
+constexpr int kPairThreads = 4;             // at least so many
 // Largest snapped extent (fixed-point units) of a triangle handled with
 // 32-bit edge functions.  With every vertex and every visited pixel centre
 // (plus one step beyond the box) within 32768 units of each other, each edge
@@ -116,10 +117,22 @@ struct Setup64 {
         edges(i, j, e0, e1, e2);
         return e0 > 0 && e1 > 0 && e2 > 0;
     }
+    __device__ __forceinline__ float depth_from(long long e0, long long e1, long long e2) const {
+        return depth_of(__ll2float_rn(e1 - b1), __ll2float_rn(e2 - b2), __ll2float_rn(e0 - b0), inv, a0, a1, a2);
+    }
+    __device__ __forceinline__ float depth_from(int e0, int e1, int e2) const {
+        return depth_of(__int2float_rn(e1 - (int)b1), __int2float_rn(e2 - (int)b2), __int2float_rn(e0 - (int)b0), inv,
+                        a0, a1, a2);
+    }
     __device__ __forceinline__ float depth(int i, int j) const {
         long long e0, e1, e2;
         edges(i, j, e0, e1, e2);
-        return depth_of(__ll2float_rn(e1 - b1), __ll2float_rn(e2 - b2), __ll2float_rn(e0 - b0), inv, a0, a1, a2);
+        return depth_from(e0, e1, e2);
+    }
+    // its vertices lie within kSmallExtent of each other: edge functions at pixel centres of its box fit 32 bits
+    __device__ __forceinline__ bool small() const {
+        return max(u0, max(u1, u2)) - min(u0, min(u1, u2)) < kSmallExtent &&
+               max(v0, max(v1, v2)) - min(v0, min(v1, v2)) < kSmallExtent;
     }
 };
 
@@ -240,8 +253,9 @@ __device__ __forceinline__ unsigned Setup32::hit_bits() const {
 __device__ __forceinline__ bool setup_big(const TriView &T, int a, int res, Setup64 &S, int &i0, int &i1, int &j0,
                                           int &j1) {
     const int U = (a + 1) % 3, V = (a + 2) % 3;
-    long long u0 = T.q[0][U], u1 = T.q[1][U], u2 = T.q[2][U];
-    long long v0 = T.q[0][V], v1 = T.q[1][V], v2 = T.q[2][V];
+    const auto at = [&](int k, int c) { return (long long)(c == 0 ? T.q[k][0] : (c == 1 ? T.q[k][1] : T.q[k][2])); };
+    long long u0 = at(0, U), u1 = at(1, U), u2 = at(2, U);
+    long long v0 = at(0, V), v1 = at(1, V), v2 = at(2, V);
     long long A2 = (u1 - u0) * (v2 - v0) - (v1 - v0) * (u2 - u0);
     if (A2 == 0) return false;
     float a0 = comp(T.p[0], a), a1 = comp(T.p[1], a), a2 = comp(T.p[2], a);
@@ -267,9 +281,90 @@ __device__ __forceinline__ bool setup_big(const TriView &T, int a, int res, Setu
     return i0 <= i1 && j0 <= j1;
 }
 
+// The crossed centres of a big pair's pixel box, swept by `step` threads of
+// which this is number `first`, kBatch pixels at a time: hits(v, i, j, depth)
+// for the batches with one, v[u] telling which of the kBatch pixels (i[u], j[u])
+// are crossed and depth(u) the depth there.  The threads cover a patch 32, 16,
+// ... pixels wide, as the box and their number allow, and the edge functions
+// advance by additions, in 32 bits for nearly every triangle (Word unsigned:
+// additions past the box may wrap, their results are not used), where a pixel
+// of the flattened box took a 64-bit division and six 64-bit products.
+template <int kBatch, class Word, class Int, class F>
+__device__ __forceinline__ void sweep_patch(const Setup64 &S, int i0, int i1, int j0, int j1, int first, int step,
+                                            F &&hits) {
+    int lw = 0;  // the patch is 2^lw wide
+    while (lw < 5 && (1 << lw) <= i1 - i0 && (2 << lw) <= step) ++lw;
+    const int i = i0 + (first & ((1 << lw) - 1)), rows = step >> lw;
+    int j = j0 + (first >> lw), x = i;
+    if (j > j1 || x > i1) return;
+    long long q0, q1, q2;
+    S.edges(i, j, q0, q1, q2);
+    Word r0 = (Word)q0, r1 = (Word)q1, r2 = (Word)q2, e0 = r0, e1 = r1, e2 = r2;
+    const Word c0 = (Word)(S.v0 - S.v1) * kSubpix << lw, c1 = (Word)(S.v1 - S.v2) * kSubpix << lw,
+               c2 = (Word)(S.v2 - S.v0) * kSubpix << lw;  // a patch to the right
+    const Word t0 = (Word)(S.u1 - S.u0) * kSubpix * (Word)rows, t1 = (Word)(S.u2 - S.u1) * kSubpix * (Word)rows,
+               t2 = (Word)(S.u0 - S.u2) * kSubpix * (Word)rows;  // the next patch row
+    while (j <= j1) {
+        bool v[kBatch], any = false;
+        int px[kBatch], py[kBatch];
+        Int f0[kBatch], f1[kBatch], f2[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            f0[u] = (Int)e0, f1[u] = (Int)e1, f2[u] = (Int)e2;
+            px[u] = x, py[u] = j;
+            v[u] = j <= j1 && f0[u] > 0 && f1[u] > 0 && f2[u] > 0;
+            any |= v[u];
+            x += 1 << lw;
+            e0 += c0, e1 += c1, e2 += c2;
+            if (x > i1) {
+                x = i;
+                j += rows;
+                r0 += t0, r1 += t1, r2 += t2;
+                e0 = r0, e1 = r1, e2 = r2;
+            }
+        }
+        if (any) hits(v, px, py, [&](int u) { return S.depth_from(f0[u], f1[u], f2[u]); });
+    }
+}
+
+template <int kBatch, class F>
+__device__ __forceinline__ void sweep_box(const Setup64 &S, int i0, int i1, int j0, int j1, int first, int step,
+                                          F &&hits) {
+    if (S.small())
+        sweep_patch<kBatch, unsigned, int>(S, i0, i1, j0, j1, first, step, hits);
+    else
+        sweep_patch<1, unsigned long long, long long>(S, i0, i1, j0, j1, first, step, hits);
+}
+
+// The fill pass's visit of the crossings among kN pixels of one face: all their
+// cursors are in flight before any sample is stored.
+constexpr int kFillBatch = 4;
+template <int kN, class Depth>
+__device__ __forceinline__ void fill_batch(const bool (&v)[kN], const int (&i)[kN], const int (&j)[kN], int res, int exiting, int t, int *cur, float *D,
+                                           int *Tr, long long cap, ldni_info_t *info, Depth depth) {
+    unsigned c[kN];
+#pragma unroll
+    for (int u = 0; u < kN; ++u) c[u] = v[u] ? (unsigned)cur[(long long)j[u] * res + i[u]] : 0u;
+#pragma unroll
+    for (int u = 0; u < kN; ++u)
+        if (v[u])
+            c[u] = c[u] & 0x80000000u ? (c[u] & 0x7fffffffu) + (unsigned)exiting
+                                      : (unsigned)atomicAdd(cur + (long long)j[u] * res + i[u], 1);
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+        if (!v[u]) continue;
+        if ((long long)c[u] >= cap) {
+            set_status(info, LDNI_ST_CAPACITY);
+            continue;
+        }
+        D[c[u]] = depth(u);
+        Tr[c[u]] = t;
+    }
+}
+
 // Queue of big (triangle, image) pairs: boxes up to kHugePixels from the
-// front (a warp each), larger ones from the back (a block each); n[0], n[1]
-// count the two ends.  The queue holds qcap entries.
+// front (a few threads each), larger ones from the back (blocks each); n[0],
+// n[1] count the two ends.  The queue holds qcap entries.
 template <class Code>
 __device__ __forceinline__ void enqueue_big(Code *q, long long qcap, int *n, Code code, long long npx) {
     if (npx > kHugePixels)
@@ -279,8 +374,12 @@ __device__ __forceinline__ void enqueue_big(Code *q, long long qcap, int *n, Cod
 }
 
 // Visit every queued pair with body(code, first, step), which walks the
-// pair's box pixels first, first + step, ...  Blocks blk of nblk: the
-// medium pairs a warp each; the huge pairs are shared out to groups of
+// pair's box with `step` threads.  Blocks blk of nblk: the medium pairs get a
+// warp each, or fewer threads, down to kPairThreads, when there are more pairs
+// than that leaves threads for (every thread of a pair repeats its loads and
+// setup, and waits for its own crossings' slots: 306,000 pairs of a batch of 48
+// meshes take 56 us (count) and 203 us (fill) with 4 threads each, 190 and 604
+// with 32); the huge pairs are shared out to groups of
 // nblk / (huge pairs) blocks (at least one), each group sweeping its pairs
 // with all its threads, so that a few faces of hundreds of thousands of
 // pixels keep every SM busy and many huge faces run side by side.
@@ -290,9 +389,11 @@ __device__ __forceinline__ void for_each_big(const Code *q, long long qcap, cons
                                              int huge_blocks, F &&body) {
     (void)huge_blocks;
     const int nmed = n[0];
-    const int wpb = blockDim.x >> 5;
-    for (int e = blk * wpb + (threadIdx.x >> 5); e < nmed; e += nblk * wpb)
-        body(q[e], (int)(threadIdx.x & 31), 32);
+    int pt = 32;
+    while (pt > kPairThreads && (long long)nmed * pt > (long long)nblk * blockDim.x) pt >>= 1;
+    const int gpb = blockDim.x / pt;
+    for (int e = blk * gpb + (int)threadIdx.x / pt; e < nmed; e += nblk * gpb)
+        body(q[e], (int)threadIdx.x & (pt - 1), pt);
     const int nh = n[1];
     if (nh <= 0) return;
     const int G = max(1, nblk / nh);  // blocks per huge pair
@@ -358,6 +459,7 @@ __device__ __forceinline__ int rank_step(unsigned long long kj, unsigned long lo
 }
 
 constexpr int kLanePer = 4;        // a lane orders rays of up to 4 samples by itself
+constexpr int kLaneSort = 8;       // longest ray a lane sorts in registers
 constexpr int kWarpSortMax = 128;  // longest ray a warp stages in shared memory
 constexpr int kRankMax = 768;      // longest ray ordered by ranks in place
 
@@ -373,14 +475,6 @@ struct RayOut {
     int *Tr;
     float *X, *Y, *Z;  // FP32 normals, or packed 8-bit normals in X with Y = Z = nullptr
 };
-
-// Takes the next slot of ray p (cursor word at cur + p) for a crossing that
-// leaves the solid or enters it: a pair's two slots follow from that alone, so
-// its cursor is only read, and stays in L1 for the neighbouring crossings.
-__device__ __forceinline__ long long claim_slot(int *cur, long long p, int exiting) {
-    const unsigned c = (unsigned)cur[p];
-    return c & 0x80000000u ? (long long)(c & 0x7fffffffu) + exiting : (long long)(unsigned)atomicAdd(cur + p, 1);
-}
 
 // Unit normals of a mesh's triangles, w: packed 8-bit codes.  An index outside
 // the mesh (a slot that no crossing filled: the mesh changed between count and
@@ -398,21 +492,6 @@ __device__ __forceinline__ void put_normal(const RayOut &o, long long at, const 
         o.Z[at] = q.z;
     }
 }
-
-// source of a ray's samples that were filled without normals
-struct TableSrc {
-    RayOut o;
-    long long b;
-    NormalTable nrm;
-    __device__ __forceinline__ void operator()(int i, float &d, int &t, float &x, float &y, float &z) const {
-        d = o.D[b + i];
-        t = o.Tr[b + i];
-        const float4 q = nrm(t);
-        x = o.Y ? q.x : q.w;
-        y = q.y;
-        z = q.z;
-    }
-};
 
 // source of a ray's samples that sits where the ordered ray goes
 struct InPlace {
@@ -519,24 +598,14 @@ __device__ __forceinline__ void rank_long(long long b, int n, const RayOut &o, S
     __syncwarp();
 }
 
-__device__ __forceinline__ RayOut shfl_out(const RayOut &o, int src) {
-    RayOut r;
-    r.D = reinterpret_cast<float *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(o.D), src));
-    r.Tr = reinterpret_cast<int *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(o.Tr), src));
-    r.X = reinterpret_cast<float *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(o.X), src));
-    r.Y = reinterpret_cast<float *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(o.Y), src));
-    r.Z = reinterpret_cast<float *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(o.Z), src));
-    return r;
-}
-
 // Orders the rays of the 32 lanes of a warp; every lane calls it, with n = 0
 // when it has nothing to order.  Rays of up to kLanePer samples are ordered
 // by their own lane, up to kWarpSortMax by the warp from the staged samples,
 // up to kRankMax by the warp in place (their samples must already sit at b),
 // longer ones by their lane's insertion.  make(sb, b, o) gives the source of
-// a ray whose samples are read from sb and go to b in o.  kOneOut: o is the
-// same in every lane.
-template <bool kOneOut, class Make>
+// a ray whose samples are read from sb and go to b in o.  o is the same
+// in every lane.
+template <class Make>
 __device__ __forceinline__ void order_warp_rays(long long b, int n, long long sb, const Make &make, const RayOut &o,
                                                 SortStage &st, int lane) {
     if (n >= 2 && n <= kLanePer) rank_staged<false>(b, n, make(sb, b, o), o, st, lane, kLanePer * lane);
@@ -546,70 +615,227 @@ __device__ __forceinline__ void order_warp_rays(long long b, int n, long long sb
     while (deep) {
         const int src = __ffs(deep) - 1;
         deep &= deep - 1;
-        const RayOut oo = kOneOut ? o : shfl_out(o, src);
         const long long bb = __shfl_sync(0xffffffffu, b, src);
         const long long sbb = __shfl_sync(0xffffffffu, sb, src);
         const int nn = __shfl_sync(0xffffffffu, n, src);
         if (nn <= kWarpSortMax)
-            rank_staged<true>(bb, nn, make(sbb, bb, oo), oo, st, lane, 0);
+            rank_staged<true>(bb, nn, make(sbb, bb, o), o, st, lane, 0);
         else
-            rank_long(bb, nn, oo, st, lane);
+            rank_long(bb, nn, o, st, lane);
     }
 }
 
-// Orders the rays of a warp's lanes whose samples were filled without normals,
-// and gives every sample its normal.  Every lane calls it, with n = 0 when it
-// has none.  pairs8: the arrays are 8-byte aligned.
-template <bool kOneOut>
-__device__ __forceinline__ void finish_warp_rays(long long b, int n, const RayOut &r, const NormalTable &nrm, bool pairs8,
-                                                 SortStage &st, int lane) {
-    if (n == 2) {  // the common case: everything in registers
-        const bool even = pairs8 && (b & 1) == 0;  // one 8-byte access per field
-        float d0, d1;
-        int t0, t1;
-        if (even) {
-            const float2 d = *reinterpret_cast<const float2 *>(r.D + b);
-            const int2 t = *reinterpret_cast<const int2 *>(r.Tr + b);
-            d0 = d.x, d1 = d.y, t0 = t.x, t1 = t.y;
-        } else {
-            d0 = r.D[b], d1 = r.D[b + 1], t0 = r.Tr[b], t1 = r.Tr[b + 1];
+// Rays of kLaneSort < n <= kFlatMax samples, ordered side by side: the samples
+// of as many of the warp's rays as fit are staged one after another, whatever
+// their lengths, and every lane ranks every 32nd of them within its own ray.
+// (One ray at a time leaves most lanes of a warp idle on rays of ten or
+// twenty samples, and moved every field through shared memory.)
+constexpr int kFlatMax = 256;
+struct FlatStage {
+    unsigned long long key[kFlatMax];
+    long long first[32];  // per lane: the ray's first slot
+    int before[32];       // per lane: staged samples before the ray's
+};
+static_assert(sizeof(FlatStage) <= sizeof(SortStage), "shares the warp's staging area");
+
+__device__ __forceinline__ void order_flat(long long b, int n, const RayOut &r, const NormalTable &nrm, SortStage &stage,
+                                           int lane) {
+    FlatStage &st = reinterpret_cast<FlatStage &>(stage);
+    int incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    for (int done = 0; done < total;) {
+        const bool fits = incl - done <= kFlatMax;  // this round's rays, and those before
+        const int m = __reduce_max_sync(0xffffffffu, fits ? incl : 0) - done;
+        st.first[lane] = b;
+        st.before[lane] = incl - n - done;
+        __syncwarp();
+        // (loads before stores throughout: the stores could be to anything for all the compiler knows)
+        constexpr int kPer = kFlatMax / 32, kHalf = kPer / 2;
+        float d[kPer];
+        int at[kPer], t[kPer];  // the sample's ray (its lane), its triangle
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const int s = 32 * q + lane;
+            at[q] = 0;
+            if (s >= m) continue;
+            int lo = 0;  // the last lane that begins at or before s: the one ray that holds it
+#pragma unroll
+            for (int h = 16; h > 0; h >>= 1)
+                if (st.before[lo + h] <= s) lo += h;
+            at[q] = lo;
+            const long long g = st.first[lo] + (s - st.before[lo]);
+            d[q] = r.D[g];
+            t[q] = r.Tr[g];
         }
-        if (key_less(d1, t1, d0, t0)) {
-            r.D[b] = d1, r.D[b + 1] = d0;
-            r.Tr[b] = t1, r.Tr[b + 1] = t0;
-            const int t = t0;
-            t0 = t1;
-            t1 = t;
-        }
-        const float4 q0 = nrm(t0), q1 = nrm(t1);
-        if (even) {
-            *reinterpret_cast<float2 *>(r.X + b) = r.Y ? make_float2(q0.x, q1.x) : make_float2(q0.w, q1.w);
-            if (r.Y) {
-                *reinterpret_cast<float2 *>(r.Y + b) = make_float2(q0.y, q1.y);
-                *reinterpret_cast<float2 *>(r.Z + b) = make_float2(q0.z, q1.z);
+#pragma unroll
+        for (int q = 0; q < kPer; ++q)
+            if (32 * q + lane < m) st.key[32 * q + lane] = sort_key(d[q], t[q]);
+        __syncwarp();
+        const int upto = incl - done;  // lane: end of its ray
+#pragma unroll
+        for (int hq = 0; hq < kPer; hq += kHalf) {
+            if (32 * hq >= m) break;  // the same for the whole warp
+            long long g[kHalf];
+            float4 nq[kHalf];
+#pragma unroll
+            for (int q = 0; q < kHalf; ++q) {
+                const int s = 32 * (hq + q) + lane, L = at[hq + q];
+                const int e = __shfl_sync(0xffffffffu, upto, L);
+                if (s >= m) continue;
+                const unsigned long long k = st.key[s];
+                int rank = 0, j = st.before[L];
+                for (; j + 4 <= e; j += 4) {  // four reads of shared memory in flight
+                    unsigned long long o[4];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) o[h] = st.key[j + h];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) rank += rank_step(o[h], k, j + h, s);
+                }
+                for (; j < e; ++j) rank += rank_step(st.key[j], k, j, s);
+                g[q] = st.first[L] + rank;
+                nq[q] = nrm(t[hq + q]);
             }
-        } else {
-            put_normal(r, b, q0);
-            put_normal(r, b + 1, q1);
+#pragma unroll
+            for (int q = 0; q < kHalf; ++q) {
+                if (32 * (hq + q) + lane >= m) continue;
+                r.D[g[q]] = d[hq + q];
+                r.Tr[g[q]] = t[hq + q];
+                put_normal(r, g[q], nq[q]);
+            }
         }
-        n = 0;
-    } else if (n == 1) {
+        __syncwarp();
+        done += m;
+    }
+}
+
+// ---- ordering of samples that were filled without normals -----------------------------
+//
+// Two kernels order every ray and give its samples their normals: one for rays
+// of two samples, nearly all of them, which lists the runs of 32 rays that hold
+// others, and one for those.  Together in one kernel the long rays' registers
+// spilled in the short ones' path, and a block that met many long rays made the
+// rest wait.  Batch of 48 meshes, a quarter of them noisy tori with up to 92
+// layers: 85 + 141 us, 265 to 510 us in one; 1.31 M-triangle sphere at 2048^2:
+// 73 + 6 us, 93 to 140 us in one.
+
+// A lane's range of samples in one run of 32 rays p0 .. (whole warp); odd counts
+// are reported if report.
+__device__ __forceinline__ int ray_samples(const int *__restrict__ off, long long p0, long long N, long long cap,
+                                           int lane, bool report, ldni_info_t *info, long long &b) {
+    const long long p = p0 + lane;
+    b = p < N ? off[p] : 0;
+    long long e = __shfl_down_sync(0xffffffffu, b, 1);
+    if (p >= N) return 0;
+    if (lane == 31 || p + 1 == N) e = off[p + 1];
+    if (report && ((e - b) & 1)) {
+        atomicAdd(&info->odd_rays, 1u);
+        set_status(info, LDNI_ST_ODD);
+    }
+    e = min(e, cap);
+    return range_ok(b, max(b, e), cap, info) ? (int)max(e - b, 0ll) : 0;
+}
+
+// A ray of two samples from slot b on.  pairs8: the arrays are 8-byte aligned.
+__device__ __forceinline__ void finish_pair(long long b, const RayOut &r, const NormalTable &nrm, bool pairs8) {
+    const bool even = pairs8 && (b & 1) == 0;  // one 8-byte access per field
+    float d0, d1;
+    int t0, t1;
+    if (even) {
+        const float2 d = *reinterpret_cast<const float2 *>(r.D + b);
+        const int2 t = *reinterpret_cast<const int2 *>(r.Tr + b);
+        d0 = d.x, d1 = d.y, t0 = t.x, t1 = t.y;
+    } else {
+        d0 = r.D[b], d1 = r.D[b + 1], t0 = r.Tr[b], t1 = r.Tr[b + 1];
+    }
+    const bool swap = key_less(d1, t1, d0, t0);
+    const float4 q0 = nrm(swap ? t1 : t0), q1 = nrm(swap ? t0 : t1);
+    if (swap) {
+        r.D[b] = d1, r.D[b + 1] = d0;
+        r.Tr[b] = t1, r.Tr[b + 1] = t0;
+    }
+    if (even) {
+        *reinterpret_cast<float2 *>(r.X + b) = r.Y ? make_float2(q0.x, q1.x) : make_float2(q0.w, q1.w);
+        if (r.Y) {
+            *reinterpret_cast<float2 *>(r.Y + b) = make_float2(q0.y, q1.y);
+            *reinterpret_cast<float2 *>(r.Z + b) = make_float2(q0.z, q1.z);
+        }
+    } else {
+        put_normal(r, b, q0);
+        put_normal(r, b + 1, q1);
+    }
+}
+
+// A warp's rays (b, n) of other numbers of samples (n = 0: none in this lane).
+__device__ __forceinline__ void finish_rest(long long b, int n, const RayOut &r, const NormalTable &nrm, SortStage &st,
+                                         int lane) {
+    if (n == 1) {
         put_normal(r, b, nrm(r.Tr[b]));
         n = 0;
+    } else if (n > 2 && n <= kLaneSort) {
+        // the lanes' rays side by side, each in its lane's registers (kLaneSort's network)
+        unsigned long long key[kLaneSort];
+        float d[kLaneSort];
+#pragma unroll
+        for (int i = 0; i < kLaneSort; ++i) {
+            d[i] = i < n ? r.D[b + i] : 0.0f;
+            key[i] = i < n ? sort_key(d[i], r.Tr[b + i]) : ~0ull;
+        }
+#pragma unroll
+        for (int p = 1; p < kLaneSort; p <<= 1)  // Batcher's odd-even merge sort
+#pragma unroll
+            for (int k = p; k >= 1; k >>= 1)
+#pragma unroll
+                for (int j = k % p; j + k < kLaneSort; j += 2 * k)
+#pragma unroll
+                    for (int i = 0; i < k; ++i)
+                        if (i + j + k < kLaneSort && (i + j) / (2 * p) == (i + j + k) / (2 * p)) {
+                            const bool swap = key[i + j + k] < key[i + j];
+                            const unsigned long long a = key[i + j], c = key[i + j + k];
+                            const float x = d[i + j], y = d[i + j + k];
+                            key[i + j] = swap ? c : a;
+                            key[i + j + k] = swap ? a : c;
+                            d[i + j] = swap ? y : x;
+                            d[i + j + k] = swap ? x : y;
+                        }
+        // (a store could be to the table for all the compiler knows: four normals are read before the
+        // first of their samples is stored, or each would wait for the one before)
+#pragma unroll
+        for (int h = 0; h < kLaneSort; h += 4) {
+            if (h >= n) break;
+            float4 q[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (h + i < n) q[i] = nrm(key_tri(key[h + i]));
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (h + i < n) {
+                    r.D[b + h + i] = d[h + i];
+                    r.Tr[b + h + i] = key_tri(key[h + i]);
+                    put_normal(r, b + h + i, q[i]);
+                }
+        }
+        n = 0;
     }
-    // rays that are ordered in place get their normals first
-    unsigned longer = __ballot_sync(0xffffffffu, n > kWarpSortMax);
+    const bool flat = n > 0 && n <= kFlatMax;
+    if (__any_sync(0xffffffffu, flat)) order_flat(b, flat ? n : 0, r, nrm, st, lane);
+    if (flat) n = 0;
+    // longer rays are ordered in place, and get their normals first
+    unsigned longer = __ballot_sync(0xffffffffu, n > 0);
+    if (!longer) return;
     while (longer) {
         const int src = __ffs(longer) - 1;
         longer &= longer - 1;
-        const RayOut o = kOneOut ? r : shfl_out(r, src);
         const long long bb = __shfl_sync(0xffffffffu, b, src);
         const int nn = __shfl_sync(0xffffffffu, n, src);
-        for (int i = lane; i < nn; i += 32) put_normal(o, bb + i, nrm(o.Tr[bb + i]));
-        __syncwarp();
+        for (int i = lane; i < nn; i += 32) put_normal(r, bb + i, nrm(r.Tr[bb + i]));
     }
-    order_warp_rays<kOneOut>(
-        b, n, b, [&](long long, long long at, const RayOut &o) { return TableSrc{o, at, nrm}; }, r, st, lane);
+    __syncwarp();
+    order_warp_rays(b, n, b, [](long long, long long at, const RayOut &o) { return InPlace{o, at}; }, r, st, lane);
 }
 
 }  // namespace ldni

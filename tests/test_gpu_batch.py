@@ -196,3 +196,34 @@ def test_full_union_chain_workload(ldni):
         for k in range(1, 64):
             acc = oracle.boolean(acc, P[k].numpy(), "union")
         assert bit_equal(got, acc)
+
+
+@pytest.mark.parametrize("packed", [False, True])
+@pytest.mark.parametrize("slabs,res", [(1, 33), (2, 64), (4, 31), (5, 40), (64, 24), (70, 17), (300, 9), (400, 8)])
+def test_ray_lengths(ldni, slabs, res, packed):
+    """Rays of every length the ordering treats apart (2, up to 8, staged side
+    by side up to 256, in place up to 768, beyond), single-mesh and batched,
+    FP32 and packed normals: depths, ids and normals against the mesh itself."""
+    v, t = M.slab_stack(slabs, axis=2, seed=res)
+    grid = ldni.Grid.cube((-0.5, -0.5, -0.5), 1.0, res)
+    one = ldni.sample(v, t, grid, "all", packed=packed)
+    p = v.astype(np.float64)[t]
+    nrm = np.cross(p[:, 1] - p[:, 0], p[:, 2] - p[:, 0])
+    nrm /= np.linalg.norm(nrm, axis=1, keepdims=True)
+    for a in range(3):
+        g = one[a].numpy()
+        ray = np.repeat(np.arange(res * res), np.diff(g["offsets"]))
+        order = np.lexsort((g["tri"], g["depth"], ray))
+        assert np.array_equal(order, np.arange(len(ray)))  # ascending by (depth, id) in every ray
+        assert np.all(np.abs(nrm[g["tri"]][:, a]) == 1.0)  # only faces across the ray
+        assert np.all(np.abs(g["depth"] - v[t[g["tri"]][:, 0], a]) <= 1e-5 * 3 ** 0.5)  # the sampling bound
+        if packed:
+            code = np.rint((nrm[g["tri"]] + 1) * 127.5).astype(np.uint32)
+            assert np.array_equal(g["nrm8"], code[:, 0] | (code[:, 1] << 8) | (code[:, 2] << 16))
+        else:
+            assert np.all(np.abs(g["nrm"] - nrm[g["tri"]]) <= 1e-5)  # the sampling bound
+    if not packed:
+        plan = ldni.BatchPlan([(v, t), (v, t)], [grid, grid], [[L.n for L in one]] * 2)
+        plan.run()
+        for outs in plan.finish():
+            assert all(ldni.identical(x, y) for x, y in zip(outs, one))
