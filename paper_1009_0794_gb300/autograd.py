@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import torch
 
+from . import _lib
 from . import ldni as _L
 
 
@@ -21,18 +22,21 @@ class LDNIVolume(torch.autograd.Function):
         t = tris.to("cuda", torch.int32).contiguous()
         layers = _L.sample(v, t, grid, axis)
         layers = layers if isinstance(layers, list) else [layers]
-        vols = [_L.volume(L) for L in layers]
+        # the images' volumes in one launch and one readback (their status); the mean stays on the device
+        infos = torch.zeros(len(layers), _lib.INFO_BYTES // 8, dtype=torch.int64, device="cuda")
+        vols = _L.volume_many(layers, infos=infos, sync=False)
+        if any(row[3] & _lib.ST_ODD for row in infos.tolist()):
+            raise _lib.LDNIError(-3, "ldni_volume")
         ctx.save_for_backward(v, t)
         ctx.layers = layers
-        return torch.tensor(sum(vols) / len(vols), dtype=torch.float64, device="cuda")
+        return vols.mean()
 
     @staticmethod
     def backward(ctx, g):
         v, t = ctx.saved_tensors
         grad = torch.zeros(v.shape[0], 3, dtype=torch.float32, device="cuda")
         w = float(g.item()) / len(ctx.layers)
-        for L in ctx.layers:
-            _L.volume_grad(v, t, L, w, grad)
+        _L.volume_grads(v, t, ctx.layers, w, grad)
         return grad.to(torch.float64 if g.dtype == torch.float64 else grad.dtype), None, None, None
 
 

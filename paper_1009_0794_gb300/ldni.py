@@ -23,6 +23,9 @@ OPS = {"union": _lib.OP_UNION, "inter": _lib.OP_INTER, "intersection": _lib.OP_I
        "diff": _lib.OP_DIFF, "difference": _lib.OP_DIFF}
 
 
+_CUDA = torch.device("cuda")  # the current device
+
+
 @dataclass(frozen=True)
 class Grid:
     """The cube shared by the three images (Definition 3)."""
@@ -47,12 +50,7 @@ class Grid:
         return self.width / self.res
 
     def c(self) -> _CGrid:
-        g = _CGrid()
-        for k in range(3):
-            g.origin[k] = self.origin[k]
-        g.width = self.width
-        g.res = self.res
-        return g
+        return _CGrid((ctypes.c_float * 3)(*self.origin), self.width, self.res)
 
 
 class LDNI:
@@ -76,16 +74,9 @@ class LDNI:
         return int(self.depth.numel())
 
     def c(self) -> _CLayers:
-        L = _CLayers()
-        L.offsets = self.offsets.data_ptr()
-        L.depth = self.depth.data_ptr() if self.depth.numel() else None
-        L.nx = self.nx.data_ptr() if self.nx.numel() else None
-        L.ny = self.ny.data_ptr() if self.ny.numel() else None
-        L.nz = self.nz.data_ptr() if self.nz.numel() else None
-        L.tri_id = self.tri.data_ptr() if self.tri.numel() else None
-        L.capacity = self.capacity
-        L.nrm8 = (self.nrm8.data_ptr() if self.nrm8.numel() else None) if self.packed else None
-        return L
+        ptr = lambda t: t.data_ptr() if t is not None and t.numel() else None
+        return _CLayers(self.offsets.data_ptr(), ptr(self.depth), ptr(self.nx), ptr(self.ny), ptr(self.nz),
+                        ptr(self.tri), self.capacity, ptr(self.nrm8))
 
     def counts(self):
         return self.offsets[1:] - self.offsets[:-1]
@@ -117,8 +108,9 @@ def identical(A: "LDNI", B: "LDNI") -> bool:
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _dev(x, dtype) -> torch.Tensor:
@@ -136,14 +128,12 @@ def _axes(axis) -> List[int]:
 
 
 def new_info() -> torch.Tensor:
-    return torch.zeros(_lib.INFO_BYTES // 8, dtype=torch.int64, device="cuda")
+    return torch.zeros(_lib.INFO_BYTES // 8, dtype=torch.int64, device=_CUDA)
 
 
 def info_decode(info: torch.Tensor) -> dict:
-    h = info.cpu().numpy()
-    st = int(h[3]) & 0xFFFFFFFF
-    odd = (int(h[3]) >> 32) & 0xFFFFFFFF
-    return {"n": [int(x) for x in h[:3]], "status": st, "odd_rays": odd}
+    h = info.tolist()
+    return {"n": h[:3], "status": h[3] & 0xFFFFFFFF, "odd_rays": (h[3] >> 32) & 0xFFFFFFFF}
 
 
 def _raise_status(st: int, what: str):
@@ -172,11 +162,19 @@ def sample_workspace_size(nv: int, nt: int, res: int, axis=_lib.AXIS_ALL) -> int
 def empty_layers(grid: Grid, axis: int, capacity: int, packed: bool = False) -> LDNI:
     """Device buffers of one image; packed: 8-bit normals (one int32 word per
     sample) instead of three FP32 arrays."""
-    N = grid.res * grid.res
-    f = lambda k: torch.empty(k, dtype=torch.float32, device="cuda")
-    i = lambda k: torch.empty(k, dtype=torch.int32, device="cuda")
+    return _around(grid, axis, _empty_offsets(grid), capacity, packed)
+
+
+def _empty_offsets(grid: Grid) -> torch.Tensor:
+    return torch.empty(grid.res * grid.res + 1, dtype=torch.int32, device=_CUDA)
+
+
+def _around(grid: Grid, axis: int, offsets: torch.Tensor, capacity: int, packed: bool) -> LDNI:
+    """An image with the given offsets and new sample arrays."""
+    f = lambda k: torch.empty(k, dtype=torch.float32, device=_CUDA)
+    i = lambda k: torch.empty(k, dtype=torch.int32, device=_CUDA)
     nc = 0 if packed else capacity
-    return LDNI(grid, axis, i(N + 1), f(capacity), f(nc), f(nc), f(nc), i(capacity), 0,
+    return LDNI(grid, axis, offsets, f(capacity), f(nc), f(nc), f(nc), i(capacity), 0,
                 nrm8=i(capacity) if packed else None)
 
 
@@ -235,8 +233,8 @@ def sample(verts, tris, grid: Grid, axis="all", mode: str = "exact2", stream=Non
     wsz = (sample_binned_workspace_size if binned else sample_workspace_size)(v.shape[0], t.shape[0], grid.res, cax)
     ws = torch.empty(wsz, dtype=torch.uint8, device="cuda")
     info = new_info()
-    outs = [empty_layers(grid, a, 0) for a in axes]
-    arr = (_CLayers * len(axes))(*[o.c() for o in outs])
+    offsets = [_empty_offsets(grid) for _ in axes]  # the count pass writes these alone
+    arr = (_CLayers * len(axes))(*[_CLayers(o.data_ptr()) for o in offsets])
     g = grid.c()
     sp = _stream_ptr(stream)
     _lib.check(count_fn(v.data_ptr(), v.shape[0], t.data_ptr(), t.shape[0], ctypes.byref(g), cax, arr,
@@ -245,10 +243,8 @@ def sample(verts, tris, grid: Grid, axis="all", mode: str = "exact2", stream=Non
     _raise_status(meta["status"], "ldni_sample_count")
     res_list = []
     for k, a in enumerate(axes):
-        n = meta["n"][a]
-        L = empty_layers(grid, a, n, packed)
-        L.offsets = outs[k].offsets
-        L.n = n
+        L = _around(grid, a, offsets[k], meta["n"][a], packed)
+        L.n = meta["n"][a]
         res_list.append(L)
     arr = (_CLayers * len(axes))(*[o.c() for o in res_list])
     _lib.check(fill_fn(v.data_ptr(), v.shape[0], t.data_ptr(), t.shape[0], ctypes.byref(g), cax, arr,
@@ -338,6 +334,10 @@ def volume(L: LDNI, stream=None, out: Optional[torch.Tensor] = None, ws: Optiona
            info: Optional[torch.Tensor] = None, sync: bool = True):
     """Enclosed volume seen by one LDNI (odd-to-even ranges inside)."""
     lib = _lib.load()
+    both = None
+    if out is None and info is None:  # side by side: one clear, one readback
+        both = torch.zeros(_lib.INFO_BYTES // 8 + 1, dtype=torch.int64, device=_CUDA)
+        info, out = both[:-1], both[-1:].view(torch.float64)
     if out is None:
         out = torch.zeros(1, dtype=torch.float64, device="cuda")
     if ws is None:
@@ -349,10 +349,11 @@ def volume(L: LDNI, stream=None, out: Optional[torch.Tensor] = None, ws: Optiona
                                ws.numel(), _stream_ptr(stream)), "ldni_volume")
     if not sync:
         return out
-    meta = info_decode(info)
+    host = both.cpu() if both is not None else None
+    meta = info_decode(info if host is None else host[:-1])
     if meta["status"] & _lib.ST_ODD:
         raise _lib.LDNIError(-3, "ldni_volume")
-    return float(out.item())
+    return float(out.item()) if host is None else float(host[-1:].view(torch.float64).item())
 
 
 def boolean_many_workspace_size(res: int, count: int) -> int:
@@ -694,15 +695,23 @@ def depth_vjp(verts: torch.Tensor, tris: torch.Tensor, L: LDNI, grad_depth: torc
 def volume_grad(verts: torch.Tensor, tris: torch.Tensor, L: LDNI, grad_volume: float = 1.0,
                 grad_verts: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """grad_verts += grad_volume * d(volume of L)/d(verts), fixed crossing set."""
+    return volume_grads(verts, tris, [L], grad_volume, grad_verts, stream)
+
+
+def volume_grads(verts: torch.Tensor, tris: torch.Tensor, Ls: Sequence[LDNI], grad_volume: float = 1.0,
+                 grad_verts: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
+    """volume_grad of several images, added up in grad_verts."""
     v = verts.contiguous()
     t = tris.contiguous()
     if grad_verts is None:
         grad_verts = torch.zeros(v.shape[0], 3, dtype=torch.float32, device="cuda")
     info = new_info()
-    lc, g = L.c(), L.grid.c()
-    _lib.check(_lib.load().ldni_volume_grad(v.data_ptr(), v.shape[0], t.data_ptr(), t.shape[0], ctypes.byref(g),
-                                            L.axis, ctypes.byref(lc), float(grad_volume), grad_verts.data_ptr(),
-                                            info.data_ptr(), _stream_ptr(stream)), "ldni_volume_grad")
+    sp = _stream_ptr(stream)
+    for L in Ls:
+        lc, g = L.c(), L.grid.c()
+        _lib.check(_lib.load().ldni_volume_grad(v.data_ptr(), v.shape[0], t.data_ptr(), t.shape[0], ctypes.byref(g),
+                                                L.axis, ctypes.byref(lc), float(grad_volume), grad_verts.data_ptr(),
+                                                info.data_ptr(), sp), "ldni_volume_grad")
     return grad_verts
 
 
