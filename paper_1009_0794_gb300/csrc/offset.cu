@@ -347,7 +347,11 @@ __device__ __forceinline__ void put_result(const OffArgs &A, int b, long long hb
 // One pixel row of a tile of image blockIdx.y, a warp per ray.  The block
 // walks the tile's list, kStage spheres at a time (the next ones' loads in
 // flight), and stages those that reach its row (about a third), with their
-// distance from the row, which all its rays share.  Every warp then tests
+// distance from the row, which all its rays share, in the list's order: the
+// buffer's merges then fall on the same spheres in both passes, which agree
+// on every ray.  (Slots handed out by one shared counter depended on the
+// warps' timing, and a warp that was late to read that counter could find it
+// cleared for the next round.)  Every warp then tests
 // them against its ray; the ones that meet it become intervals, whose
 // components are found by warp-wide minima and maxima, about a dozen sweeps
 // over the five intervals a lane holds (150 a ray on the 128^2 flower by 2.5
@@ -361,7 +365,9 @@ template <bool kDeep>
 __device__ __forceinline__ void ray_row(const OffArgs &A, int bx, int b, ldni_info_t *info) {
     __shared__ float4 sc[kStage];  // (centre along the ray, u, squared distance from the row, sphere)
     __shared__ uint4 sbuf[kOffWarps][kBuf];
-    __shared__ int s_n, s_deep;
+    __shared__ int s_cnt[kStagePer * kOffWarps];  // staged spheres of each warp's 32, in list order
+    __shared__ int s_deep;
+    static_assert(kStagePer * kOffWarps <= 32, "a lane per count");
     if (threadIdx.x == 0) s_deep = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -420,21 +426,31 @@ __device__ __forceinline__ void ray_row(const OffArgs &A, int bx, int b, ldni_in
     };
     fetch(0);
     for (int base = 0; base < nl; base += kStage) {
-        if (threadIdx.x == 0) s_n = 0;
-        __syncthreads();  // the previous round's spheres are read
+        float dv2[kStagePer];
+        unsigned in[kStagePer];
 #pragma unroll
         for (int k = 0; k < kStagePer; ++k) {
-            const float dv = __fsub_rn(pv, c4(cc[k], bv)), dv2 = __fmul_rn(dv, dv);
-            const bool in = sid[k] >= 0 && dv2 < A.r2;  // (du du + dv dv, rounded, is no smaller than dv dv)
-            const unsigned m = __ballot_sync(kAll, in);
-            int at = 0;
-            if (lane == 0 && m) at = atomicAdd(&s_n, __popc(m));
-            at = __shfl_sync(kAll, at, 0) + __popc(m & ((1u << lane) - 1u));
-            if (in) sc[at] = make_float4(c4(cc[k], b), c4(cc[k], bu), dv2, __int_as_float(sid[k]));
+            const float dv = __fsub_rn(pv, c4(cc[k], bv));
+            dv2[k] = __fmul_rn(dv, dv);
+            in[k] = __ballot_sync(kAll, sid[k] >= 0 && dv2[k] < A.r2);  // (du du + dv dv, rounded, is no smaller)
+            if (lane == 0) s_cnt[k * kOffWarps + w] = __popc(in[k]);
+        }
+        __syncthreads();  // the counts are in; the previous round's spheres are read
+        int upto = lane < kStagePer * kOffWarps ? s_cnt[lane] : 0;  // staged by the first lane + 1 of them
+#pragma unroll
+        for (int o = 1; o < kStagePer * kOffWarps; o <<= 1) {
+            const int x = __shfl_up_sync(kAll, upto, o);
+            if (lane >= o) upto += x;
+        }
+        const int ns = __shfl_sync(kAll, upto, kStagePer * kOffWarps - 1);
+#pragma unroll
+        for (int k = 0; k < kStagePer; ++k) {
+            const int end = __shfl_sync(kAll, upto, k * kOffWarps + w);
+            if ((in[k] >> lane) & 1u)
+                sc[end - __popc(in[k] >> lane)] = make_float4(c4(cc[k], b), c4(cc[k], bu), dv2[k], __int_as_float(sid[k]));
         }
         fetch(base + kStage);
-        __syncthreads();
-        const int ns = s_n;
+        __syncthreads();  // the spheres are staged; the counts are read
         for (int k0 = 0; k0 < ns && live && !over; k0 += 32) {
             float4 c;
             float q = INFINITY;
@@ -475,12 +491,13 @@ __device__ __forceinline__ void ray_row(const OffArgs &A, int bx, int b, ldni_in
         return __reduce_min_sync(kAll, at);
     };
     const long long oslot = kDeep ? (long long)pick(A.ooff, b)[p] : 0;
+    const int room = kDeep ? pick(A.cnt, b)[p] : 0;  // the ray's slots: what the count pass found
     unsigned tags[kKept] = {};
     int nout = 0;
     // one interval of the result, thinner than eps removed
     auto emit = [&](unsigned tag0, unsigned tag1) {
         if (kDeep) {
-            if (lane < 2) put_result(A, b, hb, pu, pv, lane ? tag1 : tag0, oslot + nout + lane, info);
+            if (lane < 2 && nout + lane < room) put_result(A, b, hb, pu, pv, lane ? tag1 : tag0, oslot + nout + lane, info);
         } else {
 #pragma unroll
             for (int z = 0; z < kKept; z += 2)

@@ -134,3 +134,19 @@ def test_rays_of_many_samples(ldni, slabs, res, rpix):
     for inner in (False, True):
         for eps in (0.0, 0.01):
             _check(ldni, grid, ref, H, rpix / res, inner, eps=eps)
+
+
+@pytest.mark.parametrize("inner", [False, True])
+def test_tile_lists_of_many_staging_rounds(ldni, inner):
+    """Tile lists of several staging rounds whose tiles mix rays of every
+    length with rays past the image's edge and rays that no second pass takes:
+    every ray equals the oracle's, call after call."""
+    res = 42  # the last tiles hold two rays of each row
+    grid, ref, H = _solid(ldni, M.slab_stack(40, axis=0, seed=4), res)
+    assert H[0].n > 2 * 512 * 36  # more than two rounds of 512 spheres for each of the 36 tiles, on average
+    first = _check(ldni, grid, ref, H, 0.2 / res, inner)
+    counts = first[0].counts()
+    assert int(counts.max()) > 8 and int(counts.min()) <= 8  # both ways of writing a ray
+    for _ in range(20):
+        again = ldni.offset(H, 0.2 / res, inner=inner)
+        assert all(ldni.identical(x, y) for x, y in zip(first, again))
