@@ -47,8 +47,9 @@ namespace {
 constexpr int kOffWarps = 8;      // rays (warps) per block: one pixel row of a tile
 constexpr int kStagePer = 2;      // spheres of the tile's list a thread looks at per round
 constexpr int kStage = kOffWarps * 32 * kStagePer;
-constexpr int kBuf = 288;         // intervals of one ray held in shared memory
-constexpr int kMaxComp = 256;     // components a ray may keep when its intervals are merged to make room
+constexpr int kMaxComp = 257;     // components a ray may keep when its intervals are merged to make room: those
+                                  // of 512 samples (an inner offset's are bounded by one more than its intervals)
+constexpr int kBuf = kMaxComp + 32;  // intervals of one ray held in shared memory: room for a warp's after a merge
 constexpr int kMaxHSamples = 384; // H's samples on one ray
 constexpr int kKept = 8;          // samples whose sources the count pass leaves to the write pass
 constexpr int kTile = kOffWarps;  // pixels per side of a sphere-list tile

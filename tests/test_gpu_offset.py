@@ -150,3 +150,56 @@ def test_tile_lists_of_many_staging_rounds(ldni, inner):
     for _ in range(20):
         again = ldni.offset(H, 0.2 / res, inner=inner)
         assert all(ldni.identical(x, y) for x, y in zip(first, again))
+
+
+def _by_hand(rays, res):
+    """An image with the given samples ({ray: ascending depths}), normals and
+    ids made up."""
+    off = np.zeros(res * res + 1, np.int64)
+    for p, d in rays.items():
+        off[p + 1] = len(d)
+    off = np.cumsum(off)
+    d = np.concatenate([np.asarray(rays[p], np.float32) for p in sorted(rays)] or [np.zeros(0, np.float32)])
+    n = len(d)
+    nrm = np.tile(np.float32([0.6, 0.0, -0.8]), (n, 1))
+    return {"offsets": off, "depth": d, "nrm": nrm, "tri": np.arange(n, dtype=np.int32)}
+
+
+@pytest.mark.parametrize("inside,fits", [(255, True), (300, False)])
+def test_most_components_of_an_inner_ray(ldni, inside, fits):
+    """One ray whose solid interval holds `inside` spheres of their own: 256
+    result intervals (512 samples) are the most a ray may have while its
+    buffer is merged, which 50 more spheres in its gap make happen; more
+    than the buffer holds at all are reported."""
+    res, gap = 360, 50
+    c = (np.float32(-0.5) + (np.arange(res, dtype=np.float32) + np.float32(0.5)) * (np.float32(1.0) / np.float32(res)))
+    h, j, k = 1.0 / res, 7, 9
+    far = float(c[40]) + 0.5 * h  # meets no ray of the other images
+    X = {k * res + j: [float(c[gap]) + 0.5 * h, float(c[gap + inside + 1]) - 0.5 * h + h]}
+    Y = {i * res + k: [float(c[j]), far] for i in range(gap + inside + 1)}
+    ref = [_by_hand(X, res), _by_hand(Y, res), _by_hand({}, res)]
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    H = [_upload(ldni, grid, a, L) for a, L in enumerate(ref)]
+    if fits:
+        got = _check(ldni, grid, ref, H, 0.2 * h, True)
+        assert int(got[0].counts().max()) == 512
+    else:
+        with pytest.raises(ldni.LDNIError) as e:
+            ldni.offset(H, 0.2 * h, inner=True)
+        assert e.value.code == -4
+
+
+@pytest.mark.parametrize("samples,fits", [(384, True), (386, False)])
+def test_most_samples_of_the_solid_on_a_ray(ldni, samples, fits):
+    res = 8
+    X = {19: (np.arange(samples) / np.float32(1024) - np.float32(0.25)).tolist()}
+    ref = [_by_hand(X, res), _by_hand({}, res), _by_hand({}, res)]
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    H = [_upload(ldni, grid, a, L) for a, L in enumerate(ref)]
+    for inner in (False, True):
+        if fits:
+            _check(ldni, grid, ref, H, 1e-4, inner)
+        else:
+            with pytest.raises(ldni.LDNIError) as e:
+                ldni.offset(H, 1e-4, inner=inner)
+            assert e.value.code == -4
