@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(kThreads) batch_tri_pass(const ldni_batch_item
 
 template <bool kFill>
 __global__ void __launch_bounds__(kThreads, 4) batch_big(const ldni_batch_item_t *items, Tables T, int *counts,
-                                                      int huge_blocks, ldni_info_t *infos) {
-    for_each_big(T.big, T.qcap, T.big_n, (int)blockIdx.x, (int)gridDim.x, huge_blocks,
+                                                      ldni_info_t *infos) {
+    for_each_big(T.big, T.qcap, T.big_n, (int)blockIdx.x, (int)gridDim.x,
                  [&](long long code, int first, int step) {
         const int m = (int)(code >> 34), t = (int)((code >> 2) & 0xFFFFFFFF), a = (int)(code & 3);
         const ldni_batch_item_t &it = items[m];
@@ -455,7 +455,7 @@ extern "C" int ldni_sample_batch(const ldni_batch_item_t *items_dev, const ldni_
         LDNI_LAUNCH(K_BATCH, s, batch_tri_pass<false><<<(unsigned)tiles, kThreads, 0, s>>>(items_dev, count, w.T,
                                                                                              w.counts, infos));
         LDNI_LAUNCH(K_BATCH, s,
-                    batch_big<false><<<5 * num_sms(), kThreads, 0, s>>>(items_dev, w.T, w.counts, num_sms(), infos));
+                    batch_big<false><<<5 * num_sms(), kThreads, 0, s>>>(items_dev, w.T, w.counts, infos));
     }
     LDNI_LAUNCH(K_BATCH, s,
                 batch_scan<<<(unsigned)chunks, kThreads, 0, s>>>(items_dev, count, w.T, w.counts, w.words, infos,
@@ -464,7 +464,7 @@ extern "C" int ldni_sample_batch(const ldni_batch_item_t *items_dev, const ldni_
         LDNI_LAUNCH(K_BATCH, s, batch_tri_pass<true><<<(unsigned)tiles, kThreads, 0, s>>>(items_dev, count, w.T,
                                                                                             w.counts, infos));
         LDNI_LAUNCH(K_BATCH, s,
-                    batch_big<true><<<5 * num_sms(), kThreads, 0, s>>>(items_dev, w.T, w.counts, num_sms(), infos));
+                    batch_big<true><<<5 * num_sms(), kThreads, 0, s>>>(items_dev, w.T, w.counts, infos));
     }
     LDNI_LAUNCH(K_BATCH, s,
                 batch_sort<<<(unsigned)(chunks * kSortParts), kThreads, 0, s>>>(items_dev, count, w.T, infos));

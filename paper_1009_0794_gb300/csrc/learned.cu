@@ -422,8 +422,8 @@ __global__ void __launch_bounds__(kThreads, kOnepassBlocksPerSm) onepass_kernel(
 
 __global__ void __launch_bounds__(kThreads) onepass_big(const float *__restrict__ verts, const int *__restrict__ tris,
                                                         int nv, GridDev g, LImg o, const int *big_q, long long qcap,
-                                                        const int *big_n, int huge_blocks) {
-    for_each_big(big_q, qcap, big_n, (int)blockIdx.x, (int)gridDim.x, huge_blocks, [&](int code, int first, int step) {
+                                                        const int *big_n) {
+    for_each_big(big_q, qcap, big_n, (int)blockIdx.x, (int)gridDim.x, [&](int code, int first, int step) {
         const int t = code >> 2, a = code & 3;
         TriView T;
         if (load_tri(verts, tris, t, nv, g, T)) return;
@@ -490,7 +490,7 @@ __device__ __forceinline__ void redo_axis(const TriView &T, int t, const float3 
 __device__ __forceinline__ void redo_big_block(const float *__restrict__ verts, const int *__restrict__ tris, int nv,
                                                const GridDev &g, const LImg &o, const int *big_q, long long qcap,
                                                const int *big_n, int blk, int nblk, ldni_info_t *info) {
-    for_each_big(big_q, qcap, big_n, blk, nblk, max(1, nblk / 3), [&](int code, int first, int step) {
+    for_each_big(big_q, qcap, big_n, blk, nblk, [&](int code, int first, int step) {
         const int t = code >> 2, a = code & 3;
         TriView T;
         if (load_tri(verts, tris, t, nv, g, T)) return;
@@ -913,7 +913,7 @@ extern "C" int ldni_sample_learned(const float *verts, int64_t nv, const int32_t
                                                                         o, w.big_q, w.qcap, w.big_n, info));
         LDNI_LAUNCH(K_ONEPASS_BIG, s,
                     onepass_big<<<5 * num_sms(), kThreads, 0, s>>>(verts, tris, (int)nv, g, o, w.big_q, w.qcap,
-                                                                   w.big_n, num_sms()));
+                                                                   w.big_n));
     }
     const int *cnt[3];
     int *off[3];

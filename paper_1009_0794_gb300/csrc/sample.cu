@@ -147,8 +147,8 @@ __global__ void __launch_bounds__(kThreads) tri_pass(const float *__restrict__ v
 template <bool kFill>
 __global__ void __launch_bounds__(kThreads) big_pass(const float *__restrict__ verts, const int *__restrict__ tris,
                                                      int nv, GridDev g, Img o, const int *big_q, long long qcap,
-                                                     const int *big_n, int huge_blocks, ldni_info_t *info) {
-    for_each_big(big_q, qcap, big_n, (int)blockIdx.x, (int)gridDim.x, huge_blocks, [&](int code, int first, int step) {
+                                                     const int *big_n, ldni_info_t *info) {
+    for_each_big(big_q, qcap, big_n, (int)blockIdx.x, (int)gridDim.x, [&](int code, int first, int step) {
         const int t = code >> 2, a = code & 3;
         TriView T;
         if (load_tri(verts, tris, t, nv, g, T)) return;
@@ -502,7 +502,7 @@ int run_count(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, c
                                                                           C.w.qcap, C.w.big_n, info));
         LDNI_LAUNCH(K_COUNT_BIG, C.s,
                     big_pass<false><<<5 * num_sms(), kThreads, 0, C.s>>>(verts, tris, (int)nv, C.g, C.o, C.w.big_q,
-                                                                        C.w.qcap, C.w.big_n, num_sms(), info));
+                                                                        C.w.qcap, C.w.big_n, info));
     }
     const int *cnt[3];
     int *off[3];
@@ -534,7 +534,7 @@ int run_fill(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, co
                                                                          C.w.qcap, C.w.big_n, info));
         LDNI_LAUNCH(K_FILL_BIG, C.s,
                     big_pass<true><<<5 * num_sms(), kThreads, 0, C.s>>>(verts, tris, (int)nv, C.g, C.o, C.w.big_q,
-                                                                       C.w.qcap, C.w.big_n, num_sms(), info));
+                                                                       C.w.qcap, C.w.big_n, info));
     }
     run_sort(C, info);
     return cuda_status();
@@ -616,7 +616,7 @@ int run_binned_count(const float *verts, int64_t nv, const int32_t *tris, int64_
     if (nt > 0)
         LDNI_LAUNCH(K_COUNT_BIG, C.s,
                     big_pass<false><<<5 * num_sms(), kThreads, 0, C.s>>>(verts, tris, (int)nv, C.g, C.o, C.w.big_q,
-                                                                        C.w.qcap, C.w.big_n, num_sms(), info));
+                                                                        C.w.qcap, C.w.big_n, info));
     const int *cnt[3];
     int *off[3];
     for (int k = 0; k < C.naxes; ++k) {
@@ -637,7 +637,7 @@ int run_binned_fill(const float *verts, int64_t nv, const int32_t *tris, int64_t
     if (nt > 0)
         LDNI_LAUNCH(K_FILL_BIG, C.s,
                     big_pass<true><<<5 * num_sms(), kThreads, 0, C.s>>>(verts, tris, (int)nv, C.g, C.o, C.w.big_q,
-                                                                       C.w.qcap, C.w.big_n, num_sms(), info));
+                                                                       C.w.qcap, C.w.big_n, info));
     run_sort(C, info);
     return cuda_status();
 }

@@ -383,11 +383,8 @@ __device__ __forceinline__ void enqueue_big(Code *q, long long qcap, int *n, Cod
 // nblk / (huge pairs) blocks (at least one), each group sweeping its pairs
 // with all its threads, so that a few faces of hundreds of thousands of
 // pixels keep every SM busy and many huge faces run side by side.
-// huge_blocks is unused (kept for the callers' launch shapes).
 template <class Code, class F>
-__device__ __forceinline__ void for_each_big(const Code *q, long long qcap, const int *n, int blk, int nblk,
-                                             int huge_blocks, F &&body) {
-    (void)huge_blocks;
+__device__ __forceinline__ void for_each_big(const Code *q, long long qcap, const int *n, int blk, int nblk, F &&body) {
     const int nmed = n[0];
     int pt = 32;
     while (pt > kPairThreads && (long long)nmed * pt > (long long)nblk * blockDim.x) pt >>= 1;
