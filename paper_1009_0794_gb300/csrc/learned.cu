@@ -300,7 +300,9 @@ __global__ void __launch_bounds__(kCapWarps * 32) capacity_kernel(int ntiles, lo
 // crossed twice is entered once and left once, so the entering crossing
 // takes slot 0 and the leaving one slot 1 - no returned atomic, only counts.
 // The scan (csr_scan with ScanVerify) later sends every tile where some ray
-// broke that pattern to the exact redo.
+// broke that pattern to the exact redo; only there do the count words hold the
+// exits (with exits in every tile's words the two-at-a-time visit kept more
+// registers than it has: 75 against 65 us for 300,000 triangles at 1024^2).
 __device__ __forceinline__ void onepass_hit(int a, long long p, float d, int t, const float3 &n, int exiting,
                                             const LImg &o) {
     const int tile = (int)(p >> kTileBits);
@@ -311,7 +313,7 @@ __device__ __forceinline__ void onepass_hit(int a, long long p, float d, int t, 
         if (range_ok(slot, slot + 1, o.slab_cap, o.info)) o.slab[slot] = make_int2(__float_as_int(d), t);
         return;
     }
-    const int k = count_of(atomicAdd(pick3(o.count, a) + p, count_word(exiting)));
+    const int k = atomicAdd(pick3(o.count, a) + p, 1);
     if (k < kt) {
         const long long slot = pick3(o.slab_base, a)[tile] + (p & (kTilePix - 1)) * kt + k;
         if (range_ok(slot, slot + 1, o.slab_cap, o.info)) o.slab[slot] = make_int2(__float_as_int(d), t);
@@ -356,7 +358,7 @@ __device__ __forceinline__ void onepass_hits(const Setup32 &S, unsigned m, int t
             base[u] = v[u] ? sb[tile] : 0;
         }
 #pragma unroll
-        for (int u = 0; u < kHitBatch; ++u) k[u] = v[u] && kt[u] != 2 ? count_of(atomicAdd(cnt + pr[u], word)) : 0;
+        for (int u = 0; u < kHitBatch; ++u) k[u] = v[u] && kt[u] != 2 ? atomicAdd(cnt + pr[u], 1) : 0;
 #pragma unroll
         for (int u = 0; u < kHitBatch; ++u) {
             if (!v[u]) continue;
