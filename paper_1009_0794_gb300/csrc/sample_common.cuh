@@ -373,16 +373,28 @@ __device__ __forceinline__ void enqueue_big(Code *q, long long qcap, int *n, Cod
         q[atomicAdd(n, 1)] = code;
 }
 
-// Visit every queued pair with body(code, first, step), which walks the
-// pair's box with `step` threads.  Blocks blk of nblk: the medium pairs get a
-// warp each, or fewer threads, down to kPairThreads, when there are more pairs
-// than that leaves threads for (every thread of a pair repeats its loads and
-// setup, and waits for its own crossings' slots: 306,000 pairs of a batch of 48
-// meshes take 56 us (count) and 203 us (fill) with 4 threads each, 190 and 604
-// with 32); the huge pairs are shared out to groups of
-// nblk / (huge pairs) blocks (at least one), each group sweeping its pairs
-// with all its threads, so that a few faces of hundreds of thousands of
-// pixels keep every SM busy and many huge faces run side by side.
+// Visit every queued huge pair with body(code, first, step), which walks the
+// pair's box with `step` threads.  Blocks blk of nblk: the pairs are shared out
+// to groups of nblk / (huge pairs) blocks (at least one), each group sweeping
+// its pairs with all its threads, so that a few faces of hundreds of thousands
+// of pixels keep every SM busy and many huge faces run side by side.
+template <class Code, class F>
+__device__ __forceinline__ void for_each_huge(const Code *q, long long qcap, const int *n, int blk, int nblk, F &&body) {
+    const int nh = n[1];
+    if (nh <= 0) return;
+    const int G = max(1, nblk / nh);  // blocks per huge pair
+    const int groups = nblk / G, grp = blk / G, sub = blk - grp * G;
+    if (grp >= groups) return;  // the blocks left over when nblk is no multiple of G
+    for (int e = grp; e < nh; e += groups)
+        body(q[qcap - 1 - e], sub * (int)blockDim.x + (int)threadIdx.x, G * (int)blockDim.x);
+}
+
+// Visit every queued pair in the same way: the medium pairs get a warp each, or
+// fewer threads, down to kPairThreads, when there are more pairs than that
+// leaves threads for (every thread of a pair repeats its loads and setup, and
+// waits for its own crossings' slots: 306,000 pairs of a batch of 48 meshes take
+// 56 us (count) and 203 us (fill) with 4 threads each, 190 and 604 with 32; the
+// one-pass traversal's pairs of a 50,000-triangle sphere at 1280^2 164 and 549).
 template <class Code, class F>
 __device__ __forceinline__ void for_each_big(const Code *q, long long qcap, const int *n, int blk, int nblk, F &&body) {
     const int nmed = n[0];
@@ -391,13 +403,7 @@ __device__ __forceinline__ void for_each_big(const Code *q, long long qcap, cons
     const int gpb = blockDim.x / pt;
     for (int e = blk * gpb + (int)threadIdx.x / pt; e < nmed; e += nblk * gpb)
         body(q[e], (int)threadIdx.x & (pt - 1), pt);
-    const int nh = n[1];
-    if (nh <= 0) return;
-    const int G = max(1, nblk / nh);  // blocks per huge pair
-    const int groups = nblk / G, grp = blk / G, sub = blk - grp * G;
-    if (grp >= groups) return;  // the blocks left over when nblk is no multiple of G
-    for (int e = grp; e < nh; e += groups)
-        body(q[qcap - 1 - e], sub * (int)blockDim.x + (int)threadIdx.x, G * (int)blockDim.x);
+    for_each_huge(q, qcap, n, blk, nblk, body);
 }
 
 __device__ __forceinline__ bool key_less(float d0, int t0, float d1, int t1) {

@@ -162,3 +162,37 @@ def test_training_lowers_loss_and_beats_fixed_capacity(ldni, cap, small_net):
         slab_kmax += int(np.max(k_true)) * k_true.size
     assert over_net < over_k2
     assert slab_net < slab_kmax
+
+
+@pytest.mark.parametrize("mesh,res,layers", [
+    ("few tiles", 512, 2), ("few tiles", 512, 4), ("every tile", 320, 2), ("every tile", 1000, 2), ("huge", 700, 2),
+    ("narrow", 2100, 2)])
+def test_coarse_meshes_redo_their_big_pairs(ldni, mesh, res, layers):
+    """Meshes whose triangles cover many pixels, with tiles that hold more
+    layers than they were given: the pairs whose boxes reach a redone tile are
+    filled again, the others not, from boxes of a few rows to boxes of many
+    tiles and of more tiles than a pair is looked up in."""
+    if mesh == "few tiles":  # a ball, and a short stack of slabs above it
+        v0, t0 = M.icosphere(12, r=0.2, noise=0.03, seed=2)
+        v1, t1 = M.slab_stack(3, axis=1, seed=1, lo=0.3, hi=0.45)
+        v, t = np.concatenate([v0, (v1 * np.float32([0.2, 1, 0.2])).astype(np.float32)]), np.concatenate([t0, t1 + len(v0)])
+    elif mesh == "every tile":
+        v, t = M.flower(40, 40)
+    elif mesh == "huge":
+        v, t = M.slab_stack(4, axis=2, seed=3)
+    else:  # boxes a few pixels wide and most of the image long, one within another
+        bs = [M.box([-0.004 - 0.002 * k, -0.45, -0.004 - 0.002 * k], [0.004 + 0.002 * k, 0.45, 0.004 + 0.002 * k])
+              for k in range(3)]
+        v, t = np.concatenate([b[0] for b in bs]), np.concatenate([b[1] + 8 * k for k, b in enumerate(bs)])
+    mesh = (v.astype(np.float32), t.astype(np.int32))
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    ref = _exact(ldni, mesh, grid)
+    for packed in (False, True):
+        if packed:
+            ref = [L.numpy() for L in ldni.sample(*mesh, grid, "all", packed=True)]
+        got, n_over = _learned(ldni, mesh, grid, layers=layers, packed=packed)
+        assert n_over > 0 or layers > 2
+        for a in range(3):
+            assert all(np.array_equal(got[a][k].view(np.uint32) if got[a][k].dtype == np.float32 else got[a][k],
+                                      ref[a][k].view(np.uint32) if ref[a][k].dtype == np.float32 else ref[a][k])
+                       for k in ref[a]), a
