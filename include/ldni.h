@@ -213,7 +213,11 @@ int ldni_sample_count(const float *verts, int64_t nv, const int32_t *tris, int64
                       void *stream);
 
 /* Second half of ldni_sample (fill pass + per-ray sort + CSR write) after
- * ldni_sample_count on the same workspace, same inputs and same offsets. */
+ * ldni_sample_count on the same workspace, same inputs and same offsets.  Each
+ * fill needs a count of its own: a second one (say with larger arrays after
+ * LDNI_ST_CAPACITY), or one of a mesh with other crossings than were counted,
+ * sets LDNI_ST_CAPACITY and leaves rays without their samples, but writes no
+ * slot outside the ray that it belongs to. */
 int ldni_sample_fill(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, const ldni_grid_t *grid,
                      int32_t axis, ldni_layers_t *out, ldni_info_t *info, void *ws, size_t ws_bytes,
                      void *stream);

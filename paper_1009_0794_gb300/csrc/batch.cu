@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_big(const ldni_batch_item_t
         int *Tr = L.tri_id;
         const long long cap = L.capacity;
         sweep_box<kFillBatch>(S, i0, i1, j0, j1, first, step, [&](auto &v, auto &i, auto &j, auto depth) {
-            fill_batch(v, i, j, g.res, S.exiting, t, cnt, D, Tr, cap, infos + m, depth);
+            fill_batch(v, i, j, g.res, S.exiting, t, cnt, nullptr, D, Tr, cap, infos + m, depth);
         });
     });
 }

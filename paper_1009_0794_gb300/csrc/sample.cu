@@ -25,6 +25,12 @@
 // stored by the sort passes, ray after ray (79 us; 102 us when it had only the
 // swaps to do).
 //
+// A fill may meet other crossings than its count did: the two are separate
+// calls, and the cursors of a count serve one fill.  So no slot beyond its ray's
+// end is written (a pair's slots are its own, other rays' claims are held
+// against the next offset), and the crossings are counted once more: a fill
+// that did not see as many as the count reports LDNI_ST_CAPACITY.
+//
 // Triangles whose pixel box is large are handed to a block-per-triangle
 // kernel with 64-bit edge functions.
 #include <algorithm>
@@ -48,7 +54,17 @@ struct Img {
     float4 *nrm;            // per-triangle normals (x, y, z, packed codes)
     int nt;
     bool pairs8;            // every sample array 8-byte aligned
+    int *rest_n;            // listed runs of 32 rays left to sort_rest, and the list's length
+    int rest_cap;
+    unsigned *seen;         // [kSeen] crossings seen by fills since the count, in parts
 };
+constexpr int kSeen = 32;
+
+// Adds a warp's crossings to the fill's (whole warp).
+__device__ __forceinline__ void add_seen(const Img &o, unsigned seen) {
+    seen = __reduce_add_sync(0xffffffffu, seen);
+    if (seen && (threadIdx.x & 31) == 0) atomicAdd(o.seen + (blockIdx.x & (kSeen - 1)), seen);
+}
 
 __device__ __forceinline__ int *sel(int *const (&arr)[3], int a) { return a == 0 ? arr[0] : (a == 1 ? arr[1] : arr[2]); }
 
@@ -59,10 +75,11 @@ template <int A>
 __device__ __forceinline__ void fill_hits(const Setup32 &S, unsigned m, int t, const Img &o, int res, ldni_info_t *info) {
     const int wdiv = (256 + S.w - 1) / S.w;  // y = (b * wdiv) >> 8 = b / w for b < 16, w <= 16
     int *cur = o.count[A];
+    const int *off = o.offsets[A];
     const long long cap = o.cap[A];
     while (m) {
         int pr[2];
-        unsigned c[2];
+        unsigned c[2], end[2];
         float d[2];
         bool v[2];
 #pragma unroll
@@ -79,13 +96,19 @@ __device__ __forceinline__ void fill_hits(const Setup32 &S, unsigned m, int t, c
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
+            end[u] = 0xffffffffu;
             if (!v[u]) continue;
-            c[u] = c[u] & 0x80000000u ? (c[u] & 0x7fffffffu) + (unsigned)S.exiting : (unsigned)atomicAdd(cur + pr[u], 1);
+            if (c[u] & 0x80000000u) {
+                c[u] = (c[u] & 0x7fffffffu) + (unsigned)S.exiting;
+            } else {
+                c[u] = (unsigned)atomicAdd(cur + pr[u], 1);
+                end[u] = (unsigned)off[pr[u] + 1];
+            }
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             if (!v[u]) continue;
-            if ((long long)c[u] >= cap) {
+            if (c[u] >= end[u] || (long long)c[u] >= cap) {
                 set_status(info, LDNI_ST_CAPACITY);
                 continue;
             }
@@ -95,22 +118,25 @@ __device__ __forceinline__ void fill_hits(const Setup32 &S, unsigned m, int t, c
     }
 }
 
+// Returns the crossings filled.
 template <bool kFill, int A>
-__device__ __forceinline__ void tri_axis(const TriView &T, int t, const Img &o, int res, int *big_q, long long qcap,
-                                         int *big_n, ldni_info_t *info) {
+__device__ __forceinline__ int tri_axis(const TriView &T, int t, const Img &o, int res, int *big_q, long long qcap,
+                                        int *big_n, ldni_info_t *info) {
     Setup32 S;
     const int kind = setup_axis<A, kFill>(T, res, S);
-    if (kind == kNone) return;
+    if (kind == kNone) return 0;
     if (kind == kBig) {
         if (!kFill) enqueue_big(big_q, qcap, big_n, t * 4 + A, (long long)S.w * S.h);  // the fill pass reuses it
-        return;
+        return 0;
     }
     if (!kFill) {
         const int word = count_word(S.exiting);
         S.for_each_hit([&](int i, int j, int, int, int) { atomicAdd(o.count[A] + (long long)j * res + i, word); });
-        return;
+        return 0;
     }
-    fill_hits<A>(S, S.hit_bits(), t, o, res, info);
+    const unsigned m = S.hit_bits();
+    fill_hits<A>(S, m, t, o, res, info);
+    return __popc(m);
 }
 
 // Entry t of the per-triangle table.
@@ -128,6 +154,8 @@ __global__ void __launch_bounds__(kThreads) tri_pass(const float *__restrict__ v
                                                      int nt, int nv, GridDev g, int ax_lo, int ax_hi, Img o,
                                                      int *big_q, long long qcap, int *big_n, ldni_info_t *info) {
     if (gridDim.y > 1) ax_lo = ax_hi = ax_lo + (int)blockIdx.y;
+    if (kFill && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *o.rest_n = 0;  // sort_rays fills it anew
+    int seen = 0;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += gridDim.x * blockDim.x) {
         TriView T;
         const unsigned bad = load_tri(verts, tris, t, nv, g, T);
@@ -136,10 +164,11 @@ __global__ void __launch_bounds__(kThreads) tri_pass(const float *__restrict__ v
             continue;
         }
         if (kFill && blockIdx.y == 0) put_table(T, t, o);
-        if (ax_lo <= 0 && 0 <= ax_hi) tri_axis<kFill, 0>(T, t, o, g.res, big_q, qcap, big_n, info);
-        if (ax_lo <= 1 && 1 <= ax_hi) tri_axis<kFill, 1>(T, t, o, g.res, big_q, qcap, big_n, info);
-        if (ax_lo <= 2 && 2 <= ax_hi) tri_axis<kFill, 2>(T, t, o, g.res, big_q, qcap, big_n, info);
+        if (ax_lo <= 0 && 0 <= ax_hi) seen += tri_axis<kFill, 0>(T, t, o, g.res, big_q, qcap, big_n, info);
+        if (ax_lo <= 1 && 1 <= ax_hi) seen += tri_axis<kFill, 1>(T, t, o, g.res, big_q, qcap, big_n, info);
+        if (ax_lo <= 2 && 2 <= ax_hi) seen += tri_axis<kFill, 2>(T, t, o, g.res, big_q, qcap, big_n, info);
     }
+    if (kFill) add_seen(o, (unsigned)seen);
 }
 
 // The queued big (triangle, image) pairs (for_each_big), each swept by its
@@ -148,6 +177,7 @@ template <bool kFill>
 __global__ void __launch_bounds__(kThreads) big_pass(const float *__restrict__ verts, const int *__restrict__ tris,
                                                      int nv, GridDev g, Img o, const int *big_q, long long qcap,
                                                      const int *big_n, ldni_info_t *info) {
+    unsigned seen = 0;
     for_each_big(big_q, qcap, big_n, (int)blockIdx.x, (int)gridDim.x, [&](int code, int first, int step) {
         const int t = code >> 2, a = code & 3;
         TriView T;
@@ -166,10 +196,13 @@ __global__ void __launch_bounds__(kThreads) big_pass(const float *__restrict__ v
         float *D = a == 0 ? o.depth[0] : (a == 1 ? o.depth[1] : o.depth[2]);
         int *Tr = a == 0 ? o.tri[0] : (a == 1 ? o.tri[1] : o.tri[2]);
         const long long cap = a == 0 ? o.cap[0] : (a == 1 ? o.cap[1] : o.cap[2]);
+        const int *off = a == 0 ? o.offsets[0] : (a == 1 ? o.offsets[1] : o.offsets[2]);
         sweep_box<kFillBatch>(S, i0, i1, j0, j1, first, step, [&](auto &v, auto &i, auto &j, auto depth) {
-            fill_batch(v, i, j, g.res, S.exiting, t, cnt, D, Tr, cap, info, depth);
+            for (bool hit : v) seen += hit;
+            fill_batch(v, i, j, g.res, S.exiting, t, cnt, off, D, Tr, cap, info, depth);
         });
     });
+    if (kFill) add_seen(o, seen);
 }
 
 struct Image {  // one image's arrays
@@ -192,7 +225,7 @@ __device__ __forceinline__ Image image_of(const Img &o, int a) {
 // Per-ray ordering by (depth, tri_id) in place, and the samples' normals; also
 // flags odd rays.  A warp takes 32 consecutive rays; the runs with rays of
 // other than two samples are listed (image << 28 | run) for sort_rest.
-__global__ void __launch_bounds__(kThreads, 8) sort_rays(long long nrays, int ax_lo, Img o, int *rest, int *rest_n,
+__global__ void __launch_bounds__(kThreads, 8) sort_rays(long long nrays, int ax_lo, Img o, int *rest,
                                                          ldni_info_t *info) {
     const int a = ax_lo + blockIdx.y;
     const Image m = image_of(o, a);
@@ -202,16 +235,26 @@ __global__ void __launch_bounds__(kThreads, 8) sort_rays(long long nrays, int ax
          base += (long long)gridDim.x * blockDim.x) {
         long long b;
         const int n = ray_samples(m.off, base, nrays, m.cap, lane, true, info, b);
-        if (__any_sync(0xffffffffu, n != 0 && n != 2) && lane == 0) rest[atomicAdd(rest_n, 1)] = (a << 28) | (int)(base >> 5);
+        if (__any_sync(0xffffffffu, n != 0 && n != 2) && lane == 0) {
+            const int at = atomicAdd(o.rest_n, 1);
+            if (at < o.rest_cap) rest[at] = (a << 28) | (int)(base >> 5);
+        }
         if (n == 2) finish_pair(b, m.r, nrm, o.pairs8);
     }
 }
 
-__global__ void __launch_bounds__(kThreads) sort_rest(long long nrays, Img o, const int *rest, const int *rest_n,
+// (ax_lo, ax_hi: the images filled; as many crossings must have been met as their
+// offsets have room for.)
+__global__ void __launch_bounds__(kThreads) sort_rest(long long nrays, int ax_lo, int ax_hi, Img o, const int *rest,
                                                       ldni_info_t *info) {
     __shared__ SortStage stage[kThreads / 32];
-    const int lane = threadIdx.x & 31, warps = gridDim.x * (kThreads / 32);
-    for (int q = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); q < *rest_n; q += warps) {
+    const int lane = threadIdx.x & 31, warps = gridDim.x * (kThreads / 32), n_rest = min(*o.rest_n, o.rest_cap);
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        unsigned seen = __reduce_add_sync(0xffffffffu, o.seen[lane]);
+        for (int a = ax_lo; a <= ax_hi; ++a) seen -= (unsigned)image_of(o, a).off[nrays];
+        if (lane == 0 && seen != 0u) set_status(info, LDNI_ST_CAPACITY);
+    }
+    for (int q = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); q < n_rest; q += warps) {
         const int code = rest[q];
         const Image m = image_of(o, code >> 28);
         long long b;
@@ -349,10 +392,13 @@ __global__ void __launch_bounds__(kThreads) tile_pass(const float *__restrict__ 
     const long long p = (long long)j * g.res + i;
     int found = 0;          // count: the word so far; fill: the crossings so far
     unsigned cursor = 0;
-    long long cap = 0;
+    long long cap = 0;      // the slots end here
+    if (kFill && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *o.rest_n = 0;  // sort_rays fills it anew
     if (kFill && mine) {
         cursor = (unsigned)sel(o.count, a)[p];
         cap = a == 0 ? o.cap[0] : (a == 1 ? o.cap[1] : o.cap[2]);
+        const int *off = a == 0 ? o.offsets[0] : (a == 1 ? o.offsets[1] : o.offsets[2]);
+        if (!(cursor >> 31)) cap = min(cap, (long long)off[p + 1]);  // (a pair's slots are its own)
     }
     for (int k0 = 0; k0 < n; k0 += kTileStage) {
         const int k = k0 + threadIdx.x;
@@ -394,6 +440,7 @@ __global__ void __launch_bounds__(kThreads) tile_pass(const float *__restrict__ 
         }
         __syncthreads();
     }
+    if (kFill) add_seen(o, (unsigned)found);
     if (!mine) return;
     if (!kFill)
         sel(o.count, a)[p] = found;  // the big pairs add theirs afterwards
@@ -403,8 +450,9 @@ __global__ void __launch_bounds__(kThreads) tile_pass(const float *__restrict__ 
 
 struct SampleWs {
     int *count[3];
-    int *big_n;          // two queue counts and rest's right after the counts: one memset clears all
+    int *big_n;          // two queue counts, rest's and the fill's right after the counts: one memset clears all
     int *rest;           // runs of 32 rays left to sort_rest
+    long long rest_cap;
     long long qcap;
     size_t clear_bytes;
     long long *scan_words;
@@ -416,11 +464,12 @@ SampleWs carve_sample_ws(Carver &c, long long nt, int res, int naxes) {
     SampleWs w{};
     const long long N = (long long)res * res;
     const long long stride = (N + 63) / 64 * 64;  // every image's counts start 256-byte aligned
-    int *block = c.take<int>((size_t)(stride * naxes + 3));
+    int *block = c.take<int>((size_t)(stride * naxes + 3 + kSeen));
     for (int a = 0; a < naxes; ++a) w.count[a] = block ? block + (size_t)a * stride : nullptr;
     w.big_n = block ? block + (size_t)stride * naxes : nullptr;
-    w.clear_bytes = sizeof(int) * (size_t)(stride * naxes + 3);
-    w.rest = c.take<int>((size_t)((N + 31) / 32 * naxes));
+    w.clear_bytes = sizeof(int) * (size_t)(stride * naxes + 3 + kSeen);
+    w.rest_cap = (N + 31) / 32 * naxes;
+    w.rest = c.take<int>((size_t)w.rest_cap);
     w.scan_words = c.take<long long>(csr_scan_partials(N) * naxes);
     w.qcap = nt * naxes > 0 ? nt * naxes : 1;
     w.big_q = c.take<int>((size_t)w.qcap);
@@ -457,6 +506,9 @@ int prepare(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, con
     C.o = Img{};
     C.o.nrm = w.nrm;
     C.o.nt = (int)nt;
+    C.o.rest_n = w.big_n + 2;
+    C.o.rest_cap = (int)w.rest_cap;
+    C.o.seen = reinterpret_cast<unsigned *>(w.big_n + 3);
     C.o.pairs8 = true;
     for (int k = 0; k < C.naxes; ++k) {
         const int a = C.ax_lo + k;
@@ -516,14 +568,13 @@ int run_count(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, c
 }
 
 void run_sort(const Call &C, ldni_info_t *info) {
-    int *rest_n = C.w.big_n + 2;
     LDNI_LAUNCH(K_SORT, C.s,
                 sort_rays<<<dim3(grid_blocks(C.nrays), C.naxes), kThreads, 0, C.s>>>(C.nrays, C.ax_lo, C.o, C.w.rest,
-                                                                                    rest_n, info));
+                                                                                    info));
     const long long runs = (C.nrays + 31) / 32 * C.naxes, blocks = (runs + kThreads / 32 - 1) / (kThreads / 32);
     LDNI_LAUNCH(K_SORT, C.s,
-                sort_rest<<<(unsigned)std::min(blocks, 3ll * num_sms()), kThreads, 0, C.s>>>(C.nrays, C.o, C.w.rest,
-                                                                                           rest_n, info));
+                sort_rest<<<(unsigned)std::min(blocks, 3ll * num_sms()), kThreads, 0, C.s>>>(
+                    C.nrays, C.ax_lo, C.ax_hi, C.o, C.w.rest, info));
 }
 
 int run_fill(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, const Call &C, ldni_info_t *info) {

@@ -337,23 +337,33 @@ __device__ __forceinline__ void sweep_box(const Setup64 &S, int i0, int i1, int 
 }
 
 // The fill pass's visit of the crossings among kN pixels of one face: all their
-// cursors are in flight before any sample is stored.
+// cursors are in flight before any sample is stored.  off: the image's offsets,
+// when a claimed slot has to be held against its ray's end (a fill that may see
+// other crossings than its count did), else null.
 constexpr int kFillBatch = 4;
 template <int kN, class Depth>
-__device__ __forceinline__ void fill_batch(const bool (&v)[kN], const int (&i)[kN], const int (&j)[kN], int res, int exiting, int t, int *cur, float *D,
-                                           int *Tr, long long cap, ldni_info_t *info, Depth depth) {
-    unsigned c[kN];
+__device__ __forceinline__ void fill_batch(const bool (&v)[kN], const int (&i)[kN], const int (&j)[kN], int res,
+                                           int exiting, int t, int *cur, const int *off, float *D, int *Tr,
+                                           long long cap, ldni_info_t *info, Depth depth) {
+    unsigned c[kN], end[kN];
 #pragma unroll
     for (int u = 0; u < kN; ++u) c[u] = v[u] ? (unsigned)cur[(long long)j[u] * res + i[u]] : 0u;
 #pragma unroll
-    for (int u = 0; u < kN; ++u)
-        if (v[u])
-            c[u] = c[u] & 0x80000000u ? (c[u] & 0x7fffffffu) + (unsigned)exiting
-                                      : (unsigned)atomicAdd(cur + (long long)j[u] * res + i[u], 1);
+    for (int u = 0; u < kN; ++u) {
+        end[u] = 0xffffffffu;
+        if (!v[u]) continue;
+        const long long p = (long long)j[u] * res + i[u];
+        if (c[u] & 0x80000000u) {
+            c[u] = (c[u] & 0x7fffffffu) + (unsigned)exiting;
+        } else {
+            c[u] = (unsigned)atomicAdd(cur + p, 1);
+            if (off) end[u] = (unsigned)off[p + 1];
+        }
+    }
 #pragma unroll
     for (int u = 0; u < kN; ++u) {
         if (!v[u]) continue;
-        if ((long long)c[u] >= cap) {
+        if (c[u] >= end[u] || (long long)c[u] >= cap) {
             set_status(info, LDNI_ST_CAPACITY);
             continue;
         }

@@ -206,3 +206,108 @@ def test_max_resolution_sampled_rays(ldni):
     assert np.all(np.diff(off) % 2 == 0)
     ref = oracle.sample(v, t, grid.origin, 1.0, res, 1, "scan")
     assert np.array_equal(off, ref["offsets"])
+
+
+def _count_then_fill(ldni, binned, first, second, grid, fills, fresh=False):
+    """ldni_sample_count of mesh `first`, then `fills` times ldni_sample_fill of
+    mesh `second` on the same workspace and offsets (fresh: the last one into
+    arrays of its own).  Returns the images and each fill's status; the bytes
+    around the workspace and past the arrays are checked."""
+    import ctypes
+    from paper_1009_0794_gb300 import _lib
+    lib = _lib.load()
+    count = lib.ldni_sample_binned_count if binned else lib.ldni_sample_count
+    fill = lib.ldni_sample_binned_fill if binned else lib.ldni_sample_fill
+    size = ldni.sample_binned_workspace_size if binned else ldni.sample_workspace_size
+    up = lambda m: (torch.from_numpy(m[0]).cuda(), torch.from_numpy(m[1]).cuda())
+    (v, t), (v2, t2) = up(first), up(second)
+    assert t.shape == t2.shape
+    need = size(len(v), len(t), grid.res, "all")
+    buf = torch.full((need + (1 << 20),), 0x5A, dtype=torch.uint8, device="cuda")
+    ws, past = buf[:need], buf[need:]
+    info, g = ldni.new_info(), grid.c()
+    offsets = [torch.zeros(grid.res ** 2 + 1, dtype=torch.int32, device="cuda") for _ in range(3)]
+    arr = (_lib.Layers * 3)(*[_lib.Layers(o.data_ptr()) for o in offsets])
+    args = lambda v, t, arr: (v.data_ptr(), len(v), t.data_ptr(), len(t), ctypes.byref(g), 3, arr, info.data_ptr(),
+                              ws.data_ptr(), need, None)
+    torch.cuda.synchronize()
+    assert count(*args(v, t, arr)) == 0
+    n = [int(x) for x in info[:3].tolist()]
+    slack = 1000  # never written: the arrays end at the count
+
+    def arrays(a):
+        f = lambda x: torch.full((n[a] + slack,), x, dtype=torch.float32, device="cuda")
+        return ldni.LDNI(grid, a, offsets[a], f(-7.0), f(-7.0), f(-7.0), f(-7.0),
+                         torch.full((n[a] + slack,), -1, dtype=torch.int32, device="cuda"), n[a])
+
+    outs, status = [arrays(a) for a in range(3)], []
+    for k in range(fills):
+        if fresh and k == fills - 1:
+            outs = [arrays(a) for a in range(3)]
+        info.zero_()
+        arr = (_lib.Layers * 3)(*[o.c() for o in outs])
+        torch.cuda.synchronize()
+        assert fill(*args(v2, t2, arr)) == 0
+        torch.cuda.synchronize()
+        status.append(int(info[3].item()) & 0xFFFFFFFF)
+    assert bool((past == 0x5A).all())
+    for L in outs:
+        for x in (L.depth, L.nx, L.ny, L.nz):
+            assert bool((x[L.n:] == -7.0).all())
+        assert bool((L.tri[L.n:] == -1).all())
+    return outs, status
+
+
+@pytest.mark.parametrize("binned", [False, True])
+@pytest.mark.parametrize("mesh,res", [("box", 700), ("ball", 96), ("slabs", 65), ("flower", 200)])
+def test_a_second_fill_is_reported_and_stays_in_place(ldni, binned, mesh, res):
+    """The cursors of a count serve one fill: further ones report
+    LDNI_ST_CAPACITY, leave the first one's samples as they are, and write
+    nothing past the workspace (few triangles, many rays: the list of runs is
+    its largest part) or outside a ray of the arrays."""
+    from paper_1009_0794_gb300 import _lib
+    m = {"box": M.box([-0.4, -0.3, -0.2], [0.3, 0.35, 0.4]), "ball": M.icosphere(8, r=0.4, noise=0.05, seed=1),
+         "slabs": M.slab_stack(9, axis=1, seed=2), "flower": M.flower(60, 60)}[mesh]
+    grid = ldni.Grid.cube((-0.5, -0.5, -0.5), 1.0, res)
+    ref = ldni.sample(*m, grid, "all")
+    outs, status = _count_then_fill(ldni, binned, m, m, grid, 4)
+    assert not status[0] & _lib.ST_CAPACITY and all(s & _lib.ST_CAPACITY for s in status[1:])
+    assert all(ldni.identical(x, y) for x, y in zip(outs, ref))
+    outs, status = _count_then_fill(ldni, binned, m, m, grid, 3, fresh=True)
+    assert status[2] & _lib.ST_CAPACITY
+    _check_rays(outs, ref)
+
+
+def _check_rays(outs, ref):
+    """Every slot holds a sample of its own ray, or none (id -1)."""
+    for L, R in zip(outs, ref):
+        ray = np.repeat(np.arange(L.grid.res ** 2), np.diff(L.offsets.cpu().numpy()))
+        rray = np.repeat(np.arange(L.grid.res ** 2), np.diff(R.offsets.cpu().numpy()))
+        key = lambda r, t: r.astype(np.int64) << 32 | t.astype(np.int64)
+        tri = L.tri[:L.n].cpu().numpy()
+        have = key(ray, tri)[tri >= 0]
+        assert np.isin(have, key(rray, R.tri[:R.n].cpu().numpy())).all(), L.axis
+
+
+@pytest.mark.parametrize("binned", [False, True])
+@pytest.mark.parametrize("change", ["wider", "twice", "fewer", "deeper"])
+def test_a_fill_of_another_mesh_is_reported(ldni, binned, change):
+    """More crossings than were counted (new rays, more per ray, on rays that
+    were pairs and on others) or fewer: reported, and no slot of another ray
+    is written."""
+    from paper_1009_0794_gb300 import _lib
+    def join(*ms):
+        at = np.cumsum([0] + [len(m[0]) for m in ms[:-1]])
+        return (np.concatenate([m[0] for m in ms]).astype(np.float32),
+                np.concatenate([m[1] + k for m, k in zip(ms, at)]).astype(np.int32))
+    A, T = M.box([-0.4, -0.3, -0.2], [0.3, 0.35, 0.4]), M.box([0.41, 0.41, 0.41], [0.42, 0.42, 0.42])
+    one, two = join(A, T), join(A, A)
+    S = M.slab_stack(7, axis=0, seed=5)
+    W = ((S[0] * np.float32([1, 1.15, 0.9])).astype(np.float32), S[1])
+    first, second = {"wider": (one, (one[0] * np.float32(1.1), one[1])), "twice": (one, two), "fewer": (two, one),
+                     "deeper": (S, W)}[change]
+    grid = ldni.Grid.cube((-0.5, -0.5, -0.5), 1.0, 90)
+    ref = ldni.sample(*second, grid, "all")
+    outs, status = _count_then_fill(ldni, binned, first, second, grid, 1)
+    assert status[0] & _lib.ST_CAPACITY
+    _check_rays(outs, ref)
