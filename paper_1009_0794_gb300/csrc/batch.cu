@@ -333,7 +333,7 @@ __device__ __forceinline__ ItemImage item_image(const ldni_batch_item_t *items, 
     I.off = L.offsets;
     I.r = L.nrm8 ? RayOut{L.depth, L.tri_id, reinterpret_cast<float *>(L.nrm8), nullptr, nullptr}
                  : RayOut{L.depth, L.tri_id, L.nx, L.ny, L.nz};
-    I.nrm = NormalTable{T.nrm + T.tri_prefix[m], (int)items[m].nt};
+    I.nrm = NormalTable{T.nrm + T.tri_prefix[m], (int)items[m].nt, false};
     I.cap = L.capacity;
     I.N = (long long)items[m].grid.res * items[m].grid.res;
     I.pairs8 = ((reinterpret_cast<uintptr_t>(I.r.D) | reinterpret_cast<uintptr_t>(I.r.Tr) |

@@ -53,6 +53,7 @@ struct Img {
     long long cap[3];
     float4 *nrm;            // per-triangle normals (x, y, z, packed codes)
     int nt;
+    bool codes;             // ... of the codes alone
     bool pairs8;            // every sample array 8-byte aligned
     int *rest_n;            // listed runs of 32 rays left to sort_rest, and the list's length
     int rest_cap;
@@ -143,42 +144,44 @@ __device__ __forceinline__ int tri_axis(const TriView &T, int t, const Img &o, i
 __device__ __forceinline__ void put_table(const TriView &T, int t, const Img &o) {
     float3 n;
     face_normal(T.p[0], T.p[1], T.p[2], n.x, n.y, n.z);
-    o.nrm[t] = make_float4(n.x, n.y, n.z, __uint_as_float(encode_normal8(n.x, n.y, n.z)));
+    const float code = __uint_as_float(encode_normal8(n.x, n.y, n.z));
+    if (o.codes)
+        reinterpret_cast<float *>(o.nrm)[t] = code;
+    else
+        o.nrm[t] = make_float4(n.x, n.y, n.z, code);
 }
 
-// One thread per triangle; big triangles are queued (count pass) for big_pass.
-// With gridDim.y > 1 a thread takes its triangle on one image, ax_lo +
-// blockIdx.y, only (spread_images).
+// Triangles of blocks blk of nblk, a thread each; big ones are queued (count
+// pass).  A block takes its triangles on images ax_lo .. ax_hi.  Returns the
+// thread's crossings (fill pass).
 template <bool kFill>
-__global__ void __launch_bounds__(kThreads) tri_pass(const float *__restrict__ verts, const int *__restrict__ tris,
-                                                     int nt, int nv, GridDev g, int ax_lo, int ax_hi, Img o,
-                                                     int *big_q, long long qcap, int *big_n, ldni_info_t *info) {
-    if (gridDim.y > 1) ax_lo = ax_hi = ax_lo + (int)blockIdx.y;
-    if (kFill && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *o.rest_n = 0;  // sort_rays fills it anew
+__device__ __forceinline__ int tri_blocks(const float *__restrict__ verts, const int *__restrict__ tris, int nt, int nv,
+                                          const GridDev &g, int ax_lo, int ax_hi, const Img &o, int *big_q,
+                                          long long qcap, int *big_n, ldni_info_t *info, int blk, int nblk, bool table) {
     int seen = 0;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += gridDim.x * blockDim.x) {
+    for (int t = blk * blockDim.x + threadIdx.x; t < nt; t += nblk * blockDim.x) {
         TriView T;
         const unsigned bad = load_tri(verts, tris, t, nv, g, T);
         if (bad) {
             if (!kFill) set_status(info, bad);
             continue;
         }
-        if (kFill && blockIdx.y == 0) put_table(T, t, o);
+        if (table) put_table(T, t, o);
         if (ax_lo <= 0 && 0 <= ax_hi) seen += tri_axis<kFill, 0>(T, t, o, g.res, big_q, qcap, big_n, info);
         if (ax_lo <= 1 && 1 <= ax_hi) seen += tri_axis<kFill, 1>(T, t, o, g.res, big_q, qcap, big_n, info);
         if (ax_lo <= 2 && 2 <= ax_hi) seen += tri_axis<kFill, 2>(T, t, o, g.res, big_q, qcap, big_n, info);
     }
-    if (kFill) add_seen(o, (unsigned)seen);
+    return seen;
 }
 
 // The queued big (triangle, image) pairs (for_each_big), each swept by its
-// threads.
+// threads, on blocks blk of nblk.  Returns the thread's crossings (fill pass).
 template <bool kFill>
-__global__ void __launch_bounds__(kThreads) big_pass(const float *__restrict__ verts, const int *__restrict__ tris,
-                                                     int nv, GridDev g, Img o, const int *big_q, long long qcap,
-                                                     const int *big_n, ldni_info_t *info) {
+__device__ __forceinline__ unsigned big_blocks(const float *__restrict__ verts, const int *__restrict__ tris, int nv,
+                                               const GridDev &g, const Img &o, const int *big_q, long long qcap,
+                                               const int *big_n, ldni_info_t *info, int blk, int nblk) {
     unsigned seen = 0;
-    for_each_big(big_q, qcap, big_n, (int)blockIdx.x, (int)gridDim.x, [&](int code, int first, int step) {
+    for_each_big(big_q, qcap, big_n, blk, nblk, [&](int code, int first, int step) {
         const int t = code >> 2, a = code & 3;
         TriView T;
         if (load_tri(verts, tris, t, nv, g, T)) return;
@@ -202,7 +205,44 @@ __global__ void __launch_bounds__(kThreads) big_pass(const float *__restrict__ v
             fill_batch(v, i, j, g.res, S.exiting, t, cnt, off, D, Tr, cap, info, depth);
         });
     });
+    return seen;
+}
+
+// The count pass's triangles.  With gridDim.y > 1 a thread takes its triangle on
+// one image, ax_lo + blockIdx.y, only (tri_grid).
+__global__ void __launch_bounds__(kThreads) count_tri(const float *__restrict__ verts, const int *__restrict__ tris,
+                                                      int nt, int nv, GridDev g, int ax_lo, int ax_hi, Img o, int *big_q,
+                                                      long long qcap, int *big_n, ldni_info_t *info) {
+    if (gridDim.y > 1) ax_lo = ax_hi = ax_lo + (int)blockIdx.y;
+    tri_blocks<false>(verts, tris, nt, nv, g, ax_lo, ax_hi, o, big_q, qcap, big_n, info, (int)blockIdx.x,
+                      (int)gridDim.x, false);
+}
+
+template <bool kFill>
+__global__ void __launch_bounds__(kThreads) big_pass(const float *__restrict__ verts, const int *__restrict__ tris,
+                                                     int nv, GridDev g, Img o, const int *big_q, long long qcap,
+                                                     const int *big_n, ldni_info_t *info) {
+    const unsigned seen = big_blocks<kFill>(verts, tris, nv, g, o, big_q, qcap, big_n, info, (int)blockIdx.x,
+                                            (int)gridDim.x);
     if (kFill) add_seen(o, seen);
+}
+
+// The fill pass: the count has left the whole queue, so its pairs are filled
+// beside the triangles, on the first `nbig` blocks.
+__global__ void __launch_bounds__(kThreads, 4) fill_pass(const float *__restrict__ verts, const int *__restrict__ tris,
+                                                         int nt, int nv, GridDev g, int ax_lo, int ax_hi, int nbig, Img o,
+                                                         int *big_q, long long qcap, int *big_n, ldni_info_t *info) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *o.rest_n = 0;  // sort_rays fills it anew
+    unsigned seen = 0;
+    if ((int)blockIdx.x < nbig) {
+        if (blockIdx.y != 0 || big_n[0] + big_n[1] == 0) return;
+        seen = big_blocks<true>(verts, tris, nv, g, o, big_q, qcap, big_n, info, (int)blockIdx.x, nbig);
+    } else {
+        if (gridDim.y > 1) ax_lo = ax_hi = ax_lo + (int)blockIdx.y;
+        seen = tri_blocks<true>(verts, tris, nt, nv, g, ax_lo, ax_hi, o, big_q, qcap, big_n, info,
+                                (int)blockIdx.x - nbig, (int)gridDim.x - nbig, blockIdx.y == 0);
+    }
+    add_seen(o, seen);
 }
 
 struct Image {  // one image's arrays
@@ -224,42 +264,66 @@ __device__ __forceinline__ Image image_of(const Img &o, int a) {
 
 // Per-ray ordering by (depth, tri_id) in place, and the samples' normals; also
 // flags odd rays.  A warp takes 32 consecutive rays; the runs with rays of
-// other than two samples are listed (image << 28 | run) for sort_rest.
+// more than four samples are listed (image << 28 | run) for sort_rest.  (Rays of
+// up to four here: torus of 1.2 M triangles at 1900^2 298 -> 283 us a call; spilled
+// registers that cost the sphere, whose rays are all pairs, 5 us of 331.)
 __global__ void __launch_bounds__(kThreads, 8) sort_rays(long long nrays, int ax_lo, Img o, int *rest,
                                                          ldni_info_t *info) {
     const int a = ax_lo + blockIdx.y;
     const Image m = image_of(o, a);
-    const NormalTable nrm{o.nrm, o.nt};
+    const NormalTable nrm{o.nrm, o.nt, o.codes};
     const int lane = threadIdx.x & 31;
     for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); base < nrays;
          base += (long long)gridDim.x * blockDim.x) {
         long long b;
         const int n = ray_samples(m.off, base, nrays, m.cap, lane, true, info, b);
-        if (__any_sync(0xffffffffu, n != 0 && n != 2) && lane == 0) {
+        if (__any_sync(0xffffffffu, n > 4) && lane == 0) {
             const int at = atomicAdd(o.rest_n, 1);
             if (at < o.rest_cap) rest[at] = (a << 28) | (int)(base >> 5);
         }
         if (n == 2) finish_pair(b, m.r, nrm, o.pairs8);
+        else if (n > 0 && n <= 4) finish_few(b, n, m.r, nrm);
     }
 }
 
-// (ax_lo, ax_hi: the images filled; as many crossings must have been met as their
-// offsets have room for.)
+// As many crossings must have been met as the offsets have room for (a warp).
+__device__ __forceinline__ void check_seen(long long nrays, int ax_lo, int ax_hi, const Img &o, ldni_info_t *info) {
+    const int lane = threadIdx.x & 31;
+    unsigned seen = __reduce_add_sync(0xffffffffu, o.seen[lane]);
+    for (int a = ax_lo; a <= ax_hi; ++a) seen -= (unsigned)image_of(o, a).off[nrays];
+    if (lane == 0 && seen != 0u) set_status(info, LDNI_ST_CAPACITY);
+}
+
 __global__ void __launch_bounds__(kThreads) sort_rest(long long nrays, int ax_lo, int ax_hi, Img o, const int *rest,
                                                       ldni_info_t *info) {
     __shared__ SortStage stage[kThreads / 32];
     const int lane = threadIdx.x & 31, warps = gridDim.x * (kThreads / 32), n_rest = min(*o.rest_n, o.rest_cap);
-    if (blockIdx.x == 0 && threadIdx.x < 32) {
-        unsigned seen = __reduce_add_sync(0xffffffffu, o.seen[lane]);
-        for (int a = ax_lo; a <= ax_hi; ++a) seen -= (unsigned)image_of(o, a).off[nrays];
-        if (lane == 0 && seen != 0u) set_status(info, LDNI_ST_CAPACITY);
-    }
+    if (blockIdx.x == 0 && threadIdx.x < 32) check_seen(nrays, ax_lo, ax_hi, o, info);
     for (int q = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); q < n_rest; q += warps) {
         const int code = rest[q];
         const Image m = image_of(o, code >> 28);
         long long b;
         const int n = ray_samples(m.off, (long long)(code & 0xfffffff) << 5, nrays, m.cap, lane, false, info, b);
-        finish_rest(b, n == 2 ? 0 : n, m.r, NormalTable{o.nrm, o.nt}, stage[threadIdx.x >> 5], lane);
+        finish_rest(b, n <= 4 ? 0 : n, m.r, NormalTable{o.nrm, o.nt, o.codes}, stage[threadIdx.x >> 5], lane);
+    }
+}
+
+// Both in one kernel, for images of few rays (kSmallSort).
+__global__ void __launch_bounds__(kThreads, 4) sort_small(long long nrays, int ax_lo, Img o, ldni_info_t *info) {
+    __shared__ SortStage stage[kThreads / 32];
+    const int a = ax_lo + blockIdx.y;
+    const Image m = image_of(o, a);
+    const NormalTable nrm{o.nrm, o.nt, o.codes};
+    const int lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32)
+        check_seen(nrays, ax_lo, ax_lo + (int)gridDim.y - 1, o, info);
+    for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); base < nrays;
+         base += (long long)gridDim.x * blockDim.x) {
+        long long b;
+        const int n = ray_samples(m.off, base, nrays, m.cap, lane, true, info, b);
+        if (n == 2) finish_pair(b, m.r, nrm, o.pairs8);
+        if (__any_sync(0xffffffffu, n != 0 && n != 2))
+            finish_rest(b, n == 2 ? 0 : n, m.r, nrm, stage[threadIdx.x >> 5], lane);
     }
 }
 
@@ -545,13 +609,20 @@ dim3 tri_grid(long long nt, int naxes) {
     return dim3((unsigned)grid_blocks(nt), spread ? (unsigned)naxes : 1u);
 }
 
+// Rays up to which the order is made in one kernel: below it the second launch
+// costs more than the registers of the long rays' path, above it less.  us a
+// call in one kernel and in two: 30,000-triangle torus 56 and 62 at 400^2 (three
+// images), 87 and 91 at 700^2, 120 and 117 at 1000^2; 300,000-triangle sphere 57
+// and 60, 87 and 87, 124 and 118.
+constexpr long long kSmallSort = 2000000;
+
 int run_count(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, const Call &C, ldni_info_t *info) {
     if (int rc_ = cuda_check(cudaMemsetAsync(C.w.count[0], 0, C.w.clear_bytes, C.s))) return rc_;
     if (nt > 0) {
         LDNI_LAUNCH(K_COUNT_TRI, C.s,
-                    tri_pass<false><<<tri_grid(nt, C.naxes), kThreads, 0, C.s>>>(verts, tris, (int)nt, (int)nv, C.g,
-                                                                          C.ax_lo, C.ax_hi, C.o, C.w.big_q,
-                                                                          C.w.qcap, C.w.big_n, info));
+                    count_tri<<<tri_grid(nt, C.naxes), kThreads, 0, C.s>>>(verts, tris, (int)nt, (int)nv, C.g, C.ax_lo,
+                                                                          C.ax_hi, C.o, C.w.big_q, C.w.qcap,
+                                                                          C.w.big_n, info));
         LDNI_LAUNCH(K_COUNT_BIG, C.s,
                     big_pass<false><<<5 * num_sms(), kThreads, 0, C.s>>>(verts, tris, (int)nv, C.g, C.o, C.w.big_q,
                                                                         C.w.qcap, C.w.big_n, info));
@@ -568,6 +639,11 @@ int run_count(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, c
 }
 
 void run_sort(const Call &C, ldni_info_t *info) {
+    if (C.nrays * C.naxes <= kSmallSort) {
+        LDNI_LAUNCH(K_SORT, C.s,
+                    sort_small<<<dim3(grid_blocks(C.nrays), C.naxes), kThreads, 0, C.s>>>(C.nrays, C.ax_lo, C.o, info));
+        return;
+    }
     LDNI_LAUNCH(K_SORT, C.s,
                 sort_rays<<<dim3(grid_blocks(C.nrays), C.naxes), kThreads, 0, C.s>>>(C.nrays, C.ax_lo, C.o, C.w.rest,
                                                                                     info));
@@ -577,15 +653,26 @@ void run_sort(const Call &C, ldni_info_t *info) {
                     C.nrays, C.ax_lo, C.ax_hi, C.o, C.w.rest, info));
 }
 
-int run_fill(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, const Call &C, ldni_info_t *info) {
+int run_fill(const float *verts, int64_t nv, const int32_t *tris, int64_t nt, Call &C, ldni_info_t *info) {
+    // images that all take packed normals need a table of the codes alone (16 -> 4 bytes a triangle)
+    C.o.codes = true;
+    for (int a = C.ax_lo; a <= C.ax_hi; ++a) C.o.codes &= C.o.ny[a] == nullptr;
     if (nt > 0) {
+        // Beside the triangles, which saves a launch (4 to 6 us a call) and overlaps the two (300,000
+        // triangles at 1900^2: 468 -> 412 us a call), except in large images of meshes whose mean face
+        // covers a huge box: their pairs take whole blocks, and longer in this kernel's registers (1,000
+        // triangles at 1900^2: 131 and 119 us).
+        const bool beside = C.nrays <= (long long)kHugePixels * nt || C.nrays * C.naxes <= kSmallSort;
+        const int nbig = beside ? 5 * num_sms() : 0;
+        dim3 grid = tri_grid(nt, C.naxes);
+        grid.x += (unsigned)nbig;
         LDNI_LAUNCH(K_FILL_TRI, C.s,
-                    tri_pass<true><<<tri_grid(nt, C.naxes), kThreads, 0, C.s>>>(verts, tris, (int)nt, (int)nv, C.g,
-                                                                         C.ax_lo, C.ax_hi, C.o, C.w.big_q,
-                                                                         C.w.qcap, C.w.big_n, info));
-        LDNI_LAUNCH(K_FILL_BIG, C.s,
-                    big_pass<true><<<5 * num_sms(), kThreads, 0, C.s>>>(verts, tris, (int)nv, C.g, C.o, C.w.big_q,
-                                                                       C.w.qcap, C.w.big_n, info));
+                    fill_pass<<<grid, kThreads, 0, C.s>>>(verts, tris, (int)nt, (int)nv, C.g, C.ax_lo, C.ax_hi, nbig,
+                                                          C.o, C.w.big_q, C.w.qcap, C.w.big_n, info));
+        if (!beside)
+            LDNI_LAUNCH(K_FILL_BIG, C.s,
+                        big_pass<true><<<5 * num_sms(), kThreads, 0, C.s>>>(verts, tris, (int)nv, C.g, C.o, C.w.big_q,
+                                                                           C.w.qcap, C.w.big_n, info));
     }
     run_sort(C, info);
     return cuda_status();

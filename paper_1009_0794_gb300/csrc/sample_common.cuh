@@ -489,13 +489,17 @@ struct RayOut {
     float *X, *Y, *Z;  // FP32 normals, or packed 8-bit normals in X with Y = Z = nullptr
 };
 
-// Unit normals of a mesh's triangles, w: packed 8-bit codes.  An index outside
-// the mesh (a slot that no crossing filled: the mesh changed between count and
-// fill) reads as triangle 0.
+// Unit normals of a mesh's triangles, w: packed 8-bit codes, or a table of the
+// codes alone (codes).  An index outside the mesh (a slot that no crossing
+// filled: the mesh changed between count and fill) reads as triangle 0.
 struct NormalTable {
     const float4 *n;
     int nt;
-    __device__ __forceinline__ float4 operator()(int t) const { return n[(unsigned)t < (unsigned)nt ? t : 0]; }
+    bool codes;
+    __device__ __forceinline__ float4 operator()(int t) const {
+        const int at = (unsigned)t < (unsigned)nt ? t : 0;
+        return codes ? make_float4(0.0f, 0.0f, 0.0f, reinterpret_cast<const float *>(n)[at]) : n[at];
+    }
 };
 
 __device__ __forceinline__ void put_normal(const RayOut &o, long long at, const float4 &q) {
@@ -729,12 +733,12 @@ __device__ __forceinline__ void order_flat(long long b, int n, const RayOut &r, 
 // ---- ordering of samples that were filled without normals -----------------------------
 //
 // Two kernels order every ray and give its samples their normals: one for rays
-// of two samples, nearly all of them, which lists the runs of 32 rays that hold
+// of few samples, nearly all of them, which lists the runs of 32 rays that hold
 // others, and one for those.  Together in one kernel the long rays' registers
-// spilled in the short ones' path, and a block that met many long rays made the
-// rest wait.  Batch of 48 meshes, a quarter of them noisy tori with up to 92
-// layers: 85 + 141 us, 265 to 510 us in one; 1.31 M-triangle sphere at 2048^2:
-// 73 + 6 us, 93 to 140 us in one.
+// spill in the short ones' path, and a block that meets many long rays makes the
+// rest wait, which only images of few rays repay (kSmallSort).  Batch of 48 meshes,
+// a quarter of them noisy tori with up to 92 layers: 85 + 141 us, 265 to 510 us in
+// one; 1.31 M-triangle sphere at 2048^2: 73 + 6 us, 93 to 140 us in one.
 
 // A lane's range of samples in one run of 32 rays p0 .. (whole warp); odd counts
 // are reported if report.
@@ -783,13 +787,52 @@ __device__ __forceinline__ void finish_pair(long long b, const RayOut &r, const 
     }
 }
 
+// A ray of up to four samples from slot b on, ordered in registers.
+__device__ __forceinline__ void finish_few(long long b, int n, const RayOut &r, const NormalTable &nrm) {
+    float d[4];
+    int t[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        d[i] = i < n ? r.D[b + i] : INFINITY;
+        t[i] = i < n ? r.Tr[b + i] : INT_MAX;
+    }
+    const auto order = [&](int i, int j) {
+        if (key_less(d[j], t[j], d[i], t[i])) {
+            const float x = d[i];
+            d[i] = d[j];
+            d[j] = x;
+            const int y = t[i];
+            t[i] = t[j];
+            t[j] = y;
+        }
+    };
+    order(0, 1);
+    order(2, 3);
+    order(0, 2);
+    order(1, 3);
+    order(1, 2);
+#pragma unroll
+    for (int h = 0; h < 4; h += 2) {  // two normals are read before either of their samples is stored
+        if (h >= n) break;
+        const float4 q0 = nrm(t[h]), q1 = nrm(h + 1 < n ? t[h + 1] : 0);
+        r.D[b + h] = d[h];
+        r.Tr[b + h] = t[h];
+        put_normal(r, b + h, q0);
+        if (h + 1 < n) {
+            r.D[b + h + 1] = d[h + 1];
+            r.Tr[b + h + 1] = t[h + 1];
+            put_normal(r, b + h + 1, q1);
+        }
+    }
+}
+
 // A warp's rays (b, n) of other numbers of samples (n = 0: none in this lane).
 __device__ __forceinline__ void finish_rest(long long b, int n, const RayOut &r, const NormalTable &nrm, SortStage &st,
                                          int lane) {
-    if (n == 1) {
-        put_normal(r, b, nrm(r.Tr[b]));
+    if (n > 0 && n <= 4) {
+        finish_few(b, n, r, nrm);
         n = 0;
-    } else if (n > 2 && n <= kLaneSort) {
+    } else if (n > 4 && n <= kLaneSort) {
         // the lanes' rays side by side, each in its lane's registers (kLaneSort's network)
         unsigned long long key[kLaneSort];
         float d[kLaneSort];

@@ -311,3 +311,66 @@ def test_a_fill_of_another_mesh_is_reported(ldni, binned, change):
     outs, status = _count_then_fill(ldni, binned, first, second, grid, 1)
     assert status[0] & _lib.ST_CAPACITY
     _check_rays(outs, ref)
+
+
+def _sheets(k, seed, lo, hi, u0, u1):
+    """k open sheets across the x-axis at random depths in [lo, hi], listed in
+    random order: every x-ray through [u0, u1]^2 has exactly k samples."""
+    rng = np.random.default_rng(seed)
+    d = rng.permutation(np.linspace(lo, hi, k)).astype(np.float32)
+    v = np.array([[x, y, z] for x in d for y, z in ((u0, u0), (u1, u0), (u1, u1), (u0, u1))], np.float32)
+    t = np.array([[4 * i + a, 4 * i + b, 4 * i + c] for i in range(k) for a, b, c in ((0, 1, 2), (0, 2, 3))], np.int32)
+    return v, t
+
+
+@pytest.mark.parametrize("packed", [False, True])
+@pytest.mark.parametrize("res", [64, 820])
+def test_rays_of_any_count_in_either_ordering(ldni, packed, res):
+    """Rays of 0 to 9, 40 and 300 samples side by side, odd counts among them,
+    in images small enough to be ordered in one kernel and in three large ones
+    that take two (820^2: 2.02 M rays): ids by ascending depth, the same in the
+    call for all images, the one for one image and the binned form."""
+    parts, at, base = [], [], 0
+    for j, k in enumerate([1, 2, 3, 4, 5, 6, 7, 8, 9, 40, 300]):
+        u0 = -0.48 + 0.085 * j
+        m = _sheets(k, j, -0.45, 0.45, u0, u0 + (0.07 if k < 40 else 3.0 / res))
+        parts.append((m[0], m[1] + base))
+        base += len(m[0])
+    v, t = np.concatenate([m[0] for m in parts]), np.concatenate([m[1] for m in parts])
+    order = np.random.default_rng(res).permutation(len(t))
+    t = t[order]
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    got = ldni.sample(v, t, grid, "all", packed=packed)
+    one = ldni.sample(v, t, grid, 0, packed=packed)
+    binned = ldni.sample(v, t, grid, "all", mode="binned2", packed=packed)
+    assert ldni.identical(got[0], one)
+    assert all(ldni.identical(x, y) for x, y in zip(got, binned))
+    g = got[0].numpy()
+    counts = np.diff(g["offsets"])
+    assert set(np.unique(counts)) >= {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 40, 300}
+    ray = np.repeat(np.arange(res * res), counts)
+    x = v[t[g["tri"]][:, 0], 0]  # a sheet's depth
+    assert np.all(np.abs(g["depth"] - x) <= 1e-5 * DIAG)  # the sampling bound
+    assert np.array_equal(np.lexsort((g["tri"], g["depth"], ray)), np.arange(len(ray)))
+    same = ray[1:] == ray[:-1]
+    assert np.all(x[1:][same] > x[:-1][same])  # one sample of every sheet
+    e1, e2 = v[t[:, 1]] - v[t[:, 0]], v[t[:, 2]] - v[t[:, 0]]
+    nrm = np.cross(e1.astype(np.float64), e2.astype(np.float64))
+    nrm /= np.linalg.norm(nrm, axis=1, keepdims=True)
+    if packed:
+        code = np.rint((nrm[g["tri"]] + 1) * 127.5).astype(np.uint32)
+        assert np.array_equal(g["nrm8"], code[:, 0] | (code[:, 1] << 8) | (code[:, 2] << 16))
+    else:
+        assert np.all(np.abs(g["nrm"] - nrm[g["tri"]]) <= 1e-5)  # the sampling bound
+
+
+@pytest.mark.parametrize("res", [40, 400, 816, 817])
+def test_big_pairs_beside_and_after_the_triangles(ldni, res):
+    """Twelve faces in images small and large enough for the fill to take their
+    pairs beside the triangles and in a launch of their own (from 2 M rays)."""
+    m = M.box([-0.41, -0.33, -0.27], [0.35, 0.39, 0.44])
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    assert (3 * res * res > 2000000) == (res >= 817)
+    _check_all_axes(ldni, m, res)
+    assert all(ldni.identical(x, y) for x, y in zip(ldni.sample(*m, grid, "all"),
+                                                    ldni.sample(*m, grid, "all", mode="binned2")))
