@@ -12,13 +12,17 @@
 // Booleans of the step-by-step evaluation, whose intermediate images would
 // each be written to and read back from memory.  Without small-interval
 // removal the fold is a union of intervals (unite_pass); with it, or where that
-// does not fit, it merges sample by sample (fold_pass).
+// does not fit, it merges sample by sample (fold_pass).  The count pass leaves
+// the sources of every interval it finds in a pool of records, from which the
+// write pass copies them; a ray whose records find no room in the pool is
+// folded again when it is written.
 //
 // The result equals the step-by-step chain bit for bit: each step is the
 // same merge (merge.cuh) with the accumulated solid as the first operand, so
 // at a shared depth the accumulated sample is kept, and a sample that first
 // enters through part k >= 1 carries the second-operand mark (tri_id bit 31)
 // from then on.
+#include <algorithm>
 #include <climits>
 
 #include "ldni_host.h"
@@ -49,26 +53,36 @@ __device__ __forceinline__ void part_range(const ldni_layers_t &P, long long p, 
 // part's are, so the offsets of kAhead parts are loaded together: loaded part
 // by part between the merges, 64 round trips to memory made up the fold.  odd
 // counts the parts with an odd number of samples (Definition 4).
-constexpr int kAhead = 8;
+// (kN a time, down to one at the end of the parts: short chains would load
+// their last part's offsets up to seven times over.)
+template <int kN>
+__device__ __forceinline__ unsigned long long present_step(const ldni_layers_t *__restrict__ parts, int &q0, long long p,
+                                                           int &odd) {
+    int b[kN], e[kN];
+#pragma unroll
+    for (int q = 0; q < kN; ++q) {
+        const int *off = parts[q0 + q].offsets;
+        b[q] = __ldg(off + p);
+        e[q] = __ldg(off + p + 1);
+    }
+    unsigned mask = 0;
+#pragma unroll
+    for (int q = 0; q < kN; ++q) {
+        odd += (e[q] - b[q]) & 1;
+        mask |= e[q] != b[q] ? 1u << q : 0u;
+    }
+    q0 += kN;
+    return (unsigned long long)mask << (q0 - kN);
+}
 __device__ __forceinline__ unsigned long long parts_present(const ldni_layers_t *__restrict__ parts, int count, int k0,
                                                             long long p, int &odd) {
     unsigned long long mask = 0;
     const int n = min(count - k0, 64);
-    for (int q0 = 0; q0 < n; q0 += kAhead) {
-        int b[kAhead], e[kAhead];
-#pragma unroll
-        for (int q = 0; q < kAhead; ++q) {
-            const int *off = parts[k0 + min(q0 + q, n - 1)].offsets;
-            b[q] = __ldg(off + p);
-            e[q] = __ldg(off + p + 1);
-        }
-#pragma unroll
-        for (int q = 0; q < kAhead; ++q) {
-            if (q0 + q >= n) continue;
-            odd += (e[q] - b[q]) & 1;
-            if (e[q] != b[q]) mask |= 1ull << (q0 + q);
-        }
-    }
+    int q0 = 0;
+    while (n - q0 >= 8) mask |= present_step<8>(parts + k0, q0, p, odd);
+    if (n - q0 >= 4) mask |= present_step<4>(parts + k0, q0, p, odd);
+    if (n - q0 >= 2) mask |= present_step<2>(parts + k0, q0, p, odd);
+    if (n - q0 >= 1) mask |= present_step<1>(parts + k0, q0, p, odd);
     return mask;
 }
 
@@ -196,50 +210,36 @@ __device__ __forceinline__ bool each_span(const ldni_layers_t *__restrict__ part
     return true;
 }
 
-// Adds a span to the n of S (in registers when kInRegs: n = kN, empty ones
-// among them); false when there is no room.
-template <int kN, bool kInRegs>
-__device__ __forceinline__ bool add_span(Span (&S)[kN], int &n, Span s) {
-    if (kInRegs) {
-        bool put = false;
+// Adds a span to S (empty ones among them); false when there is no room.
+template <int kN>
+__device__ __forceinline__ bool add_span(Span (&S)[kN], Span s) {
+    bool put = false;
 #pragma unroll
-        for (int i = 0; i < kN; ++i) s.take(S[i]);
+    for (int i = 0; i < kN; ++i) s.take(S[i]);
 #pragma unroll
-        for (int i = 0; i < kN; ++i)
-            if (!put && S[i].empty()) {
-                S[i] = s;
-                put = true;
-            }
-        return put;
-    }
-    int m = 0;
-    for (int i = 0; i < n; ++i) {  // the ones left move up
-        s.take(S[i]);
-        if (!S[i].empty()) {
-            if (m != i) S[m] = S[i];
-            ++m;
+    for (int i = 0; i < kN; ++i)
+        if (!put && S[i].empty()) {
+            S[i] = s;
+            put = true;
         }
-    }
-    n = m;
-    if (n == kN) return false;
-    S[n++] = s;
-    return true;
+    return put;
 }
 
-// Pass 1, when no thin intervals are removed: every ray's parts, its count and
-// sources (Rays) for results that never have more than kSpans disjoint
-// intervals; the other rays are listed.  Bound by the reads of the parts'
-// offsets (201 MB for 64 parts at 512^2, three images) and the chain of loads of
-// the rays that meet a part, a fifth of them: 98 us.  (Loading part by part
-// between merges in local memory took 254 us, and 248 again for the samples,
-// now 39.)
-constexpr int kSpans = 4;
-constexpr int kKept = 2 * kSpans;  // samples whose sources pass 1 leaves to the write pass
+// What the count pass leaves: every ray's count; a record per interval of its
+// result; the rays left to fold_pass, from the front of one list, and those
+// whose records found no room, from its back (a ray of the front that finds
+// none stays in the list, the others of the front are marked -1).  Rays are
+// numbered image N + ray.
+struct Record {
+    int ray, k;  // the interval's ray and its number there (-1: unused)
+};
 struct Rays {
     int *count[3];
-    unsigned long long *present[3];  // the first 64 parts that the ray meets
-    int4 *kept[3];                   // (part, sample) twice; kKept / 2 per ray
-    long long *list;                 // rays (nrays image + ray) left to fold_pass; their number first
+    int4 *src;              // per record: (part, sample) of its ends; second part -1: a sample alone
+    Record *rec;
+    int *list;
+    unsigned long long *n;  // front of the list, back of the list, records
+    long long records, rays;
 };
 
 __device__ __forceinline__ void report_odd(int odd, ldni_info_t *info) {
@@ -249,49 +249,84 @@ __device__ __forceinline__ void report_odd(int odd, ldni_info_t *info) {
     }
 }
 
+// First record of each lane's `want` (whole warp), -1 where the pool has no
+// room for all of them.
+__device__ __forceinline__ long long claim_records(const Rays &rays, int want, int lane) {
+    int upto = want;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += x;
+    }
+    const int all = __shfl_sync(0xffffffffu, upto, 31);
+    if (all == 0) return 0;
+    unsigned long long at = 0;
+    if (lane == 0) at = atomicAdd(rays.n + 2, (unsigned long long)all);
+    const long long first = (long long)__shfl_sync(0xffffffffu, at, 0) + upto - want;
+    if (first + want <= rays.records) return first;
+    for (long long i = first; i < rays.records; ++i) rays.rec[i].k = -1;  // (at most one lane's)
+    return -1;
+}
+
+__device__ __forceinline__ void put_record(const Rays &rays, long long at, long long ray, int k, int2 lo, int2 hi) {
+    rays.src[at] = make_int4(lo.x, lo.y, hi.x, hi.y);
+    rays.rec[at] = Record{(int)ray, k};
+}
+
+// Pass 1, when no thin intervals are removed: the rays whose results never have
+// more than kSpans disjoint intervals; the others are listed.  Bound by the
+// reads of the parts' offsets (201 MB for 64 parts at 512^2, three images) and
+// the chain of loads of the rays that meet a part, a fifth of them: 95 us.
+constexpr int kSpans = 4;
+
 __global__ void __launch_bounds__(kThreads, 6) unite_pass(long long N, const ldni_layers_t *__restrict__ parts_all,
                                                           int count, Rays rays, ldni_info_t *info) {
-    const int img = blockIdx.y;
+    const int img = blockIdx.y, lane = threadIdx.x & 31;
     const ldni_layers_t *parts = parts_all + (size_t)img * count;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
-        int odd = 0;
-        const unsigned long long present = parts_present(parts, count, 0, p, odd);
-        for (int k0 = 64; k0 < count; k0 += 64) parts_present(parts, count, k0, p, odd);
-        report_odd(odd, info);
-        if (present == 0 && count <= 64) {
-            rays.count[img][p] = 0;
-            continue;
-        }
+    // (whole warps: the rays' records are claimed together)
+    for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); base < N;
+         base += (long long)gridDim.x * blockDim.x) {
+        const long long p = base + lane;
         Span S[kSpans];
 #pragma unroll
         for (int i = 0; i < kSpans; ++i) S[i] = Span{INFINITY, -INFINITY, {0, 0}, {0, 0}};
-        int n = kSpans;
-        rays.present[img][p] = present;
-        if (!each_span(parts, count, p,
-                       [&](int k0) { return k0 == 0 ? present : parts_present(parts, count, k0, p, odd); },
-                       [&](const Span &s) { return add_span<kSpans, true>(S, n, s); })) {
-            rays.list[1 + atomicAdd(reinterpret_cast<unsigned long long *>(rays.list), 1ull)] = N * img + p;
-            continue;
+        bool left = false;
+        if (p < N) {
+            int odd = 0;
+            const unsigned long long present = parts_present(parts, count, 0, p, odd);
+            for (int k0 = 64; k0 < count; k0 += 64) parts_present(parts, count, k0, p, odd);
+            report_odd(odd, info);
+            if (present != 0 || count > 64)
+                left = !each_span(parts, count, p,
+                                  [&](int k0) { return k0 == 0 ? present : parts_present(parts, count, k0, p, odd); },
+                                  [&](const Span &s) { return add_span<kSpans>(S, s); });
         }
-        // ascending
+        int m = 0;
+        if (!left) {
+            // ascending, the empty ones last
 #pragma unroll
-        for (int i = 0; i < kSpans - 1; ++i)
+            for (int i = 0; i < kSpans - 1; ++i)
 #pragma unroll
-            for (int j = 0; j < kSpans - 1 - i; ++j)
-                if (S[j + 1].lo < S[j].lo) {
-                    const Span t = S[j];
-                    S[j] = S[j + 1];
-                    S[j + 1] = t;
-                }
-        int4 *kept = rays.kept[img] + kKept / 2 * p;
-        int out = 0;
+                for (int j = 0; j < kSpans - 1 - i; ++j)
+                    if (S[j + 1].lo < S[j].lo) {
+                        const Span t = S[j];
+                        S[j] = S[j + 1];
+                        S[j + 1] = t;
+                    }
 #pragma unroll
-        for (int i = 0; i < kSpans; ++i)
-            if (!S[i].empty()) {
-                kept[i] = make_int4(S[i].slo.x, S[i].slo.y, S[i].shi.x, S[i].shi.y);
-                out += 2;
-            }
-        rays.count[img][p] = out;
+            for (int i = 0; i < kSpans; ++i) m += S[i].empty() ? 0 : 1;
+        }
+        const long long ray = N * img + p;
+        const long long at = claim_records(rays, m, lane);
+        if (at >= 0) {
+#pragma unroll
+            for (int i = 0; i < kSpans; ++i)
+                if (i < m) put_record(rays, at + i, ray, i, S[i].slo, S[i].shi);
+        } else if (m > 0) {
+            rays.list[rays.rays - 1 - (long long)atomicAdd(rays.n + 1, 1ull)] = (int)ray;
+        }
+        if (left) rays.list[atomicAdd(rays.n, 1ull)] = (int)ray;
+        if (p < N) rays.count[img][p] = 2 * m;
     }
 }
 
@@ -334,90 +369,92 @@ __device__ __forceinline__ void put_samples(const ldni_layers_t *__restrict__ pa
 }
 
 // The rays that unite_pass listed, or all of them (all: with thin intervals
-// removed after every step, or one part alone): kWrite false, their counts and
-// the sources of up to kKept samples; kWrite true, the samples of longer
-// results.  A listed ray is united like unite_pass's, with room for any result
-// the chain may hold, and folded where that says no.
-template <bool kWrite>
+// removed after every step, or one part alone): their counts and records.  On as
+// many blocks as stay resident, whatever the list's length: three stacks of nine
+// slabs at 512^2, where most rays are listed, 90 us, 212 on a block per SM.
 __global__ void __launch_bounds__(kThreads) fold_pass(long long N, const ldni_layers_t *__restrict__ parts_all,
-                                                      int count, int nimg, int all, float eps, Rays rays,
-                                                      ldni_layers_t o0, ldni_layers_t o1, ldni_layers_t o2,
-                                                      ldni_info_t *info) {
+                                                      int count, int all, float eps, Rays rays, ldni_info_t *info) {
     Entry acc[2][kChainMaxLayers];
-    const long long total = all ? N * nimg : rays.list[0];
-    for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < total; r += (long long)gridDim.x * blockDim.x) {
-        const long long ray = all ? r : rays.list[1 + r];
+    const int lane = threadIdx.x & 31;
+    const long long total = all ? rays.rays : (long long)rays.n[0];
+    for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); base < total;
+         base += (long long)gridDim.x * blockDim.x) {
+        const long long r = base + lane;
+        const bool mine = r < total;
+        const long long ray = !mine ? 0 : (all ? r : rays.list[r]);
         const int img = (int)(ray / N);
         const long long p = ray - img * N;
-        if (kWrite && rays.count[img][p] <= kKept) continue;
-        const ldni_layers_t *parts = parts_all + (size_t)img * count;
-        int odd = 0;
-        unsigned long long present;
-        if (all && !kWrite) {
-            present = parts_present(parts, count, 0, p, odd);
-            for (int k0 = 64; k0 < count; k0 += 64) parts_present(parts, count, k0, p, odd);
-            report_odd(odd, info);
-            rays.present[img][p] = present;
-        } else {
-            present = rays.present[img][p];
-        }
-        const auto have = [&](int k0) { return k0 == 0 ? present : parts_present(parts, count, k0, p, odd); };
-        int cur = 0, n = -1;
-        if (!all) {
-            Span S[kChainMaxLayers / 2];
-            int m = 0;
-            if (each_span(parts, count, p, have,
-                          [&](const Span &s) { return add_span<kChainMaxLayers / 2, false>(S, m, s); })) {
-                for (int i = 1; i < m; ++i) {  // ascending
-                    const Span t = S[i];
-                    int j = i;
-                    for (; j > 0 && t.lo < S[j - 1].lo; --j) S[j] = S[j - 1];
-                    S[j] = t;
-                }
-                for (int i = 0; i < m; ++i) {
-                    acc[0][2 * i] = Entry{S[i].lo, S[i].slo.x, S[i].slo.y};
-                    acc[0][2 * i + 1] = Entry{S[i].hi, S[i].shi.x, S[i].shi.y};
-                }
-                n = 2 * m;
+        int cur = 0, n = 0;
+        if (mine) {
+            const ldni_layers_t *parts = parts_all + (size_t)img * count;
+            int odd = 0;
+            const unsigned long long present = parts_present(parts, count, 0, p, odd);
+            if (all) {
+                for (int k0 = 64; k0 < count; k0 += 64) parts_present(parts, count, k0, p, odd);
+                report_odd(odd, info);
             }
-        }
-        if (n < 0) n = fold_ray(parts, count, p, eps, acc, cur, have);
-        if (!kWrite) {
+            n = fold_ray(parts, count, p, eps, acc, cur,
+                         [&](int k0) { return k0 == 0 ? present : parts_present(parts, count, k0, p, odd); });
             if (n < 0) {
                 set_status(info, LDNI_ST_EVENTS);
                 n = 0;
             }
-            rays.count[img][p] = n;
-            if (n > kKept) continue;
-            int4 *kept = rays.kept[img] + kKept / 2 * p;
-            for (int i = 0; 2 * i < n; ++i)
-                kept[i] = make_int4(acc[cur][2 * i].part, acc[cur][2 * i].idx, acc[cur][2 * i + 1].part,
-                                    acc[cur][2 * i + 1].idx);
-        } else {
-            const ldni_layers_t &o = img == 0 ? o0 : (img == 1 ? o1 : o2);
-            for (int x = 0; x < n; ++x) {
-                const int2 one[1] = {{acc[cur][x].part, acc[cur][x].idx}};
-                put_samples(parts, o, one, 1, (long long)o.offsets[p] + x, info);
-            }
         }
+        const int m = (n + 1) / 2;
+        const long long at = claim_records(rays, m, lane);
+        if (!mine) continue;
+        if (at >= 0 || m == 0) {
+            for (int i = 0; i < m; ++i) {
+                const Entry lo = acc[cur][2 * i], hi = 2 * i + 1 < n ? acc[cur][2 * i + 1] : Entry{0.0f, -1, 0};
+                put_record(rays, at + i, ray, i, make_int2(lo.part, lo.idx), make_int2(hi.part, hi.idx));
+            }
+            if (!all) rays.list[r] = -1;
+        } else if (all) {
+            rays.list[rays.rays - 1 - (long long)atomicAdd(rays.n + 1, 1ull)] = (int)ray;
+        }
+        rays.count[img][p] = n;
     }
 }
 
-// The samples of results of up to kKept.
+// A ray without records: folded once more, and written.
+__device__ __noinline__ void write_folded(const ldni_layers_t *__restrict__ parts, int count, long long p, float eps,
+                                          const ldni_layers_t &o, ldni_info_t *info) {
+    Entry acc[2][kChainMaxLayers];
+    int cur, odd;
+    const int n = fold_ray(parts, count, p, eps, acc, cur,
+                           [&](int k0) { return parts_present(parts, count, k0, p, odd); });
+    for (int x = 0; x < n; ++x) {
+        const int2 one[1] = {{acc[cur][x].part, acc[cur][x].idx}};
+        put_samples(parts, o, one, 1, (long long)o.offsets[p] + x, info);
+    }
+}
+
+// The result's samples: a thread per record, then the rays without any.  A
+// thread per ray with its kept sources spread a fifth of the threads' work over
+// all of them: 41 us for 64 parts at 512^2, 22 now; folding deep rays again to
+// write them took 330 us for the stacks of slabs, 68 now.
 __global__ void __launch_bounds__(kThreads) chain_write(long long N, const ldni_layers_t *__restrict__ parts_all,
-                                                        int count, Rays rays, ldni_layers_t o0, ldni_layers_t o1,
-                                                        ldni_layers_t o2, ldni_info_t *info) {
-    const int img = blockIdx.y;
-    const ldni_layers_t &o = img == 0 ? o0 : (img == 1 ? o1 : o2);
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
-        const int n = rays.count[img][p];
-        if (n == 0 || n > kKept) continue;
-        const int4 *kept = rays.kept[img] + kKept / 2 * p;
-        for (int x = 0; x < n; x += 4) {
-            const int4 a = kept[x / 2], b = n > x + 2 ? kept[x / 2 + 1] : a;
-            const int2 from[4] = {{a.x, a.y}, {a.z, a.w}, {b.x, b.y}, {b.z, b.w}};
-            put_samples(parts_all + (size_t)img * count, o, from, min(n - x, 4), (long long)o.offsets[p] + x, info);
-        }
+                                                        int count, int all, float eps, Rays rays, ldni_layers_t o0,
+                                                        ldni_layers_t o1, ldni_layers_t o2, ldni_info_t *info) {
+    const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    const long long claimed = (long long)rays.n[2], n = min(claimed, rays.records);
+    for (long long i = first; i < n; i += step) {
+        const Record R = rays.rec[i];
+        const int4 v = rays.src[i];
+        if (R.k < 0) continue;
+        const int img = (unsigned)R.ray / (unsigned)N;
+        const ldni_layers_t &o = img == 0 ? o0 : (img == 1 ? o1 : o2);
+        const int2 from[2] = {{v.x, v.y}, {v.z, v.w}};
+        put_samples(parts_all + (size_t)img * count, o, from, v.z < 0 ? 1 : 2,
+                    (long long)o.offsets[R.ray - img * N] + 2 * R.k, info);
+    }
+    if (claimed <= rays.records) return;  // every ray has its records
+    const long long front = all ? 0 : (long long)rays.n[0], back = (long long)rays.n[1];
+    for (long long r = first; r < front + back; r += step) {
+        const int ray = rays.list[r < front ? r : rays.rays - 1 - (r - front)];
+        if (ray < 0) continue;
+        const int img = (unsigned)ray / (unsigned)N;
+        write_folded(parts_all + (size_t)img * count, count, ray - img * N, eps, img == 0 ? o0 : (img == 1 ? o1 : o2), info);
     }
 }
 
@@ -426,15 +463,19 @@ struct ChainWs {
     long long *partials;
 };
 
+// Records: up to 32 a ray for small images, one for every three rays of large
+// ones (a swept solid's rays are mostly empty): 16 bytes a ray in all, 0.8 GB for
+// three images of 4096^2, where sources kept for every ray took 84.
 ChainWs carve_chain_ws(Carver &c, int res, int nimg) {
     ChainWs w{};
-    const long long N = (long long)res * res;
-    for (int j = 0; j < nimg; ++j) {
-        w.rays.count[j] = c.take<int>((size_t)N);
-        w.rays.present[j] = c.take<unsigned long long>((size_t)N);
-        w.rays.kept[j] = c.take<int4>(kKept / 2 * (size_t)N);
-    }
-    w.rays.list = c.take<long long>((size_t)N * nimg + 1);
+    const long long N = (long long)res * res, rays = N * nimg;
+    for (int j = 0; j < nimg; ++j) w.rays.count[j] = c.take<int>((size_t)N);
+    w.rays.rays = rays;
+    w.rays.records = std::min(rays * (kChainMaxLayers / 2), std::max(2ll << 20, rays / 3));
+    w.rays.src = c.take<int4>((size_t)w.rays.records);
+    w.rays.rec = c.take<Record>((size_t)w.rays.records);
+    w.rays.list = c.take<int>((size_t)rays);
+    w.rays.n = c.take<unsigned long long>(3);
     w.partials = c.take<long long>(csr_scan_partials(N) * nimg);
     return w;
 }
@@ -483,24 +524,18 @@ extern "C" int ldni_union_chain(const ldni_layers_t *parts_dev, const ldni_layer
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     ldni_layers_t o[3] = {out[0], nimg > 1 ? out[1] : out[0], nimg > 2 ? out[2] : out[0]};
     const dim3 g((unsigned)grid_for(N), (unsigned)nimg);
+    const unsigned blocks = (unsigned)grid_for(N * nimg);  // the lists' lengths are known on the device
     const int all = eps == 0.0f && count > 1 ? 0 : 1;
-    const unsigned fblocks = all ? (unsigned)grid_for(N * nimg) : (unsigned)num_sms();
-    if (!all) {
-        if (int rc_ = cuda_check(cudaMemsetAsync(w.rays.list, 0, sizeof(long long), s))) return rc_;
-        LDNI_LAUNCH(K_CHAIN, s, unite_pass<<<g, kThreads, 0, s>>>(N, parts_dev, count, w.rays, info));
-    }
-    LDNI_LAUNCH(K_CHAIN, s,
-                fold_pass<false><<<fblocks, kThreads, 0, s>>>(N, parts_dev, count, nimg, all, eps, w.rays, o[0], o[1],
-                                                              o[2], info));
+    if (int rc_ = cuda_check(cudaMemsetAsync(w.rays.n, 0, 3 * sizeof(unsigned long long), s))) return rc_;
+    if (!all) LDNI_LAUNCH(K_CHAIN, s, unite_pass<<<g, kThreads, 0, s>>>(N, parts_dev, count, w.rays, info));
+    LDNI_LAUNCH(K_CHAIN, s, fold_pass<<<blocks, kThreads, 0, s>>>(N, parts_dev, count, all, eps, w.rays, info));
     int rc = cuda_status();
     if (rc != LDNI_OK) return rc;
     const int *cnt[3] = {w.rays.count[0], w.rays.count[1], w.rays.count[2]};
     int *off[3] = {out[0].offsets, nimg > 1 ? out[1].offsets : nullptr, nimg > 2 ? out[2].offsets : nullptr};
     rc = csr_scan(cnt, off, nimg, N, w.partials, info, 0, s);
     if (rc != LDNI_OK) return rc;
-    LDNI_LAUNCH(K_CHAIN, s, chain_write<<<g, kThreads, 0, s>>>(N, parts_dev, count, w.rays, o[0], o[1], o[2], info));
     LDNI_LAUNCH(K_CHAIN, s,
-                fold_pass<true><<<fblocks, kThreads, 0, s>>>(N, parts_dev, count, nimg, all, eps, w.rays, o[0], o[1],
-                                                             o[2], info));
+                chain_write<<<blocks, kThreads, 0, s>>>(N, parts_dev, count, all, eps, w.rays, o[0], o[1], o[2], info));
     return cuda_status();
 }

@@ -205,3 +205,80 @@ def test_random_intervals(ldni, count, most, levels, res):
             assert e.code == -4 and count >= 64  # a ray of more than 64 samples at some step
             continue
         assert ldni.identical(got, _stepwise(ldni, P, eps)), eps
+
+
+def _intervals(ldni, grid, counts, lo, hi, shift, seed):
+    """An image with counts[p] disjoint intervals on ray p, evenly spaced in
+    [lo, hi] and moved by `shift` of their spacing."""
+    rng = np.random.default_rng(seed)
+    counts = np.asarray(counts)
+    off = np.concatenate([[0], np.cumsum(2 * counts)])
+    n = int(off[-1])
+    j = np.arange(n) - np.repeat(off[:-1], 2 * counts)
+    k = np.repeat(np.maximum(counts, 1), 2 * counts)
+    depth = lo + (hi - lo) * (j // 2 + shift + 0.4 * (j & 1)) / (k + 1)
+    t = lambda x, dt: torch.from_numpy(np.ascontiguousarray(x, dt)).cuda()
+    nrm = rng.standard_normal((3, n))
+    return ldni.LDNI(grid, 0, t(off, np.int32), t(depth, np.float32), *[t(x, np.float32) for x in nrm],
+                     t(rng.integers(0, 1000, size=n), np.int32), n)
+
+
+def _layers_needed(ldni, P, eps):
+    """Most samples on a ray at any step, the first part alone included."""
+    acc, most = P[0], int(P[0].counts().max())
+    for k in range(1, len(P)):
+        acc = ldni.boolean(acc, P[k], "union", eps=eps)
+        most = max(most, int(acc.counts().max()))
+    return most
+
+
+@pytest.mark.parametrize("first,second,count", [(32, 0, 2), (32, 1, 2), (33, 0, 2), (33, 0, 1), (16, 16, 3), (20, 13, 2),
+                                                (31, 1, 70)])
+@pytest.mark.parametrize("eps", [0.0, 1e-6])
+def test_limit_of_layers_exactly(ldni, first, second, count, eps):
+    """A chain is reported (a ray of more than 64 samples) exactly when a step
+    of the step-by-step unions has such a ray, a last part over everything
+    notwithstanding."""
+    res = 6
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    at = np.zeros(res * res, np.int64)
+    at[[3, 17, 35]] = 1
+    P = [_intervals(ldni, grid, first * at, -0.4, 0.4, 0.0, 1)]
+    if count > 1:
+        P.append(_intervals(ldni, grid, second * at, -0.4, 0.4, 0.5, 2))  # in the gaps of equally many, else across
+    P += [_intervals(ldni, grid, at, -0.45, 2.0, 0.0, 3) for _ in range(count - len(P))]
+    most = _layers_needed(ldni, P, eps)
+    run, finish = ldni.union_chain(P, eps=eps)
+    run()
+    if most > 64:
+        with pytest.raises(ldni.LDNIError) as e:
+            finish()
+        assert e.value.code == -4
+    else:
+        assert ldni.identical(finish(), _stepwise(ldni, P, eps))
+
+
+@pytest.mark.parametrize("eps", [0.0, 1e-7])
+def test_more_intervals_than_records(ldni, eps):
+    """An image whose result has more intervals than the workspace has records
+    (2 M for 160,000 rays): rays of one to four, of more, and empty ones, with
+    and without records, equal the step-by-step unions; so does one part
+    alone."""
+    res = 400
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    rng = np.random.default_rng(9)
+    c = np.where(rng.random(res * res) < 0.75, rng.integers(16, 31, size=res * res), rng.integers(0, 4, size=res * res))
+    A = _intervals(ldni, grid, c, -0.45, 0.45, 0.0, 4)
+    B = _intervals(ldni, grid, rng.integers(0, 2, size=res * res), -0.3, 0.3, 0.2, 5)
+    for P in ([A, B, A], [A]):
+        run, finish = ldni.union_chain(P, eps=eps)
+        run()
+        got = finish()
+        assert got.n > 2 * (2 << 20)
+        assert ldni.identical(got, _stepwise(ldni, P, eps))
+
+
+def test_workspace_stays_small(ldni):
+    """About 16 bytes a ray for large images."""
+    for res in (2048, 4096, 8192):
+        assert ldni.union_chain_workspace_size(res, 3) <= 17 * 3 * res * res
