@@ -16,13 +16,23 @@ constexpr size_t kAlign = 256;
 
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
-// Hands out aligned slices of one caller-provided workspace.  With base ==
-// nullptr it only measures.
+// Hands out aligned slices of one caller-provided workspace, which may start at
+// any address: the slices hold 16-byte vectors, so they are counted from the
+// next multiple of 16.  With base == nullptr it only measures, with one slice's
+// alignment to spare for such a start.
 struct Carver {
     char *base;
     size_t off = 0;
     size_t cap;
-    Carver(void *b, size_t c) : base(static_cast<char *>(b)), cap(c) {}
+    Carver(void *b, size_t c) : base(static_cast<char *>(b)), cap(c) {
+        if (!b) {
+            off = 1;
+            return;
+        }
+        const size_t skip = (0 - reinterpret_cast<uintptr_t>(b)) & 15;
+        base += skip;
+        cap -= skip < cap ? skip : cap;
+    }
     template <class T>
     T *take(size_t count) {
         size_t at = align_up(off);

@@ -249,7 +249,7 @@ using namespace ldni;
 extern "C" int ldni_classify_nodes_workspace_size(int32_t res, size_t *bytes) {
     if (!bytes || res < 1 || res > 4096) return LDNI_EINVAL;
     const size_t W = ((size_t)res + 31) / 32, groups = (size_t)res * W;  // as many groups in a row as words in a ray
-    *bytes = align_up(3 * (align_up(sizeof(uint2) * groups * W) + align_up(sizeof(unsigned) * groups * W * 32)));
+    *bytes = 3 * (align_up(sizeof(uint2) * groups * W) + align_up(sizeof(unsigned) * groups * W * 32)) + kAlign;
     return LDNI_OK;
 }
 
