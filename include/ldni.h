@@ -545,8 +545,8 @@ int ldni_contour_workspace_size(int32_t res, int64_t max_active, size_t *bytes_h
  * Each cluster that meets an intersect, none-intersect or complex edge gets
  * a vertex at x = m + (A^T A)^+ (A^T b - A^T A m) over its Hermite points p
  * (rows of A: the normals n; b = n . p; m: the points' mean), eigenvalues of
- * A^T A below 0.01 of the largest dropped, in FP64; with no points, at the
- * mean of its corners (npts 0).
+ * A^T A below 0.01 of the largest dropped, summed in FP64 and solved to 1e-8
+ * of its distance from m; with no points, at the mean of its corners (npts 0).
  *   L: host array of the three images x, y, z (FP32 normals); inside: the
  *   node bits; cells: device array of `capacity` records, written in
  *   ascending cell order.  info->n[0] = cells with a vertex; beyond capacity

@@ -22,9 +22,9 @@
 //    cluster of a cell that meets an intersect, none-intersect or complex
 //    edge yields a vertex;
 //  - x = m + (A^T A)^+ (A^T b - A^T A m), m the points' mean, eigenvalues of
-//    A^T A below 0.01 of the largest dropped (singular values below 0.1),
-//    in FP64; a cluster with no Hermite data sits at the mean of its corners
-//    with no points.
+//    A^T A below 0.01 of the largest dropped (singular values below 0.1), its
+//    sums in FP64 and solved to 1e-8 of its displacement from m (qef_solve); a
+//    cluster with no Hermite data sits at the mean of its corners with no points.
 //
 // Stages: active-cell marks (edges with samples, from the samples; edges
 // whose end signs differ, word-parallel from the node bits), their
@@ -302,14 +302,17 @@ __device__ __forceinline__ double dot3(const double (&a)[3], const double (&b)[3
 // call spent 400 of 529 us in it for the 255^3 cells of the united sphere and knot).
 // Here FP32 rotations find the eigenvectors, about 100 FP64 operations make
 // them orthonormal and give the matrix in their frame, S = V^T A V, whose
-// off-diagonal entries e are near 1e-7 of the largest eigenvalue:
-//  - the eigenvalues differ from S's diagonal by at most e, so the cut is
+// off-diagonal entries e may be at most 4e-7 of the largest eigenvalue (the
+// largest of 120,000 systems of unit normals at any spread: 2.7e-7):
+//  - the eigenvalues differ from S's diagonal by at most 2 e, so the cut is
 //    decided by the diagonal unless an entry lies within 1e-5 of it;
 //  - turning the kept directions away from the dropped ones by
 //    e / (gap of their eigenvalues) separates them to second order, below
 //    1e-8 with the gaps of 0.004 asked for here;
-//  - what is left is solved on the kept block with its off-diagonal entries.
-// A system that is not so clear (or not finite) goes to the eigensolver.
+//  - what is left is solved on the kept block with its off-diagonal entries, to
+//    second order too, below 2e-9.
+// A system that is not so clear (or not finite, or whose entries are too small
+// for FP32 rotations, as of normals 1e-12 long) goes to the eigensolver.
 __device__ __forceinline__ void qef_solve(const Sym3 &Q, double (&x)[3]) {
     const double inv_n = 1.0 / (double)Q.n;
     const double m[3] = {Q.px * inv_n, Q.py * inv_n, Q.pz * inv_n};
@@ -355,7 +358,7 @@ __device__ __forceinline__ void qef_solve(const Sym3 &Q, double (&x)[3]) {
         keep[c] = l[c] >= cut;
 #pragma unroll
         for (int d = 0; d < 3; ++d)
-            if (d != c) clear = clear && fabsf((float)S[c][d]) <= 1e-5f * top;
+            if (d != c) clear = clear && fabsf((float)S[c][d]) <= 4e-7f * top;
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c)

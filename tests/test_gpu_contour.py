@@ -132,3 +132,33 @@ def test_normals_around_the_cut(ldni, res, spread):
         assert rec["nvert"] == nv
         if not any(abs(r - C.QEF_TRUNC) < 1e-6 for rs in w["ratios"] for r in rs):
             assert np.abs(rec["v"][:nv] - np.asarray(w["vertices"])[:nv]).max() <= 2e-6, key
+
+
+@pytest.mark.parametrize("res", [2, 9, 33])
+@pytest.mark.parametrize("power", [-38, -41, -42, -43, -44])
+def test_vertices_do_not_depend_on_the_normals_length(ldni, res, power):
+    """Normals scaled by 2^power, down to where FP32 can no longer tell the
+    small entries of A^T A from nothing, give the vertices of the unit
+    normals: x does not depend on the scale, so the two differ by the
+    solution's bound (1e-8 of the displacement from the points' mean, which lies
+    within 1 of the origin, in each) and one FP32 rounding each (2^-25 below 1)."""
+    ref = [oracle.as_f32(oracle.sample(*M.icosphere(4, r=0.36), O3, 1.0, res, a, "scan")) for a in range(3)]
+    rng = np.random.default_rng(res)
+    ins = nodes.classify(ref, O3, 1.0, res)
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    inside = _t(_bits(ins).view(np.int32))
+    for spread in (0.02, 0.08, 0.12, 0.3, 2.0):
+        for L in ref:
+            n = np.array([0.6, -0.48, 0.64]) + spread * rng.standard_normal((len(L["depth"]), 3))
+            L["nrm"] = (n / np.linalg.norm(n, axis=1, keepdims=True)).astype(np.float32)
+        unit = ldni.contour_cells([_upload(ldni, grid, a, L) for a, L in enumerate(ref)], inside=inside)
+        want = C.contour(ref, ins, O3, 1.0, res)
+        for L in ref:
+            L["nrm"] = L["nrm"] * np.float32(2.0 ** power)
+        short = ldni.contour_cells([_upload(ldni, grid, a, L) for a, L in enumerate(ref)], inside=inside)
+        assert np.array_equal(unit["cell"], short["cell"]) and np.array_equal(unit["labels"], short["labels"])
+        for u, s in zip(unit, short):
+            if any(abs(r - C.QEF_TRUNC) < 1e-6 for rs in want[int(u["cell"])]["ratios"] for r in rs):
+                continue
+            far = float(np.abs(u["v"]).max())
+            assert np.abs(u["v"] - s["v"]).max() <= 2 * 1e-8 * (1 + far) + 2 * 2.0 ** -25 * max(1.0, far)
