@@ -50,7 +50,8 @@ class Grid:
         return self.width / self.res
 
     def c(self) -> _CGrid:
-        return _CGrid((ctypes.c_float * 3)(*self.origin), self.width, self.res)
+        o = self.origin  # three values, or an IndexError
+        return _CGrid((ctypes.c_float * 3)(o[0], o[1], o[2]), self.width, self.res)
 
 
 class LDNI:
@@ -74,9 +75,9 @@ class LDNI:
         return int(self.depth.numel())
 
     def c(self) -> _CLayers:
-        ptr = lambda t: t.data_ptr() if t is not None and t.numel() else None
+        ptr = lambda t: t.data_ptr() if t.numel() else None
         return _CLayers(self.offsets.data_ptr(), ptr(self.depth), ptr(self.nx), ptr(self.ny), ptr(self.nz),
-                        ptr(self.tri), self.capacity, ptr(self.nrm8))
+                        ptr(self.tri), self.capacity, ptr(self.nrm8) if self.packed else None)
 
     def counts(self):
         return self.offsets[1:] - self.offsets[:-1]

@@ -102,3 +102,23 @@ def test_build_stamp_is_the_same_in_another_checkout(tmp_path):
     assert copy.ROOT != build.ROOT
     assert copy._stamp() == build._stamp()
     assert copy._stamp(["learned.cu"]) == build._stamp(["learned.cu"]) != build._stamp()
+
+
+def test_python_descriptors_take_whole_grids_and_images_only():
+    """A grid needs three origin values and an image every array of its
+    format; neither is filled up with zeros or null pointers."""
+    torch = pytest.importorskip("torch")
+    g = pkg.Grid((0.5, -1.0, 2.0), 3.0, 8).c()
+    assert list(g.origin) == [0.5, -1.0, 2.0] and g.width == 3.0 and g.res == 8
+    with pytest.raises(IndexError):
+        pkg.Grid((0.5, -1.0), 3.0, 8).c()
+    grid = pkg.Grid.cube((0, 0, 0), 1.0, 2)
+    off, f, i = torch.zeros(5, dtype=torch.int32), torch.zeros(4), torch.zeros(4, dtype=torch.int32)
+    c = pkg.LDNI(grid, 0, off, f, f, f, f, i, 4).c()
+    assert (c.offsets, c.depth, c.nz, c.tri_id, c.capacity, c.nrm8) == (off.data_ptr(), f.data_ptr(), f.data_ptr(),
+                                                                        i.data_ptr(), 4, None)
+    c = pkg.LDNI(grid, 0, off, f, f[:0], f[:0], f[:0], i, 4, nrm8=i).c()
+    assert (c.nx, c.ny, c.nz, c.nrm8) == (None, None, None, i.data_ptr())
+    for arrays in ((None, f, f, f, i), (f, None, f, f, i), (f, f, f, f, None)):
+        with pytest.raises(AttributeError):
+            pkg.LDNI(grid, 0, off, *arrays, 4).c()
