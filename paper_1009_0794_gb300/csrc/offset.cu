@@ -52,6 +52,10 @@ constexpr int kMaxComp = 257;     // components a ray may keep when its interval
 constexpr int kBuf = kMaxComp + 32;  // intervals of one ray held in shared memory: room for a warp's after a merge
 constexpr int kMaxHSamples = 384; // H's samples on one ray
 constexpr int kKept = 8;          // samples whose sources the count pass leaves to the write pass
+// Rays per image up to which the three images' sources are kept side by side;
+// larger images are counted and written one after another and share the space
+// (32 instead of 96 bytes a pixel), where a few launches more do not show.
+constexpr long long kKeptTogether = 1ll << 20;
 constexpr int kTile = kOffWarps;  // pixels per side of a sphere-list tile
 constexpr int kThreads = 256;
 
@@ -71,6 +75,7 @@ struct OffArgs {
     float inv_h;
     float slack[3];  // pixels by which a shadow is widened, per world axis (off_bin)
     int inner;
+    int img0;        // first image of the launch (counts and writes)
     // sphere centres and tile lists
     float4 *C;
     int *tcnt[3];   // per tile: spheres binned (count pass), then the fill cursor
@@ -345,7 +350,7 @@ __device__ __forceinline__ void put_result(const OffArgs &A, int b, long long hb
     pick(A.ot, b)[slot] = id;
 }
 
-// One pixel row of a tile of image blockIdx.y, a warp per ray.  The block
+// One pixel row of a tile of image b, a warp per ray.  The block
 // walks the tile's list, kStage spheres at a time (the next ones' loads in
 // flight), and stages those that reach its row (about a third), with their
 // distance from the row, which all its rays share, in the list's order: the
@@ -556,7 +561,7 @@ __device__ __forceinline__ void ray_row(const OffArgs &A, int bx, int b, ldni_in
 }
 
 __global__ void __launch_bounds__(kOffWarps * 32) off_count(OffArgs A, ldni_info_t *info) {
-    ray_row<false>(A, (int)blockIdx.x, (int)blockIdx.y, info);
+    ray_row<false>(A, (int)blockIdx.x, A.img0 + (int)blockIdx.y, info);
 }
 
 // The rows that hold rays of more than kKept samples, from the list the count
@@ -571,9 +576,9 @@ __global__ void __launch_bounds__(kOffWarps * 32) off_deep(OffArgs A, ldni_info_
 }
 
 // The samples of the rays that have at most kKept, from the sources that the
-// count pass left: a thread per ray of image blockIdx.y.
+// count pass left: a thread per ray of image img0 + blockIdx.y.
 __global__ void __launch_bounds__(kThreads) off_write(OffArgs A, ldni_info_t *info) {
-    const int b = blockIdx.y;
+    const int b = A.img0 + blockIdx.y;
     const long long p = blockIdx.x * (long long)kThreads + threadIdx.x;
     if (p >= (long long)A.res * A.res) return;
     const int n = pick(A.cnt, b)[p];
@@ -619,7 +624,7 @@ bool carve_offset(Carver &c, long long S, int res, double r_pixels, OffWs &w) {
         w.toff[a] = c.take<int>((size_t)ntiles + 1);
         w.tlist[a] = c.take<int>((size_t)(pairs > 0 ? pairs : 1));
         w.cnt[a] = c.take<int>((size_t)N);
-        w.kept[a] = c.take<uint4>(2 * (size_t)N);
+        w.kept[a] = a == 0 || N <= kKeptTogether ? c.take<uint4>(2 * (size_t)N) : w.kept[0];
     }
     w.deep = c.take<int>(1 + 3 * (size_t)ntiles * kTile);
     const size_t parts = std::max(csr_scan_partials(N), csr_scan_partials(ntiles));
@@ -724,18 +729,19 @@ extern "C" int ldni_offset(const ldni_layers_t *H, const int64_t *n, const ldni_
     // the counts become the fill cursors
     if (int rc_ = cuda_check(cudaMemsetAsync(w.tcnt[0], 0, w.clear_bytes, s))) return rc_;
     if (S > 0) LDNI_LAUNCH(K_OFFSET, s, off_bin<true><<<dim3(sblocks, 3), kThreads, 0, s>>>(A));
-    const dim3 tblocks((unsigned)(ntiles * kTile), 3);
-    if (int rc_ = cuda_check(cudaMemsetAsync(w.deep, 0, sizeof(int), s))) return rc_;
-    LDNI_LAUNCH(K_OFFSET, s, off_count<<<tblocks, kOffWarps * 32, 0, s>>>(A, info));
-    rc = cuda_status();
-    if (rc != LDNI_OK) return rc;
-    {
+    const int together = N <= kKeptTogether ? 3 : 1;
+    for (A.img0 = 0; A.img0 < 3; A.img0 += together) {
+        if (int rc_ = cuda_check(cudaMemsetAsync(w.deep, 0, sizeof(int), s))) return rc_;
+        LDNI_LAUNCH(K_OFFSET, s,
+                    off_count<<<dim3((unsigned)(ntiles * kTile), together), kOffWarps * 32, 0, s>>>(A, info));
+        rc = cuda_status();
+        if (rc != LDNI_OK) return rc;
         const int *cnts[3] = {w.cnt[0], w.cnt[1], w.cnt[2]};
         int *offs[3] = {out[0].offsets, out[1].offsets, out[2].offsets};
-        rc = csr_scan(cnts, offs, 3, N, w.partials, info, 0, s);
+        rc = csr_scan(cnts + A.img0, offs + A.img0, together, N, w.partials, info, A.img0, s);
         if (rc != LDNI_OK) return rc;
+        LDNI_LAUNCH(K_OFFSET, s, off_write<<<dim3(rblocks, together), kThreads, 0, s>>>(A, info));
+        LDNI_LAUNCH(K_OFFSET, s, off_deep<<<4 * num_sms(), kOffWarps * 32, 0, s>>>(A, info));
     }
-    LDNI_LAUNCH(K_OFFSET, s, off_write<<<dim3(rblocks, 3), kThreads, 0, s>>>(A, info));
-    LDNI_LAUNCH(K_OFFSET, s, off_deep<<<4 * num_sms(), kOffWarps * 32, 0, s>>>(A, info));
     return cuda_status();
 }

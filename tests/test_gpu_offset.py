@@ -203,3 +203,16 @@ def test_most_samples_of_the_solid_on_a_ray(ldni, samples, fits):
             with pytest.raises(ldni.LDNIError) as e:
                 ldni.offset(H, 1e-4, inner=inner)
             assert e.value.code == -4
+
+
+@pytest.mark.parametrize("inner", [False, True])
+def test_large_images_one_after_another(ldni, inner):
+    """Images above 2^20 rays share the space for kept sources: rays of few
+    and of many samples in all three, against the oracle, in a workspace of
+    under 50 bytes a pixel."""
+    res = 1030
+    v, t = M.slab_stack(30, axis=0, seed=2)
+    grid, ref, H = _solid(ldni, ((v * np.float32([1.0, 0.02, 0.02])).astype(np.float32), t), res)
+    got = _check(ldni, grid, ref, H, 1.3 / res, inner, eps=1e-4)
+    assert all(int(L.counts().max()) > 8 and L.n > 0 for L in got)
+    assert ldni.offset_workspace_size([100] * 3, 8192, 1.3 / 8192, 1.0) < 50 * 8192 ** 2
