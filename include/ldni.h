@@ -58,7 +58,8 @@ extern "C" {
 #define LDNI_ST_TIMEOUT 8u        /* a bounded device wait expired */
 #define LDNI_ST_RANGE 16u         /* a vertex could not be snapped (outside +-2^24 units) */
 #define LDNI_ST_INDEX 32u         /* a triangle referenced a vertex index outside [0, nv) */
-#define LDNI_ST_EVENTS 64u        /* offsetting: a ray met more samples than one warp orders; left empty */
+#define LDNI_ST_EVENTS 64u        /* offsetting, union chains: a ray needs more samples or separate intervals than
+                                     a ray may hold; left empty */
 #define LDNI_ST_BOUNDS 128u       /* checked builds only (LDNI_CHECKS): a CSR or slab index outside its array
                                      was met and that access skipped; release builds never set it */
 
@@ -444,7 +445,8 @@ int ldni_boolean_static(const ldni_layers_t *A, const ldni_grid_t *grid_a, const
 
 /* ---- chains of unions (Sections 4.1.1 and 4.2) -------------------------- */
 
-/* Workspace bytes for ldni_union_chain of nimg (1 .. 3) images at res. */
+/* Workspace bytes for ldni_union_chain of nimg (1 .. 3) images at res: about 16
+ * a ray of large images, at most 50 MB more for small ones. */
 int ldni_union_chain_workspace_size(int32_t res, int32_t nimg, size_t *bytes_host);
 
 /*
@@ -585,17 +587,20 @@ int ldni_offset_workspace_size(const int64_t *n, int32_t res, float r, float wid
  * H, out: host arrays of 3 layers (image x, y, z) with device buffers on one
  * grid; n: host int64[3], the samples of H's images.  info: device, n[b] =
  * samples image b of the result needs; beyond out[b].capacity samples are
- * dropped (LDNI_ST_CAPACITY) while the offsets are still complete.  A ray
- * that meets more than 512 samples (H's plus two per sphere that can change
- * it) is left empty with LDNI_ST_EVENTS.  Odd input rays set LDNI_ST_ODD.
+ * dropped (LDNI_ST_CAPACITY) while the offsets are still complete.  A ray is
+ * left empty with LDNI_ST_EVENTS when it holds more than 384 samples of H, or
+ * when its intervals (H's, or for inner its gaps, and one per sphere that meets
+ * it, taken 289 at a time) still form more than 257 separate ones while they
+ * are merged; a result of up to 256 intervals always fits, one of more than
+ * 289 never does.  Odd input rays set LDNI_ST_ODD.
  */
 int ldni_offset(const ldni_layers_t *H, const int64_t *n, const ldni_grid_t *grid, float r, int32_t inner, float eps,
                 ldni_layers_t *out, ldni_info_t *info, void *ws, size_t ws_bytes, void *stream);
 
 /* ---- grid-node classification (Section 5.1, Step 1) -------------------- */
 
-/* Workspace bytes for ldni_classify_nodes at resolution res (<= 4096):
- * three bit volumes of res^2 * ceil(res / 32) words. */
+/* Workspace bytes for ldni_classify_nodes at resolution res (<= 4096): per
+ * image res * ceil(res / 32)^2 groups of 32 words and an 8-byte summary each. */
 int ldni_classify_nodes_workspace_size(int32_t res, size_t *bytes_host);
 
 /*

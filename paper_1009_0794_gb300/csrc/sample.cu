@@ -31,8 +31,9 @@
 // against the next offset), and the crossings are counted once more: a fill
 // that did not see as many as the count reports LDNI_ST_CAPACITY.
 //
-// Triangles whose pixel box is large are handed to a block-per-triangle
-// kernel with 64-bit edge functions.
+// Pairs of a triangle and an image whose pixel box is large are queued and swept
+// by several threads, huge ones by whole blocks, with 64-bit edge functions where
+// 32 bits do not hold them.
 #include <algorithm>
 
 #include "sample_common.cuh"
@@ -416,7 +417,7 @@ __global__ void __launch_bounds__(kThreads) bin_pass(const float *__restrict__ v
 }
 
 // One staged triangle of a tile: its setup (small: Setup32, big: Setup64),
-// pixel box, id and normal.
+// pixel box and id.
 struct TileTri {
     Setup64 L;
     Setup32 S;

@@ -607,7 +607,7 @@ def offset(Ls: Sequence[LDNI], r: float, inner: bool = False, eps: float = 0.0, 
         if meta["status"] & _lib.ST_ODD:
             raise _lib.LDNIError(-3, "ldni_offset")
         if meta["status"] & _lib.ST_EVENTS:
-            raise _lib.LDNIError(-4, "ldni_offset (a ray meets more sphere samples than one warp orders)")
+            raise _lib.LDNIError(-4, "ldni_offset (a ray needs more samples or separate intervals than it may hold)")
         for a in range(3):
             outs[a].n = meta["n"][a]
         return outs
