@@ -591,8 +591,8 @@ int ldni_offset_workspace_size(const int64_t *n, int32_t res, float r, float wid
  * left empty with LDNI_ST_EVENTS when it holds more than 384 samples of H, or
  * when its intervals (H's, or for inner its gaps, and one per sphere that meets
  * it, taken 289 at a time) still form more than 257 separate ones while they
- * are merged; a result of up to 256 intervals always fits, one of more than
- * 289 never does.  Odd input rays set LDNI_ST_ODD.
+ * are merged, so a result of more than 289 intervals never fits.  Odd input
+ * rays set LDNI_ST_ODD.
  */
 int ldni_offset(const ldni_layers_t *H, const int64_t *n, const ldni_grid_t *grid, float r, int32_t inner, float eps,
                 ldni_layers_t *out, ldni_info_t *info, void *ws, size_t ws_bytes, void *stream);
