@@ -351,7 +351,7 @@ __device__ __forceinline__ void qef_solve(const Sym3 &Q, double (&x)[3]) {
     // everything below that decides or corrects needs FP32 only; S and g keep their FP64 values
     const float l[3] = {(float)S[0][0], (float)S[1][1], (float)S[2][2]};
     const float top = fmaxf(l[0], fmaxf(l[1], l[2])), cut = 0.01f * top;
-    bool clear = top > 0.0f && top < 1e30f, keep[3];
+    bool clear = top > 1e-30f && top < 1e30f, keep[3];  // (the kept ones' FP32 reciprocals are finite)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         clear = clear && fabsf(l[c] - cut) > 1e-5f * top;

@@ -162,3 +162,25 @@ def test_vertices_do_not_depend_on_the_normals_length(ldni, res, power):
                 continue
             far = float(np.abs(u["v"]).max())
             assert np.abs(u["v"] - s["v"]).max() <= 2 * 1e-8 * (1 + far) + 2 * 2.0 ** -25 * max(1.0, far)
+
+
+@pytest.mark.parametrize("power", [-60, -64, -66, -70, -74, -80])
+def test_vertices_of_tiny_normals_along_an_axis(ldni, power):
+    """A^T A is diagonal, so FP32 turns nothing however small its entries are;
+    their reciprocals leave FP32 below 2^-126 (normals of 2^-64 and shorter).
+    The bound of the lengths' test above."""
+    res = 9
+    ref = [oracle.as_f32(oracle.sample(*M.icosphere(4, r=0.36), O3, 1.0, res, a, "scan")) for a in range(3)]
+    ins = nodes.classify(ref, O3, 1.0, res)
+    grid = ldni.Grid.cube(O3, 1.0, res)
+    inside = _t(_bits(ins).view(np.int32))
+    got = []
+    for scale in (1.0, 2.0 ** power):
+        for a, L in enumerate(ref):
+            L["nrm"] = np.zeros((len(L["depth"]), 3), np.float32)
+            L["nrm"][:, a] = scale
+        got.append(ldni.contour_cells([_upload(ldni, grid, a, L) for a, L in enumerate(ref)], inside=inside))
+    unit, tiny = got
+    assert np.array_equal(unit["cell"], tiny["cell"]) and np.isfinite(unit["v"]).all()
+    far = float(np.abs(unit["v"]).max())
+    assert np.abs(unit["v"] - tiny["v"]).max() <= 2 * 1e-8 * (1 + far) + 2 * 2.0 ** -25 * max(1.0, far)
